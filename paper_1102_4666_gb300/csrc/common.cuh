@@ -6,6 +6,8 @@
 
 #include <cmath>
 
+#include "fx64.cuh"
+
 #define BSDE_DMAX 16
 #define BSDE_NNZ_MAX 8  // active variates per basis function
 #define BSDE_RANKS_MAX 64  // ranks of a point-sharded solve (BSDE_MAX_RANKS of the C ABI)
@@ -63,6 +65,7 @@ struct Math;
 
 template <>
 struct Math<float> {
+  using Bm = float;
   // Box-Muller pair from two 32-bit words, u = (w + 1/2) 2^-32 in (0,1],
   // returning scale * (z0, z1).  k = bm_factor(scale) = -2 ln(2) scale^2
   // folds the scale and the change of logarithm base into one product:
@@ -109,22 +112,32 @@ struct Math<float> {
 
 template <>
 struct Math<double> {
-  // the FP64 path applies the scale after the square root
-  __device__ __forceinline__ static double bm_factor(double scale) { return scale; }
-  __device__ __forceinline__ static void box_muller(uint32_t w0, uint32_t w1, double& z0,
-                                                    double& z1, double scale) {
-    const double u0 = ((double)w0 + 0.5) * 2.3283064365386962890625e-10;
-    const double u1 = ((double)w1 + 0.5) * 2.3283064365386962890625e-10;
-    const double rad = ::sqrt(-2.0 * ::log(u0)) * scale;
-    double s, c;
-    sincospi(2.0 * u1, &s, &c);
-    z0 = rad * c;
-    z1 = rad * s;
+  // Box-Muller in 64-bit fixed point (fx64.cuh), the scale folded into the
+  // radius; a scale outside the normal range (zero, NaN) multiplies after it
+  struct Bm {
+    fx64::Scale sc;
+    double mul;
+    bool plain;
+  };
+  __device__ __forceinline__ static Bm bm_factor(double scale) {
+    Bm k;
+    k.plain = fx64::to_scale(scale, k.sc);
+    k.mul = scale;
+    if (!k.plain) fx64::to_scale(1.0, k.sc);
+    return k;
   }
-  __device__ __forceinline__ static double exp(double x) { return ::exp(x); }
+  __device__ __forceinline__ static void box_muller(uint32_t w0, uint32_t w1, double& z0,
+                                                    double& z1, const Bm& k) {
+    fx64::box_muller(w0, w1, k.sc, z0, z1);
+    if (!k.plain) {
+      z0 *= k.mul;
+      z1 *= k.mul;
+    }
+  }
+  __device__ __forceinline__ static double exp(double x) { return fx64::exp(x); }
   __device__ __forceinline__ static double sqrt(double x) { return ::sqrt(x); }
   __device__ __forceinline__ static double sin(double x) { return ::sin(x); }
-  __device__ __forceinline__ static double exp_acc(double x) { return ::exp(x); }
+  __device__ __forceinline__ static double exp_acc(double x) { return fx64::exp(x); }
   __device__ __forceinline__ static double fabs(double x) { return ::fabs(x); }
   __device__ __forceinline__ static double fmax(double a, double b) { return ::fmax(a, b); }
 };

@@ -67,6 +67,7 @@ struct Args {
   R vb;
   R rho;  // constant correlation (dense evaluation)
   alignas(16) R kc[D];  // -2 log2(e) kappa_j: e^{2 (x - kappa)} = 2^{x 2 log2(e) + kc}
+  R sj[D], cj[D];  // sin and cos of the asset number j + 1 (sin/tanh volatility, FP64 rows)
   uint32_t k;
   uint32_t key0, key1;  // Philox key
   uint32_t rk0[10], rk1[10];  // its ten round keys (kernel-parameter constants)
@@ -188,38 +189,31 @@ __device__ __forceinline__ uint4 philox_tab(const Args<R, D>& a, const PhiloxFix
 
 // r = 1 / (e^{2 y} + 1), so that tanh(y) = 1 - 2 r, with y = x - kappa_j
 // (ABS: y = |x - kappa_j|, since |tanh(x - kappa)| = tanh(|x - kappa|))
-template <bool ABS, typename R, int D>
-__device__ __forceinline__ R tanh_r(const Args<R, D>& a, int j, R xj) {
-  if constexpr (sizeof(R) == 4) {
-    float e, r;
-    const float t = fmaf(xj, 2.8853900817779268f, a.kc[j]);  // 2 log2(e) (x - kappa)
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(ABS ? fabsf(t) : t));
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(e + 1.0f));
-    return r;
-  } else {
-    const double y = xj - a.kappa[j];
-    return 1.0 / (::exp(2.0 * (ABS ? ::fabs(y) : y)) + 1.0);
-  }
+template <bool ABS, int D>
+__device__ __forceinline__ float tanh_r(const Args<float, D>& a, int j, float xj) {
+  float e, r;
+  const float t = fmaf(xj, 2.8853900817779268f, a.kc[j]);  // 2 log2(e) (x - kappa)
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(ABS ? fabsf(t) : t));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(e + 1.0f));
+  return r;
 }
 
 // local volatility of asset j at the step whose table row is tabs.  The
 // tanh families keep (A, B) = (a + phi, -2 phi) per step and asset, with phi
 // the time factor, and sigma = A + B r: a + phi tanh(y) = a + phi (1 - 2 r).
+// FP64 paths get 1 + r from fx64.cuh (the fixed-point r placed in a mantissa,
+// without a conversion) and keep A - B = a + 3 phi instead of A.
 template <int VK, typename R, int D>
 __device__ __forceinline__ R sigma_j(const Args<R, D>& a, const R* tabs, int j, R xj) {
   if constexpr (VK == VK_CONST) {
     return a.va[j];
   } else if constexpr (VK == VK_TANH || VK == VK_TANH_ABS) {
-    const R r = tanh_r<VK == VK_TANH_ABS>(a, j, xj);
-    R A, B;
     if constexpr (sizeof(R) == 4) {
-      A = tabs[4 * (j >> 1) + (j & 1)];
-      B = tabs[4 * (j >> 1) + 2 + (j & 1)];
+      const R r = tanh_r<VK == VK_TANH_ABS>(a, j, xj);
+      return tabs[4 * (j >> 1) + (j & 1)] + tabs[4 * (j >> 1) + 2 + (j & 1)] * r;
     } else {
-      A = tabs[2 * j];
-      B = tabs[2 * j + 1];
+      return tabs[2 * j] + tabs[2 * j + 1] * fx64::logistic_p1(xj - a.kappa[j], VK == VK_TANH_ABS);
     }
-    return A + B * r;
   } else {
     const R dev = Math<R>::exp(xj) * tabs[2] - a.s_dupire;
     return tabs[0] - tabs[1] * Math<R>::exp(R(-0.001) * dev * dev);
@@ -229,7 +223,7 @@ __device__ __forceinline__ R sigma_j(const Args<R, D>& a, const R* tabs, int j, 
 template <typename R, int D>
 __device__ __forceinline__ R basket_value(const Args<R, D>& a, const R* x, bool positive) {
   R s = 0;
-#pragma unroll
+#pragma unroll(sizeof(R) == 8 ? 1 : D)
   for (int j = 0; j < D; ++j) s += a.w[j] * Math<R>::exp(x[j]);
   const R v = (a.payoff == 0) ? (a.K - s) : (s - a.K);
   return positive ? Math<R>::fmax(v, R(0)) : v;
@@ -860,6 +854,71 @@ __device__ __forceinline__ void load_state(const float4* p, int stride, R (&X)[D
   }
 }
 
+// The Euler path of one FP64 thread, from X (x0 on entry) to X_T, with the
+// states before and after step s* in Xs and Xn.  Bound by the FP64 pipe (two
+// lanes per SM and clock: 64 issue slots per instruction of a warp): with
+// the normals and the logistic function in fixed point (fx64.cuh) an asset's
+// step takes seven FP64 instructions (constant correlation, tanh
+// volatility) and about 250 integer ones.  The loop runs over the normals
+// themselves, four (one Philox block) a turn, with (step, asset) counted
+// along, and the assets' states in local memory: unrolled over G steps of D
+// assets the fixed-point code would be several times the instruction cache,
+// and its states, normals and copies more registers than there are; a
+// state's load and store are nothing beside the 64-slot instructions.
+// Measured, d = 10 degree 3 (n = 1000, M = 100, N = 60): 11.08 ms a launch
+// with the library's log, sqrt, sincospi and exp, 2.24 ms with this (FP64 pipe
+// 74 % busy, a third of it the evaluation of u^k; issue 39 %).
+template <int VK, bool CC, int D>
+__device__ __forceinline__ void euler_path_f64(const Args<double, D>& a, const double* tab,
+                                               const uint4* s_ph, const PhiloxFixed& pz,
+                                               const Math<double>::Bm& bmk, double nhh, double h,
+                                               int sstar, double (&X)[D], double (&Xs)[D],
+                                               double (&Xn)[D]) {
+  const int total = a.N * D;
+  int s = 0, j = 0;
+  const double* row = tab;
+  double pre = 0.0;  // running sum of the constant-correlation factor
+  double zs[D];      // the step's normals so far (general correlation)
+#pragma unroll 1
+  for (int q = 0; q < total; q += 4) {
+    const uint4 o = philox_tab(a, pz, s_ph[q >> 2]);
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+      double z[2];
+      Math<double>::box_muller(half ? o.z : o.x, half ? o.w : o.y, z[0], z[1], bmk);
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        if (s < a.N) {
+          const double x = X[j];
+          double y;
+          if constexpr (CC) {
+            y = a.Ld[j] * z[r] + pre;
+            pre += a.Lc[j] * z[r];
+          } else {
+            zs[j] = z[r];
+            y = 0.0;
+#pragma unroll 1
+            for (int c = 0; c <= j; ++c) y += a.L[j][c] * zs[c];
+          }
+          const double sig = sigma_j<VK>(a, row, j, x);
+          const double xn = sig * (nhh * sig + y) + (h * a.rd[j] + x);
+          X[j] = xn;
+          if (s == sstar) {
+            Xs[j] = x;
+            Xn[j] = xn;
+          }
+          if (++j == D) {
+            j = 0;
+            ++s;
+            row += a.tab_stride;
+            pre = 0.0;
+          }
+        }
+      }
+    }
+  }
+}
+
 // One CTA's work: a point and a chunk of its paths (the kernels below).
 template <int VK, int EV, bool CC, typename R, int D>
 __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
@@ -921,21 +980,40 @@ __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
   for (int j = 0; j < D; ++j) x0[j] = (R)a.px[(size_t)j * a.n + i];
   const R h = (a.T - ti) / (R)a.N;
   const R sqh = Math<R>::sqrt(h);
-  const R bmk = Math<R>::bm_factor(sqh);  // Box-Muller radius factor of the step normals
-  const R bm1 = Math<R>::bm_factor(R(1));
+  // Box-Muller radius factors of the step normals and of the bridge's
+  const typename Math<R>::Bm bmk = Math<R>::bm_factor(sqh);
+  const typename Math<R>::Bm bm1 = Math<R>::bm_factor(R(1));
 
   // per-step coefficients of the local volatility (in the precision of the
   // path: accurate sinf/expf for FP32, sin/exp for FP64)
+  if constexpr (sizeof(R) == 8 && (VK == VK_TANH || VK == VK_TANH_ABS)) {
+    // rows (A_j - B_j, B_j) per asset.  One sine and cosine (or exponential)
+    // per step, the assets by the addition theorem: an FP64 sine per entry
+    // would cost more than the Euler steps of a CTA's paths.
+    for (int s = tid; s < a.N; s += tpb) {
+      const R ts = ti + (R)s * h;
+      R st = 0, ct = 0;
+      if (a.vol_sin)
+        ::sincos(ts, &st, &ct);
+      else
+        ct = a.vb * Math<R>::exp_acc(-ts);
+      R* row = tab + s * a.tab_stride;
+      for (int j = 0; j < D; ++j) {
+        const R phi = a.vol_sin ? a.vb * (a.sj[j] * ct + a.cj[j] * st) : ct;
+        row[2 * j] = a.va[j] + R(3) * phi;
+        row[2 * j + 1] = R(-2) * phi;
+      }
+    }
+  } else
   for (int idx = tid; idx < a.N * a.tab_stride; idx += tpb) {
     const int s = idx / a.tab_stride, c = idx - s * a.tab_stride;
     const R ts = ti + (R)s * h;
     R v = 0;
     if constexpr (VK == VK_TANH || VK == VK_TANH_ABS) {
       // FP32 rows: (A_j, A_j+1, B_j, B_j+1) per pair of assets, so that one
-      // 128-bit load gives the pair's A and B as two float2; FP64 rows:
-      // (A_j, B_j) per asset
-      const int j = sizeof(R) == 4 ? 2 * (c >> 2) + (c & 1) : c >> 1;
-      const bool isB = sizeof(R) == 4 ? ((c >> 1) & 1) != 0 : (c & 1) != 0;
+      // 128-bit load gives the pair's A and B as two float2
+      const int j = 2 * (c >> 2) + (c & 1);
+      const bool isB = ((c >> 1) & 1) != 0;
       const R phi = a.vol_sin ? a.vb * Math<R>::sin((R)(j + 1) + ts) : a.vb * Math<R>::exp_acc(-ts);
       v = isB ? R(-2) * phi : a.va[j < D ? j : 0] + phi;
     } else if constexpr (VK == VK_DUPIRE) {
@@ -1007,6 +1085,9 @@ __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
     }
     const R nhh = R(-0.5) * h;
     const PhiloxFixed pz = philox_fix(a, (uint32_t)m, (uint32_t)i, tagZ);
+    if constexpr (sizeof(R) == 8) {
+      euler_path_f64<VK, CC>(a, tab, s_ph, pz, bmk, nhh, h, sstar, X, Xs, Xn);
+    } else
     for (int s0 = 0; s0 < a.N; s0 += G) {
       R z[G * D];  // normals of G steps, scaled by sqrt(h)
       const uint32_t blk0 = (uint32_t)(s0 / G) * (uint32_t)NB;
@@ -1093,7 +1174,7 @@ __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
 
     // X at tau: Brownian bridge inside step s*, coefficients frozen at t_{s*}
     R zb[NBB * 4];
-#pragma unroll
+#pragma unroll(sizeof(R) == 8 ? 1 : NBB)
     for (int b = 0; b < NBB; ++b) {
       const uint4 o = philox_rk(a, (uint32_t)b, (uint32_t)m, (uint32_t)i, tagB);
       Math<R>::box_muller(o.x, o.y, zb[4 * b + 0], zb[4 * b + 1], bm1);
@@ -1102,11 +1183,16 @@ __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
     const R* tab_s = tab + sstar * a.tab_stride;
     const R bb = Math<R>::sqrt(theta * (R(1) - theta) * h);
     R Xtau[D], sig_s[D], drift_s[D];
-#pragma unroll
+#pragma unroll(sizeof(R) == 8 ? 1 : D)
     for (int j = 0; j < D; ++j) {
       R y = 0;
+      if constexpr (sizeof(R) == 8) {
+#pragma unroll 1
+        for (int q = 0; q <= j; ++q) y += a.L[j][q] * zb[q];
+      } else {
 #pragma unroll
-      for (int q = 0; q <= j; ++q) y += a.L[j][q] * zb[q];
+        for (int q = 0; q <= j; ++q) y += a.L[j][q] * zb[q];
+      }
       sig_s[j] = sigma_j<VK>(a, tab_s, j, Xs[j]);
       drift_s[j] = a.rd[j] - R(0.5) * sig_s[j] * sig_s[j];
       Xtau[j] = Xs[j] + theta * (Xn[j] - Xs[j]) + sig_s[j] * bb * y;
@@ -1340,6 +1426,8 @@ cudaError_t launch(const ModelHost& m, const GridHost& g, const ProblemDev& P, i
     a.w[j] = (R)m.w[j];
     a.va[j] = (R)m.a[j];
     a.kappa[j] = (R)m.kappa[j];
+    a.sj[j] = (R)std::sin((double)(j + 1));
+    a.cj[j] = (R)std::cos((double)(j + 1));
     for (int q = 0; q < D; ++q) {
       a.L[j][q] = (R)m.L[j * D + q];
       a.Cp[j + 1][q + 1] = (R)m.C[j * D + q];
