@@ -220,6 +220,25 @@ __device__ __forceinline__ R sigma_j(const Args<R, D>& a, const R* tabs, int j, 
   }
 }
 
+// L z for a whole vector (constant correlation: running sums)
+template <bool CC, typename R, int D, int NZ>
+__device__ __forceinline__ void correlate(const Args<R, D>& a, const R (&z)[NZ], R (&y)[D]) {
+  R pre = 0;
+#pragma unroll(sizeof(R) == 8 ? 1 : D)
+  for (int j = 0; j < D; ++j) {
+    if constexpr (CC) {
+      y[j] = a.Ld[j] * z[j] + pre;
+      pre += a.Lc[j] * z[j];
+    } else {
+      R s = 0;
+#pragma unroll(sizeof(R) == 8 ? 1 : D)
+      for (int q = 0; q < D; ++q)
+        if (q <= j) s += a.L[j][q] * z[q];
+      y[j] = s;
+    }
+  }
+}
+
 template <typename R, int D>
 __device__ __forceinline__ R basket_value(const Args<R, D>& a, const R* x, bool positive) {
   R s = 0;
@@ -530,6 +549,131 @@ __device__ __forceinline__ void eval_dense4(const Args<R, D>& a, const R* __rest
   (void)us;
   u = uv;
   gen = ub + R(0.5) * ((R(1) - a.rho) * diag + a.rho * uss);
+}
+
+// The same for a full correlation matrix C, total degree DEG = 3 or 4.  With
+// W_vw = st_v st_w C_vw the diffusion term takes, from a monomial z_i z_j z_k..
+// (i <= j <= k.., repeated variates included), the sum over its pairs of
+// factors of W times the remaining ones: 1/2 sum_vw W_vw d2_vw (z_i z_j z_k) =
+// W_ij z_k + W_ik z_j + W_jk z_i.  The innermost level then accumulates, besides
+// z, zT and bt, one row of W per outer index (DEG - 1 of them) in the place of
+// st: five multiply-adds per cubic coefficient instead of four, six per
+// quartic one.  Against the per-thread Chebyshev tables, which carried such
+// models before: d = 4 degree 3 (n = 1501, M = 1003, N = 25) @@.
+template <int DEG, typename R, int D, int CS = 1>
+__device__ __forceinline__ void eval_dense_full(const Args<R, D>& a, const R* __restrict__ beta,
+                                                const R (&z)[D + 1], const R (&zT)[D + 1],
+                                                const R (&bt)[D + 1], const R (&st)[D + 1], R& u,
+                                                R& gen, R& uT) {
+  static_assert(DEG == 3 || DEG == 4, "Horner loops of degree 3 or 4");
+  static_assert(CS == 1 || (CS == 2 && sizeof(R) == 4), "paired coefficients are FP32 only");
+  constexpr int DP = D + 1;
+  constexpr int NQ = DP * (DP + 1) / 2;
+  constexpr int NC = DP * (DP + 1) * (DP + 2) / 6;
+  const R* bg = beta + CS;
+  const R* bq = bg + CS * DP;
+  const R* bc3 = bq + CS * NQ;
+  const R* bc4 = bc3 + CS * NC;
+  R W[DP][DP];  // compile-time indices: the upper triangle lives in registers
+#pragma unroll
+  for (int v = 0; v < DP; ++v) {
+#pragma unroll
+    for (int w = 0; w < DP; ++w)
+      W[v][w] = v == w ? st[v] * st[v] : (v > 0 && w > 0) ? st[v] * st[w] * a.Cp[v][w] : R(0);
+  }
+  R uv = beta[0], ub = R(0), H = R(0), sT = beta[0];
+  int iq = 0, ic = 0, i4 = 0;
+#pragma unroll
+  for (int i = 0; i < DP; ++i) {
+    R bv = bg[CS * i], bb = R(0), bT = bv;
+#pragma unroll
+    for (int j = 0; j < DP; ++j) {
+      if (j < i) continue;
+      const R q = bq[CS * iq++];
+      R av = q, ab = R(0), aT = q, w1 = R(0), w2 = R(0);
+      float2 VT = make_float2(q, q), BW = make_float2(0.f, 0.f);
+      if (DEG == 4 && i > 0) H += W[i][j] * q;
+#pragma unroll
+      for (int k = 0; k < DP; ++k) {
+        if (k < j) continue;
+        const R t = bc3[CS * ic];
+        if constexpr (DEG == 3) {
+          if constexpr (CS == 2) {
+            const float2 tt = reinterpret_cast<const float2*>(bc3)[ic];
+            VT = __ffma2_rn(tt, make_float2(z[k], zT[k]), VT);
+            BW = __ffma2_rn(tt, make_float2(bt[k], W[i][k]), BW);
+          } else {
+            av += t * z[k];
+            aT += t * zT[k];
+            ab += t * bt[k];
+            if (i > 0) w1 += t * W[i][k];
+          }
+          if (j > 0 && k > 0) w2 += t * W[j][k];
+        } else {
+          R ev = t, eb = R(0), eT = t, e1 = R(0), e2 = R(0), e3 = R(0);
+          float2 EVT = make_float2(t, t), EBW = make_float2(0.f, 0.f), EWW = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int l = 0; l < DP; ++l) {
+            if (l < k) continue;
+            if constexpr (CS == 2) {
+              const float2 ff = reinterpret_cast<const float2*>(bc4)[i4];
+              EVT = __ffma2_rn(ff, make_float2(z[l], zT[l]), EVT);
+              EBW = __ffma2_rn(ff, make_float2(bt[l], W[i][l]), EBW);
+              EWW = __ffma2_rn(ff, make_float2(W[j][l], W[k][l]), EWW);
+            } else {
+              const R f = bc4[i4];
+              ev += f * z[l];
+              eT += f * zT[l];
+              eb += f * bt[l];
+              if (i > 0) e1 += f * W[i][l];
+              if (j > 0) e2 += f * W[j][l];
+              if (k > 0) e3 += f * W[k][l];
+            }
+            ++i4;
+          }
+          if constexpr (CS == 2) {
+            ev = EVT.x;
+            eT = EVT.y;
+            eb = EBW.x;
+            e1 = EBW.y;
+            e2 = EWW.x;
+            e3 = EWW.y;
+          }
+          if (i > 0)
+            H += ev * (W[i][j] * z[k] + W[i][k] * z[j] + W[j][k] * z[i]) + z[j] * (z[k] * e1) + z[i] * (z[k] * e2);
+          else if (j > 0)
+            H += z[i] * (ev * W[j][k] + z[k] * e2);
+          if (k > 0) H += z[i] * (z[j] * e3);
+          av += z[k] * ev;
+          ab += z[k] * eb + bt[k] * ev;
+          aT += zT[k] * eT;
+          // keep the coefficient loads of one (i, j, k) group together
+          asm volatile("" ::: "memory");
+        }
+        ++ic;
+      }
+      if constexpr (DEG == 3) {
+        if constexpr (CS == 2) {
+          av = VT.x;
+          aT = VT.y;
+          ab = BW.x;
+          w1 = BW.y;
+        }
+        if (i > 0) H += W[i][j] * av + z[j] * w1;
+        if (j > 0) H += z[i] * w2;
+      }
+      bv += z[j] * av;
+      bb += z[j] * ab + bt[j] * av;
+      bT += zT[j] * aT;
+      asm volatile("" ::: "memory");
+    }
+    uv += z[i] * bv;
+    ub += z[i] * bb + bt[i] * bv;
+    sT += zT[i] * bT;
+  }
+  u = uv;
+  uT = sT;
+  gen = ub + H;
 }
 
 // ---------------------------------------------------------------------------
@@ -855,7 +999,10 @@ __device__ __forceinline__ void load_state(const float4* p, int stride, R (&X)[D
 }
 
 // The Euler path of one FP64 thread, from X (x0 on entry) to X_T, with the
-// states before and after step s* in Xs and Xn.  Bound by the FP64 pipe (two
+// states before and after step s* in Xs and Xn.  With a constant volatility
+// X is linear in the normals, X_n = x0 + n h (r - delta - sigma^2 / 2) +
+// sigma (L sum z): X, Xs and Xn are then the running sums of the normals
+// (0 on entry), one FP64 instruction per asset and step.  Bound by the FP64 pipe (two
 // lanes per SM and clock: 64 issue slots per instruction of a warp): with
 // the normals and the logistic function in fixed point (fx64.cuh) an asset's
 // step takes seven FP64 instructions (constant correlation, tanh
@@ -890,18 +1037,23 @@ __device__ __forceinline__ void euler_path_f64(const Args<double, D>& a, const d
       for (int r = 0; r < 2; ++r) {
         if (s < a.N) {
           const double x = X[j];
-          double y;
-          if constexpr (CC) {
-            y = a.Ld[j] * z[r] + pre;
-            pre += a.Lc[j] * z[r];
+          double xn;
+          if constexpr (VK == VK_CONST) {
+            xn = x + z[r];
           } else {
-            zs[j] = z[r];
-            y = 0.0;
+            double y;
+            if constexpr (CC) {
+              y = a.Ld[j] * z[r] + pre;
+              pre += a.Lc[j] * z[r];
+            } else {
+              zs[j] = z[r];
+              y = 0.0;
 #pragma unroll 1
-            for (int c = 0; c <= j; ++c) y += a.L[j][c] * zs[c];
+              for (int c = 0; c <= j; ++c) y += a.L[j][c] * zs[c];
+            }
+            const double sig = sigma_j<VK>(a, row, j, x);
+            xn = sig * (nhh * sig + y) + (h * a.rd[j] + x);
           }
-          const double sig = sigma_j<VK>(a, row, j, x);
-          const double xn = sig * (nhh * sig + y) + (h * a.rd[j] + x);
           X[j] = xn;
           if (s == sstar) {
             Xs[j] = x;
@@ -1075,13 +1227,14 @@ __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
     constexpr bool VOTE = copy_vote(EV, D) && !XCOPY;
     constexpr bool REBUILD = sizeof(R) == 4 && VOTE;
     const int g_hit = sstar - sstar % G;  // first step of the group that contains s*
+    constexpr bool ZSUM = sizeof(R) == 8 && VK == VK_CONST;  // states are sums of normals
     R X[D], Xg[D], Xs[D], Xn[D];
 #pragma unroll
     for (int j = 0; j < D; ++j) {
-      X[j] = x0[j];
-      Xg[j] = x0[j];
-      Xs[j] = x0[j];
-      Xn[j] = x0[j];
+      X[j] = ZSUM ? R(0) : x0[j];
+      Xg[j] = X[j];
+      Xs[j] = X[j];
+      Xn[j] = X[j];
     }
     const R nhh = R(-0.5) * h;
     const PhiloxFixed pz = philox_fix(a, (uint32_t)m, (uint32_t)i, tagZ);
@@ -1182,20 +1335,28 @@ __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
     }
     const R* tab_s = tab + sstar * a.tab_stride;
     const R bb = Math<R>::sqrt(theta * (R(1) - theta) * h);
-    R Xtau[D], sig_s[D], drift_s[D];
-#pragma unroll(sizeof(R) == 8 ? 1 : D)
-    for (int j = 0; j < D; ++j) {
-      R y = 0;
-      if constexpr (sizeof(R) == 8) {
+    R Xtau[D], sig_s[D], drift_s[D], y[D];
+    if constexpr (ZSUM) {
 #pragma unroll 1
-        for (int q = 0; q <= j; ++q) y += a.L[j][q] * zb[q];
-      } else {
-#pragma unroll
-        for (int q = 0; q <= j; ++q) y += a.L[j][q] * zb[q];
+      for (int j = 0; j < D; ++j) zb[j] = Xs[j] + theta * (Xn[j] - Xs[j]) + bb * zb[j];
+      correlate<CC>(a, zb, y);
+#pragma unroll 1
+      for (int j = 0; j < D; ++j) {
+        sig_s[j] = a.va[j];
+        drift_s[j] = a.rd[j] - R(0.5) * a.va[j] * a.va[j];
+        Xtau[j] = a.va[j] * y[j] + (((R)sstar + theta) * h * drift_s[j] + x0[j]);
       }
-      sig_s[j] = sigma_j<VK>(a, tab_s, j, Xs[j]);
-      drift_s[j] = a.rd[j] - R(0.5) * sig_s[j] * sig_s[j];
-      Xtau[j] = Xs[j] + theta * (Xn[j] - Xs[j]) + sig_s[j] * bb * y;
+      correlate<CC>(a, X, y);
+#pragma unroll 1
+      for (int j = 0; j < D; ++j) X[j] = a.va[j] * y[j] + ((a.T - ti) * drift_s[j] + x0[j]);
+    } else {
+      correlate<CC>(a, zb, y);
+#pragma unroll(sizeof(R) == 8 ? 1 : D)
+      for (int j = 0; j < D; ++j) {
+        sig_s[j] = sigma_j<VK>(a, tab_s, j, Xs[j]);
+        drift_s[j] = a.rd[j] - R(0.5) * sig_s[j] * sig_s[j];
+        Xtau[j] = Xs[j] + theta * (Xn[j] - Xs[j]) + sig_s[j] * bb * y[j];
+      }
     }
     const R tau = ti + ((R)sstar + theta) * h;
     if constexpr (SYNC_EVAL) __syncthreads();
@@ -1226,6 +1387,8 @@ __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
       }
       if constexpr (EV >= EV_TREE4)
         eval_tree<R, D, EV>(a, s_alpha, z, zT, bt, st, u, gsum, uT);
+      else if constexpr (!CC)
+        eval_dense_full<EV == EV_DENSE4 ? 4 : 3, R, D, PAIRS ? 2 : 1>(a, s_alpha, z, zT, bt, st, u, gsum, uT);
       else if constexpr (EV == EV_DENSE4)
         eval_dense4<R, D, PAIRS ? 2 : 1>(a, s_alpha, z, zT, bt, st, u, gsum, uT);
       else
@@ -1488,9 +1651,15 @@ cudaError_t launch(const ModelHost& m, const GridHost& g, const ProblemDev& P, i
   const int npts = P.shard_n > 0 ? P.shard_n : P.n;
   if (npts <= 0) return cudaSuccess;
   const unsigned grid = (unsigned)npts * (unsigned)P.chunks;
-  if (dense) {  // implies a constant correlation
+  if (dense) {
     // the host selects: degree <= 3 loops (any d), degree-4 loops (d <= 5),
-    // the tree recursion of degree 4 (d >= 6) or 5 and 6 (d <= 5)
+    // or, with a constant correlation, the tree recursion of degree 4 (d >= 6)
+    // or 5 and 6 (d <= 5)
+    if (!cc) {
+      if (!P.dense4) return launch_ev<EV_DENSE3, false>(vk, a, grid, tpb, smem, st);
+      if constexpr (D <= 5) return launch_ev<EV_DENSE4, false>(vk, a, grid, tpb, smem, st);
+      return cudaErrorInvalidValue;
+    }
     switch (P.tree) {
       case 0:
         if (P.dense4) {

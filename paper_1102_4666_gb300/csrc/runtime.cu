@@ -354,8 +354,8 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
           "FP32 paths d <= 10) or, with FP32 paths, <= 6 (d <= 5)";
     return BSDE_ERR_INVALID_ARG;
   }
-  // the dense evaluation needs a constant correlation (all off-diagonal
-  // entries equal)
+  // the prefix-tree evaluation needs a constant correlation (all off-diagonal
+  // entries equal); the Horner loops have a form for a full matrix too
   bool const_corr = true;
   for (int i = 0; i < d; ++i)
     for (int j = 0; j < d; ++j)
@@ -364,7 +364,7 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
     err = "solve: eval_mode 2 (dense) needs a constant correlation";
     return BSDE_ERR_INVALID_ARG;
   }
-  s.dense = pm > 0 && const_corr && prm.eval_mode != 1;
+  s.dense = pm > 0 && (const_corr || tree_deg == 0) && prm.eval_mode != 1;
   s.dense4 = s.dense && tree_deg == 0 && mono_deg == 4;
   s.tree = s.dense ? tree_deg : 0;
   if (prm.ls_mode != 0 && prm.ls_mode != 1) {
