@@ -210,9 +210,9 @@ struct ProblemDev {
   double* qr_W = nullptr;     // [p][n_pad] design matrix, then R and the reflectors
   double* qr_y = nullptr;     // [n] right-hand side, then Q^T c
   double* qr_nrm = nullptr;   // [p] squared norms of the remaining columns
-  double* qr_tau = nullptr;   // [p] reflector coefficients
   int* qr_perm = nullptr;     // [p] column permutation
   int* qr_rank = nullptr;     // [1] numerical rank
+  uint32_t* qr_sync = nullptr;  // [2] grid barrier of the factorisation: arrivals, abort
 };
 
 // offsets in ProblemDev::out

@@ -5,8 +5,7 @@
 //
 // The design matrix X[i][l] = B_l(t_i, x_i) is stored column by column
 // (B[l][i], point index fastest), which is the layout Householder needs.
-// Step j: pick the remaining column of largest norm, swap it to position j,
-// build the reflector H_j = I - tau v v^T (v_0 = 1) that zeroes it below the
+// Step j: pick the remaining column of largest norm as column j, build the reflector H_j = I - tau v v^T (v_0 = 1) that zeroes it below the
 // diagonal, apply H_j to the remaining columns and to the right-hand side c,
 // and refresh the remaining columns' norms.  Columns whose diagonal |R_jj|
 // falls below 1e-13 |R_00| are treated as dependent (rank truncation); the
@@ -19,7 +18,9 @@ namespace {
 // copy B -> W, c -> y, squared column norms
 __global__ void k_qr_init(int n, int n_pad, int p, const double* __restrict__ B,
                           const double* __restrict__ c, double* __restrict__ W,
-                          double* __restrict__ y, double* __restrict__ nrm, int* __restrict__ perm) {
+                          double* __restrict__ y, double* __restrict__ nrm, int* __restrict__ perm,
+                          uint32_t* __restrict__ sync) {
+  if (blockIdx.x == 0 && threadIdx.x < 2) sync[threadIdx.x] = 0u;
   const int l = blockIdx.x;  // column (p of them) or the right-hand side (l == p)
   const double* src = (l < p) ? B + (size_t)l * n_pad : c;
   double* dst = (l < p) ? W + (size_t)l * n_pad : y;
@@ -42,162 +43,291 @@ __global__ void k_qr_init(int n, int n_pad, int p, const double* __restrict__ B,
   }
 }
 
-// step j: pivot (largest remaining norm, first index on ties), swap, reflector
-__global__ void __launch_bounds__(256) k_qr_pivot(int n, int n_pad, int p, int j,
-                                                  double* __restrict__ W, double* __restrict__ nrm,
-                                                  int* __restrict__ perm, double* __restrict__ tau) {
-  __shared__ double sv[256];
-  __shared__ int si[256];
-  __shared__ double s_beta, s_scale;
+constexpr int QR_THREADS = 256;
+constexpr int QR_WARPS = QR_THREADS / 32;
+// polls of a grid barrier before it gives up (each takes about a microsecond;
+// a step of the factorisation takes a few)
+constexpr uint32_t QR_WAIT_LIMIT = 1u << 24;
+
+// Sums of two values over the CTA, times k, in every thread.  A warp's FP64
+// instruction (a comparison too) holds the two-lane FP64 pipe for 64 cycles,
+// however few of its lanes matter: the threads' values are added by two warps
+// on different schedulers instead of by shuffles in every warp.  k is used by
+// warps 0 and 1 only.  buf: 2 x QR_THREADS values and 2 results; safe to call
+// again after another __syncthreads.
+__device__ __forceinline__ void qr_sum2(double& a, double& b, double k, double* buf) {
   const int tid = threadIdx.x;
-  double best = -1.0;
-  int bi = j;
-  for (int l = j + tid; l < p; l += 256) {
-    const double v = nrm[l];
-    if (v > best) {
-      best = v;
-      bi = l;
-    }
-  }
-  sv[tid] = best;
-  si[tid] = bi;
+  buf[tid] = a;
+  buf[QR_THREADS + tid] = b;
   __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (tid < o) {
-      const double a = sv[tid], b = sv[tid + o];
-      const int ia = si[tid], ib = si[tid + o];
-      if (b > a || (b == a && ib < ia)) {
-        sv[tid] = b;
-        si[tid] = ib;
-      }
-    }
-    __syncthreads();
-  }
-  const int piv = si[0];
-  if (piv != j) {
-    double* cj = W + (size_t)j * n_pad;
-    double* cp = W + (size_t)piv * n_pad;
-    for (int i = tid; i < n; i += 256) {
-      const double t = cj[i];
-      cj[i] = cp[i];
-      cp[i] = t;
-    }
-    if (tid == 0) {
-      const double t = nrm[j];
-      nrm[j] = nrm[piv];
-      nrm[piv] = t;
-      const int q = perm[j];
-      perm[j] = perm[piv];
-      perm[piv] = q;
-    }
+  if (tid < 64) {  // warp 0: the first value, warp 1: the second
+    const double* q = buf + (tid >> 5) * QR_THREADS + (tid & 31);
+    double t = ((q[0] + q[32]) + (q[64] + q[96])) + ((q[128] + q[160]) + (q[192] + q[224]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((tid & 31) == 0) buf[2 * QR_THREADS + (tid >> 5)] = k * t;
   }
   __syncthreads();
-  // Householder vector of x = W[j][j:n]
-  double* x = W + (size_t)j * n_pad;
-  double s = 0.0;
-  for (int i = j + 1 + tid; i < n; i += 256) s += x[i] * x[i];
-  sv[tid] = s;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (tid < o) sv[tid] += sv[tid + o];
-    __syncthreads();
-  }
-  if (tid == 0) {
-    const double x0 = x[j], sig = sv[0];
-    if (sig == 0.0 || j >= n) {
-      tau[j] = 0.0;
-      s_beta = x0;
-      s_scale = 0.0;
-    } else {
-      const double nx = sqrt(x0 * x0 + sig);
-      const double beta = x0 <= 0.0 ? nx : -nx;
-      tau[j] = (beta - x0) / beta;
-      s_beta = beta;
-      s_scale = 1.0 / (x0 - beta);
-    }
-  }
-  __syncthreads();
-  const double sc = s_scale;
-  for (int i = j + 1 + tid; i < n; i += 256) x[i] *= sc;  // v (v_0 = 1 implied)
-  if (tid == 0) x[j] = s_beta;                             // R_jj
+  a = buf[2 * QR_THREADS];
+  b = buf[2 * QR_THREADS + 1];
 }
 
-// step j: apply H_j to column l > j (block l - j - 1) or to y (last block),
-// then refresh the squared norm of the column below row j
-__global__ void __launch_bounds__(256) k_qr_apply(int n, int n_pad, int p, int j,
-                                                  double* __restrict__ W, double* __restrict__ y,
-                                                  double* __restrict__ nrm,
-                                                  const double* __restrict__ tau) {
-  __shared__ double red[8];
-  __shared__ double s_f;
-  const int l = j + 1 + blockIdx.x;
-  double* col = (l < p) ? W + (size_t)l * n_pad : y;
-  const double* v = W + (size_t)j * n_pad;
-  const int tid = threadIdx.x;
-  double s = 0.0;
-  for (int i = j + 1 + tid; i < n; i += 256) s += v[i] * col[i];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((tid & 31) == 0) red[tid >> 5] = s;
-  __syncthreads();
-  if (tid == 0) {
-    double t = col[j];  // v_0 = 1
-    for (int w = 0; w < 8; ++w) t += red[w];
-    const double f = tau[j] * t;
-    s_f = f;
-    col[j] -= f;
+// order of non-negative doubles as integers (no FP64 comparison), NaN last
+__device__ __forceinline__ long long qr_key(double a) {
+  const long long b = __double_as_longlong(a);
+  return b > 0x7ff0000000000000ll ? -1ll : b;
+}
+
+// 1 / a and sqrt(a) for normal a from the 20-bit FP64 approximations and
+// Newton steps (relative error below 2^-52): a tenth of the instructions of
+// the correctly rounded sequences, whose latency every step would wait for
+__device__ __forceinline__ double qr_rcp(double a) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+  r = fma(r, fma(-a, r, 1.0), r);
+  r = fma(r, fma(-a, r, 1.0), r);
+  return r;
+}
+__device__ __forceinline__ double qr_sqrt(double a) {
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+  double s = a * r;
+  const double h = 0.5 * r;
+  s = fma(h, fma(-s, s, a), s);
+  s = fma(h, fma(-s, s, a), s);
+  return s;
+}
+
+// The whole factorisation in one cooperative launch, one CTA per SM at most.
+// CTA b owns the columns b, b + CTAs, ... of W (the right-hand side is column
+// p) and keeps them up to date.  Columns stay where they are; pos[] holds the
+// logical order.  Step j:
+//   1. every CTA finds the pivot from the norms in memory; its norm is that of
+//      the rows from j on, so beta = -sign(x_0) sqrt(norm) needs no further
+//      pass, and with the reflector left unscaled, v = (x_0 - beta, x_1, ...),
+//      H = I - v v^T / (beta (beta - x_0)), none but the pivot column's load;
+//   2. each CTA applies H to its own columns and refreshes their norms;
+//   3. one grid barrier (the next step reads norms and the pivot column).
+// Bound by the FP64 pipe (three multiply-adds per element of a column, two
+// lanes per SM and clock: 1 us per column of 2000 rows) and by the latencies of
+// a step (barrier, pivot column from L2, two block sums).  Measured at n = 2000,
+// p = 210 (two columns per CTA), the whole refit in a graph: 3.69 ms with two
+// launches per column, 2.11 ms now (n = 700: 2.39 -> 1.45 ms).
+// sync[0]: arrivals (zero before the launch), sync[1]: set when a wait gave up.
+// STAGE: the pivot column is copied to shared memory (n doubles); KEEP: the
+// CTA's own columns are kept there too (and written through to W, where the
+// other CTAs read a pivot column).
+template <bool STAGE, bool KEEP>
+__global__ void __launch_bounds__(QR_THREADS, 1)
+    k_qr_factor(int n, int n_pad, int p, int steps, double* W, double* y, double* nrm, int* perm,
+                uint32_t* sync, int* status) {
+  extern __shared__ double qr_smem[];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int G = gridDim.x, me = blockIdx.x;
+  const int mine = (p - me) / G + 1;  // columns of this CTA (p + 1 in all, me <= p)
+  double* v = qr_smem;                // n (STAGE)
+  double* kept = qr_smem + n;         // mine x n (KEEP)
+  int* pos = reinterpret_cast<int*>(qr_smem + (STAGE ? (size_t)n : 0) +
+                                    (KEEP ? (size_t)n * (p / G + 1) : 0));  // p
+  uint8_t* done = reinterpret_cast<uint8_t*>(pos + p);                      // p + 1
+  __shared__ double buf[2 * QR_THREADS + 2];
+  __shared__ long long bv[QR_WARPS];
+  __shared__ int bw[QR_WARPS], s_abort;
+  for (int l = tid; l <= p; l += QR_THREADS) {
+    if (l < p) pos[l] = l;
+    done[l] = 0;
   }
-  __syncthreads();
-  const double f = s_f;
-  double q = 0.0;
-  for (int i = j + 1 + tid; i < n; i += 256) {
-    const double v2 = col[i] - f * v[i];
-    col[i] = v2;
-    q += v2 * v2;
-  }
-  if (l < p) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-    __syncthreads();
-    if ((tid & 31) == 0) red[tid >> 5] = q;
-    __syncthreads();
-    if (tid == 0) {
-      double t = 0.0;
-      for (int w = 0; w < 8; ++w) t += red[w];
-      nrm[l] = t;
+  if (KEEP) {
+    for (int q = 0; q < mine; ++q) {
+      const int l = me + q * G;
+      const double* col = l < p ? W + (size_t)l * n_pad : y;
+      for (int i = tid; i < n; i += QR_THREADS) kept[(size_t)q * n + i] = col[i];
     }
   }
+  if (tid == 0) s_abort = 0;
+  __syncthreads();
+  for (int j = 0; j < steps; ++j) {
+    // pivot: the largest remaining norm, the first logical column on ties
+    long long best = -1;
+    int bi = p;
+    for (int l = j + tid; l < p; l += QR_THREADS) {
+      const long long t = qr_key(__ldcg(nrm + pos[l]));
+      if (t > best) {
+        best = t;
+        bi = l;
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long t = __shfl_xor_sync(0xffffffffu, best, o);
+      const int it = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (t > best || (t == best && it < bi)) {
+        best = t;
+        bi = it;
+      }
+    }
+    if (lane == 0) {
+      bv[warp] = best;
+      bw[warp] = bi;
+    }
+    __syncthreads();
+    for (int w = 0; w < QR_WARPS; ++w) {
+      const long long t = bv[w];
+      const int it = bw[w];
+      if (t > best || (t == best && it < bi)) {
+        best = t;
+        bi = it;
+      }
+    }
+    if (bi >= p) bi = j;  // only NaN norms left
+    const int c = pos[bi];
+    const double* x = W + (size_t)c * n_pad;
+    const double x0 = __ldcg(x + j);
+    if (STAGE) {
+#pragma unroll 8
+      for (int i = j + 1 + tid; i < n; i += QR_THREADS) v[i] = __ldcg(x + i);
+    }
+    // beta, v_0 = x_0 - beta and 1 / (beta (beta - x_0)), in the two warps that
+    // use them; a column that is zero (to the range of the approximations) is
+    // left as it is
+    double beta = x0, v0 = 0.0, kap = 0.0;
+    if (warp < 2 && !(best >= 0 && best < 0x03c0000000000000ll)) {  // norm >= 2^-963 or NaN
+      const double nx = qr_sqrt(best < 0 ? nan("") : __longlong_as_double(best));
+      beta = x0 <= 0.0 ? nx : -nx;
+      v0 = x0 - beta;
+      kap = qr_rcp(-beta * v0);
+    }
+    // H on the columns of this CTA, two at a time
+    int q = 0;
+    while (q < mine) {
+      int ql[2], m = 0;
+      for (; q < mine && m < 2; ++q) {
+        const int l = me + q * G;
+        if (!done[l] && l != c) ql[m++] = q;
+      }
+      if (m == 0) break;
+      const int l0 = me + ql[0] * G, l1 = m < 2 ? l0 : me + ql[1] * G;
+      double* g0 = l0 < p ? W + (size_t)l0 * n_pad : y;
+      double* g1 = l1 < p ? W + (size_t)l1 * n_pad : y;
+      double* c0 = KEEP ? kept + (size_t)ql[0] * n : g0;
+      double* c1 = KEEP ? kept + (size_t)(m < 2 ? ql[0] : ql[1]) * n : g1;
+      double s0 = tid == 0 ? v0 * c0[j] : 0.0, s1 = tid == 0 && m == 2 ? v0 * c1[j] : 0.0;
+#pragma unroll 4
+      for (int i = j + 1 + tid; i < n; i += QR_THREADS) {
+        const double vi = STAGE ? v[i] : __ldcg(x + i);
+        s0 += vi * c0[i];
+        if (m == 2) s1 += vi * c1[i];
+      }
+      qr_sum2(s0, s1, kap, buf);
+      const double f0 = s0, f1 = s1;
+      double q0 = 0.0, q1 = 0.0;
+#pragma unroll 4
+      for (int i = j + 1 + tid; i < n; i += QR_THREADS) {
+        const double vi = STAGE ? v[i] : __ldcg(x + i);
+        const double n0 = c0[i] - f0 * vi;
+        c0[i] = n0;
+        if (KEEP) g0[i] = n0;
+        q0 += n0 * n0;
+        if (m == 2) {
+          const double n1 = c1[i] - f1 * vi;
+          c1[i] = n1;
+          if (KEEP) g1[i] = n1;
+          q1 += n1 * n1;
+        }
+      }
+      if (tid < m) {  // row j
+        double* cc = tid ? c1 : c0;
+        const double t = cc[j] - (tid ? f1 : f0) * v0;
+        cc[j] = t;
+        if (KEEP) (tid ? g1 : g0)[j] = t;
+      }
+      __syncthreads();  // the first sums have been read
+      qr_sum2(q0, q1, 1.0, buf);
+      if (tid == 0 && l0 < p) nrm[l0] = q0;
+      if (tid == 0 && m == 2 && l1 < p) nrm[l1] = q1;
+      __syncthreads();
+    }
+    // grid barrier; every wait is bounded
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      atomicAdd(sync, 1u);
+      pos[bi] = pos[j];
+      pos[j] = c;
+      done[c] = 1;
+      const uint32_t want = (uint32_t)(j + 1) * (uint32_t)G;
+      volatile uint32_t* cnt = sync;
+      uint32_t polls = 0;
+      while (*cnt < want) {
+        if (++polls > QR_WAIT_LIMIT || cnt[1] != 0) {
+          atomicExch(sync + 1, 1u);
+          atomicOr(status, ST_TIMEOUT);
+          s_abort = 1;
+          break;
+        }
+      }
+      __threadfence();
+      // R_jj, after every CTA has read x0
+      if (c % G == me && !s_abort) W[(size_t)c * n_pad + j] = beta;
+    }
+    __syncthreads();
+    if (s_abort) return;
+  }
+  if (me == 0)
+    for (int l = tid; l < p; l += QR_THREADS) perm[l] = pos[l];
 }
 
 // basic solution: rank r from |R_jj| > 1e-13 |R_00|, R_11 d = y_1 by back
-// substitution (one CTA, column-oriented), delta[perm[j]] = d_j (0 beyond r)
-__global__ void __launch_bounds__(256) k_qr_solve(int n_pad, int p, const double* __restrict__ W,
+// substitution, delta[perm[j]] = d_j (0 beyond r).  One CTA; blocks of 32
+// columns: warp 0 solves the block's triangle with shuffles, then every thread
+// takes the block's columns off its rows, the last column first.
+__global__ void __launch_bounds__(256) k_qr_solve(int n, int n_pad, int p, const double* __restrict__ W,
                                                   const double* __restrict__ y,
                                                   const int* __restrict__ perm,
                                                   double* __restrict__ delta,
                                                   double* __restrict__ work, int* __restrict__ rank_out) {
   __shared__ int s_rank;
-  __shared__ double s_x;
-  const int tid = threadIdx.x;
-  if (tid == 0) {
-    const double r00 = fabs(W[0]);
-    int r = 0;
-    while (r < p && fabs(W[(size_t)r * n_pad + r]) > 1e-13 * r00) ++r;
-    s_rank = r;
-    *rank_out = r;
-  }
+  __shared__ double xs[32];
+  __shared__ const double* cols[32];
+  __shared__ double tri[32][33];
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid == 0) s_rank = p;
+  __syncthreads();
+  const double r00 = fabs(W[(size_t)perm[0] * n_pad]);
+  for (int c = tid; c < p; c += 256)
+    if (c >= n || !(fabs(W[(size_t)perm[c] * n_pad + c]) > 1e-13 * r00)) atomicMin(&s_rank, c);
   __syncthreads();
   const int r = s_rank;
+  if (tid == 0) *rank_out = r;
   for (int q = tid; q < p; q += 256) work[q] = (q < r) ? y[q] : 0.0;
   __syncthreads();
-  for (int c = r - 1; c >= 0; --c) {
-    if (tid == 0) {
-      s_x = work[c] / W[(size_t)c * n_pad + c];
-      work[c] = s_x;
+  for (int c1 = r; c1 > 0; c1 -= 32) {
+    const int c0 = max(0, c1 - 32), nb = c1 - c0;
+    if (tid < 32) {
+      const double* col = W + (size_t)perm[lane < nb ? c0 + lane : c0] * n_pad;
+      cols[lane] = col;
+      __syncwarp();
+#pragma unroll 8
+      for (int c = 0; c < nb; ++c)
+        if (lane < c) tri[c][lane] = cols[c][c0 + lane];
+      __syncwarp();
+      double w = lane < nb ? work[c0 + lane] : 0.0;
+      const double dg = lane < nb ? qr_rcp(col[c0 + lane]) : 1.0;
+      for (int c = nb - 1; c >= 0; --c) {
+        if (lane == c) w *= dg;
+        const double xc = __shfl_sync(0xffffffffu, w, c);
+        if (lane < c) w -= tri[c][lane] * xc;
+      }
+      xs[lane] = w;
+      if (lane < nb) work[c0 + lane] = w;
     }
     __syncthreads();
-    const double xc = s_x;
-    for (int q = tid; q < c; q += 256) work[q] -= W[(size_t)c * n_pad + q] * xc;  // R_qc = W[c][q]
+    for (int q = tid; q < c0; q += 256) {
+      double w = work[q];
+#pragma unroll 8
+      for (int c = nb - 1; c >= 0; --c) w -= cols[c][q] * xs[c];  // R_qc = W[perm[c]][q]
+      work[q] = w;
+    }
     __syncthreads();
   }
   for (int q = tid; q < p; q += 256) delta[perm[q]] = work[q];
@@ -206,15 +336,25 @@ __global__ void __launch_bounds__(256) k_qr_solve(int n_pad, int p, const double
 }  // namespace
 
 // delta = argmin |c - X delta| by pivoted QR; the workspace (W: p x n_pad,
-// y: n, norms, tau, perm, rank) is P.qr_*
+// y: n, norms, perm, rank, the barrier's words) is P.qr_*
 void launch_qr_solve(const ProblemDev& P, cudaStream_t st) {
   k_qr_init<<<P.p + 1, 256, 0, st>>>(P.n, P.n_pad, P.p, P.B, P.c, P.qr_W, P.qr_y, P.qr_nrm,
-                                     P.qr_perm);
-  const int steps = P.p < P.n ? P.p : P.n;
-  for (int j = 0; j < steps; ++j) {
-    k_qr_pivot<<<1, 256, 0, st>>>(P.n, P.n_pad, P.p, j, P.qr_W, P.qr_nrm, P.qr_perm, P.qr_tau);
-    k_qr_apply<<<P.p - j, 256, 0, st>>>(P.n, P.n_pad, P.p, j, P.qr_W, P.qr_y, P.qr_nrm, P.qr_tau);
-  }
-  k_qr_solve<<<1, 256, 0, st>>>(P.n_pad, P.p, P.qr_W, P.qr_y, P.qr_perm, P.delta, P.res,
-                                P.qr_rank);
+                                     P.qr_perm, P.qr_sync);
+  int n = P.n, n_pad = P.n_pad, p = P.p, steps = P.p < P.n ? P.p : P.n;
+  double *W = P.qr_W, *y = P.qr_y, *nrm = P.qr_nrm;
+  int *perm = P.qr_perm, *status = P.status;
+  uint32_t* sync = P.qr_sync;
+  const int sms = device_sm_count();
+  const int grid = p + 1 < sms ? p + 1 : sms;
+  const size_t order = (size_t)p * 5 + 16, col = (size_t)n * 8, room = 200 * 1024;  // order: pos and done
+  const bool stage = col + order <= room;
+  const bool keep = col * (1 + (size_t)(p / grid + 1)) + order <= room;
+  const size_t smem = order + (keep ? col * (1 + (size_t)(p / grid + 1)) : stage ? col : 0);
+  const void* kern = keep    ? (const void*)k_qr_factor<true, true>
+                     : stage ? (const void*)k_qr_factor<true, false>
+                             : (const void*)k_qr_factor<false, false>;
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  void* args[] = {&n, &n_pad, &p, &steps, &W, &y, &nrm, &perm, &sync, &status};
+  cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(QR_THREADS), args, smem, st);
+  k_qr_solve<<<1, 256, 0, st>>>(n, n_pad, p, W, y, perm, P.delta, P.res, P.qr_rank);
 }

@@ -486,9 +486,9 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
       P.qr_W = (double*)take((size_t)p * s.n_pad * 8);
       P.qr_y = (double*)take((size_t)n * 8);
       P.qr_nrm = (double*)take((size_t)p * 8 * 2);
-      P.qr_tau = P.qr_nrm + p;
       P.qr_perm = (int*)take((size_t)p * 4 + 16);
       P.qr_rank = P.qr_perm + p;
+      P.qr_sync = (uint32_t*)(P.qr_rank + 1);
     }
     dev = P;
     coeffs_valid = false;
@@ -889,15 +889,14 @@ int Problem::finish_report(const bsde_solve_params& prm, cudaStream_t st, bsde_r
     r.path_launches = prm.K_it;
     r.rank = rank;
     // launches: per iteration points, basis, (monomial conversion), paths,
-    // reduce, refit (QR: init, pivot + apply per step, solve; otherwise
+    // reduce, refit (QR: init, factorisation, solve; otherwise
     // rhs, inverse product, 3 per refinement step), update, read-out (3);
     // per factorised Gram matrix points, basis, Gram (+ split-K reduce in
     // mixed precision); per group save_diag, 3 per panel but the last
     // (diag, trsm, update), the last panel's diag, the batched inverse
     const int panels = (shape.p + 31) / 32;
-    const int steps_qr = shape.p < shape.n ? shape.p : shape.n;
     const int refine2 = prm.refine_steps >= 0 ? prm.refine_steps : (mixed ? 2 : 1);
-    const int refit = shape.qr ? (2 + 2 * steps_qr) : (2 + 3 * refine2);
+    const int refit = shape.qr ? 3 : (2 + 3 * refine2);
     int groups = 0, mats = 0;
     if (!shape.qr) {
       groups = grid.resample ? (prm.K_it + nfact - 1) / nfact : 1;

@@ -57,3 +57,19 @@ def test_qr_solve_matches_normal_equation_solve():
     assert r1.rank == r1.p
     assert rel(a_qr, a_chol) < 1e-8
     assert abs(r1.price - r0.price) < 1e-8 * abs(r0.price)
+
+
+@pytest.mark.parametrize("n,d,eta", [(26000, 1, 2), (33, 1, 1), (257, 2, 3), (1001, 5, 4), (1400, 6, 4)])
+def test_qr_refit_at_the_edges_of_its_kernel(n, d, eta):
+    """The cooperative factorisation with the reflector read from memory
+    (n above the shared memory), with one, two and three columns per CTA, with
+    fewer columns than SMs, and n next to the CTA's and the warp's size."""
+    import paper_1102_4666_gb300 as G
+    cfg = workloads.make(d=d, T=1.0, r=0.03, K=100.0, S0=100.0, vol={"kind": "const", "a": 0.2},
+                         rho=0.3 if d > 1 else 0.0, lam=0.0, n=n, M=2, N=2, eta=eta, K_it=1, seed=9)
+    nu = O.multi_index_set(d + 1, eta)
+    a0 = np.random.default_rng(5).standard_normal(len(nu)) * 0.3
+    s = G.Solver(cfg, precision="fp64")
+    t, x, c, a1 = s.iterate(0, a0, ls_mode=1)
+    s.close()
+    assert rel(a1 - a0, O.fit(O.basis_matrix(cfg, nu, t, x), c)) < 1e-9
