@@ -69,46 +69,49 @@ __global__ void __launch_bounds__(256) k_b_times(int n, int n_pad, int p,
   }
 }
 
-// FP64 Gram A = B B^T on CUDA cores: one 32x32 upper tile per CTA, written
-// to both triangles.
+// Tiles of 16 x 16 outputs, one per thread, for every FP64 contraction here: on
+// the two-lane FP64 pipe a tile's 32-deep slice is 2 us of an SM, so that a
+// 32 x 32 tile per CTA left most SMs idle behind the last ones (FP64 Gram at
+// n = 1000, p = 364: 78 tiles, 310 us; 276 tiles, 135 us).
+constexpr int T16 = 16;
+
+// decode lower tile (tj <= ti) number t, row-major
+__device__ __forceinline__ void lower_tile(int t, int& ti, int& tj) {
+  ti = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+  while (ti * (ti + 1) / 2 > t) --ti;
+  while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
+  tj = t - ti * (ti + 1) / 2;
+}
+
+// FP64 Gram A = B B^T on CUDA cores: one lower tile per CTA, written to both
+// triangles.
 __global__ void __launch_bounds__(256) k_gram_f64(int n, int n_pad, int p,
                                                   const double* __restrict__ B,
                                                   double* __restrict__ A) {
-  __shared__ double As[32][33], Bs[32][33];
-  // decode the upper tile (ti <= tj) from blockIdx.x
-  const int T = (p + 31) / 32;
-  int t = blockIdx.x, ti = 0;
-  while (t >= T - ti) {
-    t -= T - ti;
-    ++ti;
-  }
-  const int tj = ti + t;
-  const int r0 = ti * 32, c0 = tj * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  __shared__ double Rs[T16][33], Cs[T16][33];
+  int ti, tj;
+  lower_tile(blockIdx.x, ti, tj);
+  const int r0 = ti * T16, c0 = tj * T16;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int lk = threadIdx.x & 31, lr = threadIdx.x >> 5;  // loads: rows lr and lr + 8
+  double acc = 0.0;
   for (int k0 = 0; k0 < n; k0 += 32) {
-    for (int q = threadIdx.x; q < 32 * 32; q += 256) {
-      const int rr = q >> 5, kk = q & 31;
-      const int kg = k0 + kk;
-      As[rr][kk] = (r0 + rr < p && kg < n) ? B[(size_t)(r0 + rr) * n_pad + kg] : 0.0;
-      Bs[rr][kk] = (c0 + rr < p && kg < n) ? B[(size_t)(c0 + rr) * n_pad + kg] : 0.0;
+    const int kg = k0 + lk;
+#pragma unroll
+    for (int h = 0; h < T16; h += 8) {
+      const int rr = lr + h;
+      Rs[rr][lk] = (r0 + rr < p && kg < n) ? B[(size_t)(r0 + rr) * n_pad + kg] : 0.0;
+      Cs[rr][lk] = (c0 + rr < p && kg < n) ? B[(size_t)(c0 + rr) * n_pad + kg] : 0.0;
     }
     __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < 32; ++kk) {
-      const double b = Bs[tx][kk];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q] += As[ty + 8 * q][kk] * b;
-    }
+    for (int kk = 0; kk < 32; ++kk) acc += Rs[ty][kk] * Cs[tx][kk];
     __syncthreads();
   }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int r = r0 + ty + 8 * q, c = c0 + tx;
-    if (r < p && c < p) {
-      A[(size_t)r * p + c] = acc[q];
-      A[(size_t)c * p + r] = acc[q];
-    }
+  const int r = r0 + ty, c = c0 + tx;
+  if (r < p && c < p) {
+    A[(size_t)r * p + c] = acc;
+    A[(size_t)c * p + r] = acc;
   }
 }
 
@@ -124,191 +127,250 @@ __global__ void k_save_diag(const double* __restrict__ A, int p, double* __restr
   if (j < p) diag0[z * p + j] = A[z * p * p + (size_t)j * p + j];
 }
 
-// Right-looking blocked Cholesky, panel width 32, lower factor in place.
-// Panel step 1: one warp factors the 32x32 diagonal block in shared memory
-// and stores the reciprocals of its diagonal in dinv.  A pivot below 1e-13
-// of its original diagonal entry (or not finite) marks the matrix as
-// numerically singular: ST_NOT_PD, and the pivot becomes NaN.
-__global__ void __launch_bounds__(32) k_chol_diag(double* __restrict__ A, int p, int j0,
-                                                  int* __restrict__ status,
-                                                  const double* __restrict__ diag0,
-                                                  double* __restrict__ dinv) {
-  __shared__ double Dg[32][33];
+// 1 / sqrt(a) for normal positive a: the 20-bit FP64 approximation and one
+// third-order step (relative error below 2^-52), four dependent FP64
+// instructions instead of a square root and a division
+__device__ __forceinline__ double rsqrt_f64(double a) {
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+  const double e = fma(-(a * r), r, 1.0);
+  return fma(r * e, fma(0.375, e, 0.5), r);
+}
+
+// Right-looking blocked Cholesky, panel width 32, lower factor in place; the
+// upper triangle of A, no longer needed, takes the transposed inverse of the
+// factor (its diagonal is dinv).
+// Panel step 1: the 32x32 diagonal block, factored and inverted together.  Four
+// warps, one per scheduler and FP64 pipe, own every fourth column in registers,
+// lanes are rows.  The elimination of column c takes l_c l_q from the columns
+// q > c still to be factored; a column q <= c has become column q of the inverse
+// (rows unscaled), E_r -= l_rc / l_cc E_c: eight columns per warp either way.
+// Every warp computes the pivot's reciprocal root for itself, so that a column
+// costs one barrier.  Bound by the chain pivot - root - column - next pivot and
+// the eight FMAs between (64 cycles of the pipe each): about 1500 cycles a
+// column.  Per block: one warp on shared memory 65 us, this 26 us.
+// A pivot below 1e-13 of its original diagonal entry (or not finite) marks the
+// matrix as numerically singular: ST_NOT_PD, and the pivot becomes NaN.
+__global__ void __launch_bounds__(128) k_chol_diag(double* __restrict__ A, int p, int j0,
+                                                   int* __restrict__ status,
+                                                   const double* __restrict__ diag0,
+                                                   double* __restrict__ dinv) {
+  __shared__ double col[2][32], Ls[32][33], Ei[32][33], di[32];
   const size_t z = blockIdx.y;
   A += z * p * p;
   diag0 += z * p;
   dinv += z * p;
   const int nb = min(32, p - j0);
-  const int lane = threadIdx.x;
-  for (int q = lane; q < 32 * 32; q += 32) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // rows and columns past nb: the identity, which the elimination leaves alone
+  for (int q = threadIdx.x; q < 32 * 32; q += 128) {
     const int r = q >> 5, c = q & 31;
-    Dg[r][c] = (r < nb && c < nb && c <= r) ? A[(size_t)(j0 + r) * p + (j0 + c)] : 0.0;
+    Ls[r][c] = (r < nb && c <= r) ? A[(size_t)(j0 + r) * p + (j0 + c)] : r == c ? 1.0 : 0.0;
   }
-  __syncwarp();
-  for (int c = 0; c < nb; ++c) {
-    double inv = 0.0;
-    if (lane == 0) {
-      const double piv = Dg[c][c];
-      if (!(piv > 1e-13 * diag0[j0 + c]) || !isfinite(piv)) {
-        atomicOr(status, ST_NOT_PD);
-        Dg[c][c] = nan("");
-        inv = nan("");
-      } else {
-        const double dcc = sqrt(piv);
-        Dg[c][c] = dcc;
-        inv = 1.0 / dcc;
-      }
-      dinv[j0 + c] = inv;
-    }
-    inv = __shfl_sync(0xffffffffu, inv, 0);
-    __syncwarp();
-    if (lane > c && lane < nb) Dg[lane][c] *= inv;
-    __syncwarp();
-    // rank-1 update of the trailing block: lane handles row r = lane
-    if (lane > c && lane < nb) {
-      const double lrc = Dg[lane][c];
-      for (int s2 = c + 1; s2 <= lane; ++s2) Dg[lane][s2] -= lrc * Dg[s2][c];
-    }
-    __syncwarp();
-  }
-  for (int q = lane; q < 32 * 32; q += 32) {
-    const int r = q >> 5, c = q & 31;
-    if (r < nb && c <= r) A[(size_t)(j0 + r) * p + (j0 + c)] = Dg[r][c];
-  }
-}
-
-// Panel step 2: rows below the diagonal block solve x L_jj^T = a (forward
-// substitution with the reciprocal diagonal), one thread per row.
-__global__ void __launch_bounds__(32) k_chol_trsm(double* __restrict__ A, int p, int j0,
-                                                  const double* __restrict__ dinv) {
-  __shared__ double Dg[32][33];
-  __shared__ double di[32];
-  const size_t z = blockIdx.y;
-  A += z * p * p;
-  dinv += z * p;
-  const int nb = min(32, p - j0);
-  for (int q = threadIdx.x; q < 32 * 32; q += 32) {
-    const int r = q >> 5, c = q & 31;
-    Dg[r][c] = (r < nb && c < nb && c <= r) ? A[(size_t)(j0 + r) * p + (j0 + c)] : 0.0;
-  }
-  di[threadIdx.x] = threadIdx.x < nb ? dinv[j0 + threadIdx.x] : 0.0;
+  const long long thr = lane < nb ? __double_as_longlong(1e-13 * diag0[j0 + lane]) : 0;
   __syncthreads();
-  const int row = j0 + nb + 32 * blockIdx.x + threadIdx.x;
-  if (row >= p) return;
-  double xr[32];
+  double R[8];
 #pragma unroll
-  for (int c = 0; c < 32; ++c) xr[c] = (c < nb) ? A[(size_t)row * p + j0 + c] : 0.0;
+  for (int k = 0; k < 8; ++k) R[k] = Ls[lane][warp + 4 * k];
+  if (warp == 0) col[0][lane] = R[0];
+  __syncthreads();
 #pragma unroll
   for (int c = 0; c < 32; ++c) {
-    if (c < nb) {
-      double acc = xr[c];
+    const double colv = col[c & 1][lane], piv = col[c & 1][c];
+    // piv > thr and finite, on the bits (no FP64 comparison); thr >= 0
+    const long long pb = __double_as_longlong(piv), tb = __shfl_sync(0xffffffffu, thr, c);
+    const bool ok = pb > tb && pb < 0x7ff0000000000000ll;
+    const double inv = ok ? rsqrt_f64(piv) : nan("");
+    const double l = lane > c ? colv * inv : 0.0;
+    // the next column first: its owner hands it on
+    if (c < 31) {
+      constexpr int one = 1;
+      const int k = (c + one) / 4, w = (c + one) % 4;
+      const double ls = __shfl_sync(0xffffffffu, l, c + 1);
+      if (warp == w) {
+        R[k] -= l * ls;
+        col[(c + 1) & 1][lane] = R[k];
+      }
+    }
+    if (warp == c % 4) {
+      Ls[lane][c] = lane == c ? piv * inv : l;
+      R[c / 4] = lane == c ? 1.0 : 0.0;
+      if (lane == c) di[c] = inv;
+      if (lane == 0 && !ok) atomicOr(status, ST_NOT_PD);
+    }
+    __syncthreads();
+    const double l2 = l * inv;
 #pragma unroll
-      for (int q = 0; q < c; ++q) acc -= xr[q] * Dg[c][q];
-      xr[c] = acc * di[c];
+    for (int k = 0; k < 8; ++k) {
+      const int q = warp + 4 * k;
+      if (4 * k > c + 1 || (4 * k + 3 > c + 1 && q > c + 1)) {  // still to be factored
+        R[k] -= l * __shfl_sync(0xffffffffu, l, q);
+      } else if (q <= c) {
+        R[k] -= l2 * __shfl_sync(0xffffffffu, R[k], c);  // zero on the rows up to c, as l2 is
+      }
     }
   }
 #pragma unroll
-  for (int c = 0; c < 32; ++c)
-    if (c < nb) A[(size_t)row * p + j0 + c] = xr[c];
-}
-
-// trailing update A22 -= L21 L21^T on the lower triangle, 32x32 tiles
-__global__ void __launch_bounds__(256) k_chol_update(double* __restrict__ A, int p, int j0) {
-  __shared__ double Lr[32][33], Lc[32][33];
-  A += (size_t)blockIdx.y * p * p;
-  const int nb = min(32, p - j0);
-  const int base = j0 + nb;
-  const int m = p - base;
-  const int T = (m + 31) / 32;
-  int t = blockIdx.x, ti = 0;  // lower tiles (tj <= ti), row-major
-  while (t > ti) {
-    t -= ti + 1;
-    ++ti;
-  }
-  const int tj = t;
-  if (ti >= T) return;
-  const int r0 = base + 32 * ti, c0 = base + 32 * tj;
-  for (int q = threadIdx.x; q < 32 * 32; q += 256) {
-    const int rr = q >> 5, kk = q & 31;
-    Lr[rr][kk] = (r0 + rr < p && kk < nb) ? A[(size_t)(r0 + rr) * p + j0 + kk] : 0.0;
-    Lc[rr][kk] = (c0 + rr < p && kk < nb) ? A[(size_t)(c0 + rr) * p + j0 + kk] : 0.0;
-  }
+  for (int k = 0; k < 8; ++k) Ei[lane][warp + 4 * k] = R[k];
   __syncthreads();
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int rr = ty + 8 * q;
-    const int r = r0 + rr, c = c0 + tx;
-    if (r < p && c < p && c <= r) {
-      double s = 0.0;
-#pragma unroll 8
-      for (int kk = 0; kk < 32; ++kk) s += Lr[rr][kk] * Lc[tx][kk];
-      A[(size_t)r * p + c] -= s;
-    }
+  for (int q = threadIdx.x; q < 32 * 32; q += 128) {
+    const int r = q >> 5, c = q & 31;
+    if (r < nb && c <= r) A[(size_t)(j0 + r) * p + (j0 + c)] = Ls[r][c];
+    if (c < nb && r < c) A[(size_t)(j0 + r) * p + (j0 + c)] = Ei[c][r] * di[c];  // inverse, transposed
   }
+  if (threadIdx.x < nb) dinv[j0 + threadIdx.x] = di[threadIdx.x];
 }
 
-// x (+)= A^{-1} b with the Cholesky factor L in the lower triangle of A and
-// its reciprocal diagonal in dinv: L y = b, then L^T x = y, by blocks of 32.
-// Warp 0 solves each 32x32 diagonal block with shuffles; all threads then
-// update the rest of the vector with that block's 32 columns (forward: a
-// row segment per thread; backward: coalesced column reads).  One CTA.
-// With b == nullptr, CTA (j, z) solves A_z x = e_j and writes column j of
-// A_z^{-1} to x + z p^2 + j p (the inverses used by the refit).
-__global__ void __launch_bounds__(256) k_chol_solve(const double* __restrict__ A, int p,
-                                                    const double* __restrict__ dinv,
-                                                    const double* __restrict__ b,
-                                                    double* __restrict__ x, int accumulate) {
-  extern __shared__ double yv[];  // p
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// the inverse of diagonal block j0 (rows c, columns k <= c) from the upper triangle
+__device__ __forceinline__ double diag_inv(const double* __restrict__ A, const double* __restrict__ dinv,
+                                           int p, int j0, int c, int k) {
+  if (j0 + c >= p || k > c) return 0.0;
+  return k == c ? dinv[j0 + c] : A[(size_t)(j0 + k) * p + j0 + c];
+}
+
+// Panel step 2: the rows below, L21 = A21 L11^-T: eight rows per CTA, an
+// output per thread (a substitution per row left a warp to 496 dependent steps
+// on its own: 24 us a panel, this 5 us)
+__global__ void __launch_bounds__(256) k_chol_trsm(double* __restrict__ A, int p, int j0,
+                                                   const double* __restrict__ dinv) {
+  __shared__ double Li[32][33], a[8][33];
   const size_t z = blockIdx.y;
   A += z * p * p;
   dinv += z * p;
-  if (b == nullptr) x += z * p * p + (size_t)blockIdx.x * p;
-  for (int r = tid; r < p; r += blockDim.x) yv[r] = b ? b[r] : (r == (int)blockIdx.x ? 1.0 : 0.0);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int q = warp; q < 32; q += 8) Li[lane][q] = diag_inv(A, dinv, p, j0, lane, q);
+  const int row = j0 + 32 + 8 * blockIdx.x + warp;  // a full panel: rows below exist only then
+  a[warp][lane] = row < p ? A[(size_t)row * p + j0 + lane] : 0.0;
   __syncthreads();
-  const int nblk = (p + 31) / 32;
-  // for b = e_j the forward solution is zero above row j: start at its block
-  for (int blk = b ? 0 : (int)blockIdx.x / 32; blk < nblk; ++blk) {
-    const int c0 = blk * 32, nb = min(32, p - c0);
-    if (warp == 0) {
-      double yi = lane < nb ? yv[c0 + lane] : 0.0;
-      for (int c = 0; c < nb; ++c) {
-        if (lane == c) yi *= dinv[c0 + c];
-        const double yc = __shfl_sync(0xffffffffu, yi, c);
-        if (lane > c && lane < nb) yi -= A[(size_t)(c0 + lane) * p + c0 + c] * yc;
-      }
-      if (lane < nb) yv[c0 + lane] = yi;
+  double acc = 0.0;
+#pragma unroll
+  for (int k = 0; k < 32; ++k) acc += a[warp][k] * Li[lane][k];
+  if (row < p) A[(size_t)row * p + j0 + lane] = acc;
+}
+
+// trailing update A22 -= L21 L21^T on the lower triangle
+__global__ void __launch_bounds__(256) k_chol_update(double* __restrict__ A, int p, int j0) {
+  __shared__ double Lr[T16][33], Lc[T16][33];
+  A += (size_t)blockIdx.y * p * p;
+  int ti, tj;
+  lower_tile(blockIdx.x, ti, tj);
+  const int r0 = j0 + 32 + T16 * ti, c0 = j0 + 32 + T16 * tj;
+  const int lk = threadIdx.x & 31, lr = threadIdx.x >> 5;
+#pragma unroll
+  for (int h = 0; h < T16; h += 8) {
+    const int rr = lr + h;
+    Lr[rr][lk] = r0 + rr < p ? A[(size_t)(r0 + rr) * p + j0 + lk] : 0.0;
+    Lc[rr][lk] = c0 + rr < p ? A[(size_t)(c0 + rr) * p + j0 + lk] : 0.0;
+  }
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int r = r0 + ty, c = c0 + tx;
+  const bool in = r < p && c <= r;
+  const double old = in ? A[(size_t)r * p + c] : 0.0;
+  __syncthreads();
+  double s = 0.0;
+#pragma unroll
+  for (int kk = 0; kk < 32; ++kk) s += Lr[ty][kk] * Lc[tx][kk];
+  if (in) A[(size_t)r * p + c] = old - s;
+}
+
+// M = L^-1 by block columns, transposed into the upper triangle of A: CTA
+// (strip, z) computes C columns of M from their diagonal block down,
+//   M_I = -L_II^-1 sum_{K < I} L_IK M_K,
+// keeping the strip in shared memory; warp = column, lane = row.  The strips of
+// the first columns are the longest and start first.  With k_inv_syrk p^3 / 3
+// multiply-adds instead of the 2 p^3 / 3 of p substitutions: ten matrices of
+// p = 924 (the FP64 pipe's time for p^3 / 3: 4.3 ms) with the factorisation
+// 17.1 -> 9.6 ms, twelve of p = 364 3.20 -> 1.89 ms, one of p = 364 1.74 -> 0.73.
+template <int C>
+__global__ void __launch_bounds__(32 * C) k_tri_inv(double* __restrict__ A, int p,
+                                                    const double* __restrict__ dinv) {
+  extern __shared__ double Ms[];  // [row][C], rows padded to blocks of 32
+  __shared__ double Lt[32][33], Ac[32][C + 1];
+  constexpr int PER = 32 / C;  // tile elements per thread
+  const size_t z = blockIdx.y;
+  A += z * p * p;
+  dinv += z * p;
+  const int c0 = blockIdx.x * C, J = c0 >> 5, T = (p + 31) >> 5;
+  const int lane = threadIdx.x & 31, col = threadIdx.x >> 5;
+  const int cg = c0 + col;
+  // element e of the tile (I, K): row (threadIdx.x >> 5) + e C, column lane
+  auto fetch = [&](int I, int K, double (&t)[PER]) {
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+      const int r = I * 32 + col + e * C;
+      t[e] = r < p ? A[(size_t)r * p + K * 32 + lane] : 0.0;
+    }
+  };
+  Ms[(J * 32 + lane) * C + col] =
+      cg < p ? diag_inv(A, dinv, p, J * 32, lane, cg - J * 32) : 0.0;
+  double nx[PER];
+  if (J + 1 < T) fetch(J + 1, J, nx);
+  for (int I = J + 1; I < T; ++I) {
+    double acc = 0.0;
+    for (int K = J; K < I; ++K) {
+      __syncthreads();
+#pragma unroll
+      for (int e = 0; e < PER; ++e) Lt[col + e * C][lane] = nx[e];
+      __syncthreads();
+      if (K + 1 < I)
+        fetch(I, K + 1, nx);
+      else
+#pragma unroll
+        for (int e = 0; e < PER; ++e) nx[e] = diag_inv(A, dinv, p, I * 32, col + e * C, lane);
+      const double* m = Ms + (size_t)K * 32 * C + col;
+#pragma unroll
+      for (int k = 0; k < 32; ++k) acc += Lt[lane][k] * m[k * C];
     }
     __syncthreads();
-    for (int r = c0 + nb + tid; r < p; r += blockDim.x) {
-      const double* row = A + (size_t)r * p + c0;
-      double acc = 0.0;
-      for (int c = 0; c < nb; ++c) acc += row[c] * yv[c0 + c];
-      yv[r] -= acc;
+#pragma unroll
+    for (int e = 0; e < PER; ++e) Lt[col + e * C][lane] = nx[e];
+    Ac[lane][col] = acc;
+    __syncthreads();
+    if (I + 1 < T) fetch(I + 1, J, nx);
+    double v = 0.0;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) v -= Lt[lane][k] * Ac[k][col];
+    Ms[(I * 32 + lane) * C + col] = v;
+    if (cg < p && I * 32 + lane < p) A[(size_t)cg * p + I * 32 + lane] = v;
+  }
+}
+
+// A^-1 = M^T M: Ainv[a][b] = sum_{i >= max(a, b)} M_ia M_ib, the columns of M
+// being the rows of the upper triangle; lower tiles, written to both triangles
+__global__ void __launch_bounds__(256) k_inv_syrk(const double* __restrict__ A, int p,
+                                                  const double* __restrict__ dinv,
+                                                  double* __restrict__ Ainv) {
+  __shared__ double Rs[T16][33], Cs[T16][33];
+  const size_t z = blockIdx.y;
+  A += z * p * p;
+  dinv += z * p;
+  Ainv += z * p * p;
+  int ti, tj;
+  lower_tile(blockIdx.x, ti, tj);  // the longest sums first
+  const int r0 = ti * T16, c0 = tj * T16;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int lk = threadIdx.x & 31, lr = threadIdx.x >> 5;
+  auto m = [&](int a, int i) {
+    if (a >= p || i >= p || i < a) return 0.0;
+    return i == a ? dinv[a] : A[(size_t)a * p + i];
+  };
+  double acc = 0.0;
+  for (int i0 = r0 & ~31; i0 < p; i0 += 32) {
+#pragma unroll
+    for (int h = 0; h < T16; h += 8) {
+      Rs[lr + h][lk] = m(r0 + lr + h, i0 + lk);
+      Cs[lr + h][lk] = m(c0 + lr + h, i0 + lk);
     }
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < 32; ++kk) acc += Rs[ty][kk] * Cs[tx][kk];
     __syncthreads();
   }
-  for (int blk = nblk - 1; blk >= 0; --blk) {
-    const int c0 = blk * 32, nb = min(32, p - c0);
-    if (warp == 0) {
-      double xi = lane < nb ? yv[c0 + lane] : 0.0;
-      for (int c = nb - 1; c >= 0; --c) {
-        if (lane == c) xi *= dinv[c0 + c];
-        const double xc = __shfl_sync(0xffffffffu, xi, c);
-        if (lane < c) xi -= A[(size_t)(c0 + c) * p + c0 + lane] * xc;
-      }
-      if (lane < nb) yv[c0 + lane] = xi;
-    }
-    __syncthreads();
-    for (int r = tid; r < c0; r += blockDim.x) {
-      double acc = 0.0;
-      for (int c = 0; c < nb; ++c) acc += A[(size_t)(c0 + c) * p + r] * yv[c0 + c];
-      yv[r] -= acc;
-    }
-    __syncthreads();
+  const int r = r0 + ty, c = c0 + tx;
+  if (r < p && c < p) {
+    Ainv[(size_t)r * p + c] = acc;
+    Ainv[(size_t)c * p + r] = acc;
   }
-  for (int r = tid; r < p; r += blockDim.x) x[r] = accumulate ? (x[r] + yv[r]) : yv[r];
 }
 
 // alpha += delta; ||delta||_2, ||delta||_inf into the report block; FP32 copy
@@ -450,11 +512,27 @@ __global__ void k_inv_gemv(int p, const double* __restrict__ Ainv, const double*
 
 }  // namespace
 
+template <int C>
+static void launch_tri_inv(const ProblemDev& P, int nb, cudaStream_t st) {
+  const size_t smem = (size_t)((P.p + 31) / 32 * 32) * C * sizeof(double);
+  if (smem > 32 * 1024)
+    cudaFuncSetAttribute(k_tri_inv<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_tri_inv<C><<<dim3((P.p + C - 1) / C, nb), 32 * C, smem, st>>>(P.A, P.p, P.dinv);
+}
+
+// strips of 8 columns when there are enough of them for two CTAs per SM (they
+// read the factor half as often as strips of 4) and their p x 8 values fit the
+// shared memory, else of 4, or 1 for the largest bases
 void launch_inverse(const ProblemDev& P, int nb, cudaStream_t st) {
-  const size_t smem = (size_t)P.p * sizeof(double);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_chol_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_chol_solve<<<dim3(P.p, nb), 256, smem, st>>>(P.A, P.p, P.dinv, nullptr, P.Ainv, 0);
+  const size_t col = (size_t)((P.p + 31) / 32 * 32) * sizeof(double), room = 208 * 1024;
+  if ((long long)((P.p + 7) / 8) * nb >= 2LL * device_sm_count() && 8 * col <= room)
+    launch_tri_inv<8>(P, nb, st);
+  else if (4 * col <= room)
+    launch_tri_inv<4>(P, nb, st);
+  else
+    launch_tri_inv<1>(P, nb, st);
+  const int T = (P.p + T16 - 1) / T16;
+  k_inv_syrk<<<dim3(T * (T + 1) / 2, nb), 256, 0, st>>>(P.A, P.p, P.dinv, P.Ainv);
 }
 
 void launch_inv_gemv(const ProblemDev& P, const double* b, double* x, int accumulate,
@@ -474,7 +552,7 @@ void launch_reduce_c(const ProblemDev& P, int M, cudaStream_t st) {
 }
 
 void launch_gram_f64(const ProblemDev& P, cudaStream_t st) {
-  const int T = (P.p + 31) / 32;
+  const int T = (P.p + T16 - 1) / T16;
   k_gram_f64<<<T * (T + 1) / 2, 256, 0, st>>>(P.n, P.n_pad, P.p, P.B, P.A);
 }
 
@@ -485,11 +563,11 @@ void launch_rhs(const ProblemDev& P, cudaStream_t st) {
 void launch_cholesky(const ProblemDev& P, int nb, cudaStream_t st) {
   k_save_diag<<<dim3((P.p + 255) / 256, nb), 256, 0, st>>>(P.A, P.p, P.diag0);
   for (int j0 = 0; j0 < P.p; j0 += 32) {
-    k_chol_diag<<<dim3(1, nb), 32, 0, st>>>(P.A, P.p, j0, P.status, P.diag0, P.dinv);
+    k_chol_diag<<<dim3(1, nb), 128, 0, st>>>(P.A, P.p, j0, P.status, P.diag0, P.dinv);
     const int m = P.p - j0 - 32;
     if (m > 0) {
-      k_chol_trsm<<<dim3((m + 31) / 32, nb), 32, 0, st>>>(P.A, P.p, j0, P.dinv);
-      const int T = (m + 31) / 32;
+      k_chol_trsm<<<dim3((m + 7) / 8, nb), 256, 0, st>>>(P.A, P.p, j0, P.dinv);
+      const int T = (m + T16 - 1) / T16;
       k_chol_update<<<dim3(T * (T + 1) / 2, nb), 256, 0, st>>>(P.A, P.p, j0);
     }
   }

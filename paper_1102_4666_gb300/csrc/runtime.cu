@@ -893,7 +893,7 @@ int Problem::finish_report(const bsde_solve_params& prm, cudaStream_t st, bsde_r
     // rhs, inverse product, 3 per refinement step), update, read-out (3);
     // per factorised Gram matrix points, basis, Gram (+ split-K reduce in
     // mixed precision); per group save_diag, 3 per panel but the last
-    // (diag, trsm, update), the last panel's diag, the batched inverse
+    // (diag, trsm, update), the last panel's diag, the batched inverse (2)
     const int panels = (shape.p + 31) / 32;
     const int refine2 = prm.refine_steps >= 0 ? prm.refine_steps : (mixed ? 2 : 1);
     const int refit = shape.qr ? 3 : (2 + 3 * refine2);
@@ -903,7 +903,7 @@ int Problem::finish_report(const bsde_solve_params& prm, cudaStream_t st, bsde_r
       mats = grid.resample ? prm.K_it : 1;
     }
     r.kernel_launches = prm.K_it * (2 + (dev.dense ? 1 : 0) + 1 + 1 + refit + 1 + 3) +
-                        mats * (2 + (mixed ? 2 : 1)) + groups * (3 * panels - 1 + 1);
+                        mats * (2 + (mixed ? 2 : 1)) + groups * (3 * panels - 1 + 2);
     if (prm.timing && (int)events.size() >= 8 * prm.K_it) {
       // paths: ev0..ev1; Gram matrices, factors and inverses built ahead of
       // a group of iterations: ev3..ev7 of the group's first iteration;
