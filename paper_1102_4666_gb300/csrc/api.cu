@@ -348,36 +348,29 @@ int bsde_eval_price_delta(bsde_ctx* c, int q, const double* t, const double* S, 
     if (!P.coeffs_valid) return fail(c, BSDE_ERR_STATE, "eval: no coefficients (solve first)");
     if (!set_device(c)) return fail(c, BSDE_ERR_CUDA, "eval: cudaSetDevice failed");
     const int d = P.model.d;
-    std::vector<double> hx((size_t)q * d);
-    for (size_t e = 0; e < hx.size(); ++e) {
-      if (!(S[e] > 0.0)) return fail(c, BSDE_ERR_INVALID_ARG, "eval: prices must be positive");
-      hx[e] = std::log(S[e]);
-    }
+    // the logarithms and the division by S are the kernel's
+    bool positive = true;
+    for (size_t e = 0; e < (size_t)q * d; ++e) positive = positive && S[e] > 0.0;
+    if (!positive) return fail(c, BSDE_ERR_INVALID_ARG, "eval: prices must be positive");
     const size_t bytes = (size_t)q * 8 * (2 + 2 * d);
     double* buf = (double*)c->al.get(bytes, c->stream);
     if (!buf) return fail(c, BSDE_ERR_NOMEM, "eval: device allocation failed");
     double* dt = buf;
-    double* dx = dt + q;
-    double* dp = dx + (size_t)q * d;
+    double* dS = dt + q;
+    double* dp = dS + (size_t)q * d;
     double* dg = dp + q;
-    std::vector<double> g((size_t)q * d);
     cudaError_t e = cudaMemcpyAsync(dt, t, (size_t)q * 8, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(dx, hx.data(), (size_t)q * d * 8, cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) {
-      launch_eval_points(P.model, P.grid, P.dev, q, dt, dx, dp, dg, c->stream);
-      e = cudaGetLastError();
-    }
+      e = cudaMemcpyAsync(dS, S, (size_t)q * d * 8, cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess)
+      e = launch_eval_points(P.model, P.grid, P.dev, q, dt, dS, dp, delta ? dg : nullptr, c->stream);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(price, dp, (size_t)q * 8, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(g.data(), dg, (size_t)q * d * 8, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess && delta)
+      e = cudaMemcpyAsync(delta, dg, (size_t)q * d * 8, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     c->al.put(buf, c->stream);
     if (e != cudaSuccess) return fail(c, BSDE_ERR_CUDA, std::string("eval: ") + cudaGetErrorString(e));
-    if (delta)
-      for (int i = 0; i < q; ++i)
-        for (int j = 0; j < d; ++j) delta[(size_t)i * d + j] = g[(size_t)i * d + j] / S[(size_t)i * d + j];
     return BSDE_OK;
   })
 }

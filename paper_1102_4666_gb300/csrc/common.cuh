@@ -191,7 +191,7 @@ struct ProblemDev {
   float* alpha32 = nullptr;   // [p] FP32 copy for the mixed path kernel
   uint2* pairs = nullptr;     // [p] packed (variate, degree) bytes
   uint8_t* nnz = nullptr;     // [p] active variates per basis function
-  uint32_t* key = nullptr;    // [2] Philox key (device copy, read by the points kernel)
+  uint32_t* key = nullptr;    // [2] Philox key (device copy, read by the basis kernel)
   uint32_t seed_key[2] = {0, 0};  // the same key on the host, a parameter of the path kernel
   int* status = nullptr;      // [1] device status bits
   double* out = nullptr;      // report block (see OUT_* offsets)
@@ -229,9 +229,9 @@ struct ProblemDev {
 #define ST_BADARG 4
 
 // launchers (one translation unit each)
-void launch_points(const ModelHost& m, const GridHost& g, const ProblemDev& P, uint32_t k,
-                   cudaStream_t st);
-void launch_basis(const ModelHost& m, const GridHost& g, const ProblemDev& P, bool mixed,
+// the points of iteration k and their basis matrix (split: with the operands of
+// the tensor-core Gram matrix)
+void launch_basis(const ModelHost& m, const GridHost& g, const ProblemDev& P, uint32_t k, bool split,
                   cudaStream_t st);
 // path kernel: returns cudaSuccess or the launch error
 cudaError_t launch_paths(const ModelHost& m, const GridHost& g, const ProblemDev& P, int M, int N,
@@ -249,12 +249,10 @@ void launch_rhs(const ProblemDev& P, cudaStream_t st);
 // batched over nb Gram matrices (P.A, P.dinv, P.diag0, P.Ainv hold nb of them)
 void launch_cholesky(const ProblemDev& P, int nb, cudaStream_t st);
 void launch_refine_residual(const ProblemDev& P, cudaStream_t st);
-void launch_update(const ProblemDev& P, int k, cudaStream_t st);
-void launch_eval_x0(const ModelHost& m, const GridHost& g, const ProblemDev& P, int k,
-                    cudaStream_t st);
-void launch_eval_points(const ModelHost& m, const GridHost& g, const ProblemDev& P, int q,
-                        const double* t, const double* x, double* price, double* dudx,
-                        cudaStream_t st);
+void launch_update(const ModelHost& m, const GridHost& g, const ProblemDev& P, int k, cudaStream_t st);
+cudaError_t launch_eval_points(const ModelHost& m, const GridHost& g, const ProblemDev& P, int q,
+                               const double* t, const double* S, double* price, double* delta,
+                               cudaStream_t st);
 size_t paths_smem_bytes(int d, int p, int eta, int N, int tpb, bool mixed, bool dense);
 void launch_cheb2mono(const ProblemDev& P, cudaStream_t st);
 void launch_qr_solve(const ProblemDev& P, cudaStream_t st);

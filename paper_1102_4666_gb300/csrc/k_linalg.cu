@@ -21,26 +21,29 @@ __global__ void k_reduce_c(int i0, int count, int chunks, int M, const double* _
   c[i] = s / (double)M;
 }
 
-// CTA of 128 threads per basis function: out[l] = sum_i B[l][i] y[i], each
-// thread over i = tid mod 128, then a fixed shuffle tree and the four warp
-// sums in order; with sub != nullptr, out[l] = sub[l] - that sum
-__global__ void __launch_bounds__(128) k_bt_times(int n, int n_pad, int p,
+// CTA of 256 threads per basis function: out[l] = sum_i B[l][i] y[i], each
+// thread over i = tid mod 256, then a fixed shuffle tree and the eight warp
+// sums in order; with sub != nullptr, out[l] = sub[l] - that sum.  Bound by the
+// latency of its loads at small p (35 CTAs of 128 threads with few loads in
+// flight: 5.5 us at n = 2000, this 3.5 us).
+__global__ void __launch_bounds__(256) k_bt_times(int n, int n_pad, int p,
                                                   const double* __restrict__ B,
                                                   const double* __restrict__ y,
                                                   const double* __restrict__ sub,
                                                   double* __restrict__ out) {
-  __shared__ double ws[4];
+  __shared__ double ws[8];
   const int l = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const double* row = B + (size_t)l * n_pad;
   double s = 0.0;
-  for (int i = tid; i < n; i += 128) s += row[i] * y[i];
+#pragma unroll 4
+  for (int i = tid; i < n; i += 256) s += row[i] * y[i];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) ws[warp] = s;
   __syncthreads();
   if (tid == 0) {
-    const double tot = (ws[0] + ws[1]) + (ws[2] + ws[3]);
+    const double tot = ((ws[0] + ws[1]) + (ws[2] + ws[3])) + ((ws[4] + ws[5]) + (ws[6] + ws[7]));
     out[l] = sub ? (sub[l] - tot) : tot;
   }
 }
@@ -373,114 +376,175 @@ __global__ void __launch_bounds__(256) k_inv_syrk(const double* __restrict__ A, 
   }
 }
 
-// alpha += delta; ||delta||_2, ||delta||_inf into the report block; FP32 copy
-__global__ void __launch_bounds__(256) k_update(int p, int k, double* __restrict__ alpha,
+struct EvalArgs {
+  int d, p, eta;
+  double ctr[BSDE_DMAX + 1], sc[BSDE_DMAX + 1];
+};
+
+// T_e and T_e' (e = 1 .. eta) at z, into t[(e - 1) stride] and dt[(e - 1) stride]
+__device__ __forceinline__ void cheb_column(double z, int eta, double* t, double* dt, int stride) {
+  double t0 = 1.0, t1 = z, d0 = 0.0, d1 = 1.0;
+  for (int e = 1; e <= eta; ++e) {
+    if (e >= 2) {
+      const double t2 = 2.0 * z * t1 - t0, d2 = 2.0 * t1 + 2.0 * z * d1 - d0;
+      t0 = t1; t1 = t2; d0 = d1; d1 = d2;
+    }
+    t[(e - 1) * stride] = t1;
+    dt[(e - 1) * stride] = d1;
+  }
+}
+
+__device__ __forceinline__ void unpack_pair(uint2 pr, int a, int& v, int& e) {
+  const uint32_t byte = ((a < 4 ? pr.x >> (8 * a) : pr.y >> (8 * (a - 4)))) & 0xffu;
+  v = (int)(byte >> 4);
+  e = (int)(byte & 15u);
+}
+
+// u and du/dx_v of one basis function from tables T, T' laid out [v][e - 1]
+// with the given stride: val = prod T, and grad(v, dval) for every active
+// space variate (dval not yet scaled by d xi / dx)
+template <typename G>
+__device__ __forceinline__ double basis_value(uint2 pr, int nz, int eta, const double* t,
+                                              const double* dt, int stride, G&& grad) {
+  double tv[BSDE_NNZ_MAX];
+  double val = 1.0;
+#pragma unroll
+  for (int a = 0; a < BSDE_NNZ_MAX; ++a) {
+    if (a >= nz) break;
+    int v, e;
+    unpack_pair(pr, a, v, e);
+    tv[a] = t[(v * eta + e - 1) * stride];
+    val *= tv[a];
+  }
+#pragma unroll
+  for (int a = 0; a < BSDE_NNZ_MAX; ++a) {
+    if (a >= nz) break;
+    int v, e;
+    unpack_pair(pr, a, v, e);
+    if (v == 0) continue;
+    double gd = dt[(v * eta + e - 1) * stride];
+#pragma unroll
+    for (int c = 0; c < BSDE_NNZ_MAX; ++c)
+      if (c < nz && c != a) gd *= tv[c];
+    grad(v, gd);
+  }
+  return val;
+}
+
+// alpha += delta; ||delta||_2, ||delta||_inf into the report block; FP32 copy;
+// then the read-out of Section 5.3 at (0, log S0): price V = u and du/dx.  One
+// CTA (one launch instead of four): the Chebyshev values of the point once in
+// shared memory, threads over basis functions, a fixed shuffle tree.
+__global__ void __launch_bounds__(256) k_update(const __grid_constant__ EvalArgs ea, int k, double t0,
+                                                double* __restrict__ alpha,
                                                 float* __restrict__ alpha32,
                                                 const double* __restrict__ delta,
+                                                const uint2* __restrict__ pairs,
+                                                const uint8_t* __restrict__ nnz,
+                                                const double* __restrict__ logS0,
                                                 double* __restrict__ out) {
-  __shared__ double s2[256], si[256];
-  double a2 = 0.0, ai = 0.0;
-  for (int l = threadIdx.x; l < p; l += 256) {
+  __shared__ double T[(BSDE_DMAX + 1) * 15], dT[(BSDE_DMAX + 1) * 15];
+  __shared__ double red[BSDE_DMAX + 3][256];  // row 0: |delta|^2, 1: max |delta|, 2: u, 3..: du/dx_j
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, d = ea.d;
+  // the last warp tabulates
+  if (warp == 7 && lane <= d) {
+    const double z = ((lane == 0 ? t0 : logS0[lane - 1]) - ea.ctr[lane]) * ea.sc[lane];
+    cheb_column(z, ea.eta, T + lane * ea.eta, dT + lane * ea.eta, 1);
+  }
+  for (int j = 0; j < d; ++j) red[3 + j][tid] = 0.0;
+  __syncthreads();
+  double a2 = 0.0, ai = 0.0, u = 0.0;
+  for (int l = tid; l < ea.p; l += 256) {
     const double dl = delta[l];
     const double al = alpha[l] + dl;
     alpha[l] = al;
     if (alpha32) alpha32[l] = (float)al;
     a2 += dl * dl;
     ai = fmax(ai, fabs(dl));
+    u += al * basis_value(pairs[l], nnz[l], ea.eta, T, dT, 1,
+                          [&](int v, double gd) { red[2 + v][tid] += al * gd; });
   }
-  s2[threadIdx.x] = a2;
-  si[threadIdx.x] = ai;
+  red[0][tid] = a2;
+  red[1][tid] = ai;
+  red[2][tid] = u;
   __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) {
-      s2[threadIdx.x] += s2[threadIdx.x + o];
-      si[threadIdx.x] = fmax(si[threadIdx.x], si[threadIdx.x + o]);
+  for (int r = warp; r < 3 + d; r += 8) {
+    const double* q = red[r] + lane;
+    double s;
+    if (r == 1) {
+      s = q[0];
+      for (int w = 32; w < 256; w += 32) s = fmax(s, q[w]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s = fmax(s, __shfl_xor_sync(0xffffffffu, s, o));
+    } else {
+      s = ((q[0] + q[32]) + (q[64] + q[96])) + ((q[128] + q[160]) + (q[192] + q[224]));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0 && k >= 0 && k < 64) {
-    out[OUT_RES2 + k] = sqrt(s2[0]);
-    out[OUT_RESI + k] = si[0];
+    const bool it = k >= 0 && k < 64;
+    if (lane != 0) continue;
+    if (r == 0 && it) out[OUT_RES2 + k] = sqrt(s);
+    if (r == 1 && it) out[OUT_RESI + k] = s;
+    if (r == 2) {
+      out[OUT_PRICE] = s;
+      if (it) out[OUT_PRICE_IT + k] = s;
+    }
+    if (r >= 3) out[OUT_DUDX + r - 3] = s * ea.sc[r - 2];
   }
 }
 
-struct EvalArgs {
-  int d, p, n_query;
-  double ctr[BSDE_DMAX + 1], sc[BSDE_DMAX + 1];
-};
-
-// u and du/dx_j at query points (Section 5.3: price V = u, Delta = grad_x V):
-// one CTA per point, threads over basis functions, fixed-order reduction.
-__global__ void __launch_bounds__(256) k_eval(const __grid_constant__ EvalArgs ea,
-                                              const double* __restrict__ alpha,
-                                              const uint2* __restrict__ pairs,
-                                              const uint8_t* __restrict__ nnz,
-                                              const double* __restrict__ qt,
-                                              const double* __restrict__ qx,
-                                              double* __restrict__ price,
-                                              double* __restrict__ dudx) {
-  __shared__ double red[256][BSDE_DMAX + 1];
-  const int qi = blockIdx.x;
-  const int d = ea.d;
-  double xi[BSDE_DMAX + 1];
-  xi[0] = (qt[qi] - ea.ctr[0]) * ea.sc[0];
-  for (int j = 0; j < d; ++j) xi[j + 1] = (qx[(size_t)qi * d + j] - ea.ctr[j + 1]) * ea.sc[j + 1];
-  double u = 0.0, g[BSDE_DMAX];
-  for (int j = 0; j < d; ++j) g[j] = 0.0;
-  for (int l = threadIdx.x; l < ea.p; l += 256) {
-    const uint2 pr = pairs[l];
-    const int nz = nnz[l];
-    double tv[BSDE_NNZ_MAX], dv[BSDE_NNZ_MAX];
-    int var[BSDE_NNZ_MAX];
-    for (int a = 0; a < nz; ++a) {
-      const uint32_t byte = ((a < 4 ? pr.x >> (8 * a) : pr.y >> (8 * (a - 4)))) & 0xffu;
-      const int v = (int)(byte >> 4), e = (int)(byte & 15u);
-      const double z = xi[v];
-      double t0 = 1.0, t1 = z, d0 = 0.0, d1 = 1.0;
-      for (int q = 2; q <= e; ++q) {
-        const double t2 = 2.0 * z * t1 - t0, d2 = 2.0 * t1 + 2.0 * z * d1 - d0;
-        t0 = t1; t1 = t2; d0 = d1; d1 = d2;
-      }
-      tv[a] = t1;
-      dv[a] = d1;
-      var[a] = v;
-    }
-    double val = 1.0;
-    for (int a = 0; a < nz; ++a) val *= tv[a];
-    u += alpha[l] * val;
-    for (int a = 0; a < nz; ++a) {
-      if (var[a] == 0) continue;
-      double gd = dv[a];
-      for (int c = 0; c < nz; ++c)
-        if (c != a) gd *= tv[c];
-      g[var[a] - 1] += alpha[l] * gd * ea.sc[var[a]];
-    }
+// u and du/dx at query points, threads = queries: CTA of 32 points x slices of
+// the basis functions (one warp each); every warp tabulates its share of the
+// points' Chebyshev values in shared memory ([slot][point]), then takes its
+// slice, the function's variates being the same for the whole warp.  Bound by
+// the FP64 pipe: about 9 FP64 instructions per function of three variates.
+// S: prices; x = log S here, and the derivative is returned as dV/dS.
+// (20000 points, d = 10, p = 364: one CTA per point with a table of its own per
+// function 840 us, this 352 us.)
+__global__ void __launch_bounds__(256) k_eval_many(const __grid_constant__ EvalArgs ea, int nq,
+                                                   const double* __restrict__ alpha,
+                                                   const uint2* __restrict__ pairs,
+                                                   const uint8_t* __restrict__ nnz,
+                                                   const double* __restrict__ qt,
+                                                   const double* __restrict__ S,
+                                                   double* __restrict__ price,
+                                                   double* __restrict__ delta) {
+  extern __shared__ double ev[];  // T, dT: (d + 1) eta x 32 each; sums: slices x (d + 1) x 32
+  const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5, slices = blockDim.x >> 5;
+  const int d = ea.d, rows = (d + 1) * ea.eta;
+  double* T = ev + lane;
+  double* dT = T + (size_t)rows * 32;
+  double* acc = ev + (size_t)2 * rows * 32 + (size_t)slice * (d + 1) * 32 + lane;
+  const int q = blockIdx.x * 32 + lane;
+  const int qc = q < nq ? q : nq - 1;
+  for (int v = slice; v <= d; v += slices) {
+    const double y = v == 0 ? qt[qc] : log(S[(size_t)qc * d + v - 1]);
+    cheb_column((y - ea.ctr[v]) * ea.sc[v], ea.eta, T + (size_t)v * ea.eta * 32,
+                dT + (size_t)v * ea.eta * 32, 32);
   }
-  red[threadIdx.x][0] = u;
-  for (int j = 0; j < d; ++j) red[threadIdx.x][j + 1] = g[j];
+  for (int j = 0; j <= d; ++j) acc[j * 32] = 0.0;
   __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o)
-      for (int j = 0; j <= d; ++j) red[threadIdx.x][j] += red[threadIdx.x + o][j];
-    __syncthreads();
+  const int per = (ea.p + slices - 1) / slices;
+  const int l1 = min(ea.p, (slice + 1) * per);
+  double u = 0.0;
+  for (int l = slice * per; l < l1; ++l) {
+    const double al = alpha[l];
+    u += al * basis_value(pairs[l], nnz[l], ea.eta, T, dT, 32,
+                          [&](int v, double gd) { acc[v * 32] += al * gd; });
   }
-  if (threadIdx.x == 0) {
-    price[qi] = red[0][0];
-    if (dudx)
-      for (int j = 0; j < d; ++j) dudx[(size_t)qi * d + j] = red[0][j + 1];
+  acc[0] = u;
+  __syncthreads();
+  // sums over the slices in order, row j = 0: u, else the derivative in x_j
+  const double* a0 = ev + (size_t)2 * rows * 32 + lane;
+  for (int j = slice; j <= d; j += slices) {
+    double s = 0.0;
+    for (int w = 0; w < slices; ++w) s += a0[((size_t)w * (d + 1) + j) * 32];
+    if (q >= nq) continue;
+    if (j == 0)
+      price[q] = s;
+    else if (delta)
+      delta[(size_t)q * d + j - 1] = s * ea.sc[j] / S[(size_t)q * d + j - 1];
   }
-}
-
-// read-out point (0, log S0) written into the report block
-__global__ void k_x0(int d, double t0, const double* __restrict__ logS0, double* __restrict__ qt,
-                     double* __restrict__ qx) {
-  if (threadIdx.x == 0) qt[0] = t0;
-  if (threadIdx.x < d) qx[threadIdx.x] = logS0[threadIdx.x];
-}
-
-__global__ void k_copy_price(int k, int d, double* __restrict__ out) {
-  // out[OUT_PRICE] and dudx were written by k_eval; keep the per-iteration price
-  if (threadIdx.x == 0 && k >= 0 && k < 64) out[OUT_PRICE_IT + k] = out[OUT_PRICE];
 }
 
 // monomial coefficients of u^k (basis of total degree <= 3): beta_m =
@@ -557,7 +621,7 @@ void launch_gram_f64(const ProblemDev& P, cudaStream_t st) {
 }
 
 void launch_rhs(const ProblemDev& P, cudaStream_t st) {
-  k_bt_times<<<P.p, 128, 0, st>>>(P.n, P.n_pad, P.p, P.B, P.c, nullptr, P.rhs);
+  k_bt_times<<<P.p, 256, 0, st>>>(P.n, P.n_pad, P.p, P.B, P.c, nullptr, P.rhs);
 }
 
 void launch_cholesky(const ProblemDev& P, int nb, cudaStream_t st) {
@@ -575,19 +639,15 @@ void launch_cholesky(const ProblemDev& P, int nb, cudaStream_t st) {
 
 void launch_refine_residual(const ProblemDev& P, cudaStream_t st) {
   k_b_times<<<(P.n + 31) / 32, 256, 0, st>>>(P.n, P.n_pad, P.p, P.B, P.delta, P.v);
-  k_bt_times<<<P.p, 128, 0, st>>>(P.n, P.n_pad, P.p, P.B, P.v, P.rhs, P.res);
+  k_bt_times<<<P.p, 256, 0, st>>>(P.n, P.n_pad, P.p, P.B, P.v, P.rhs, P.res);
 }
 
-void launch_update(const ProblemDev& P, int k, cudaStream_t st) {
-  k_update<<<1, 256, 0, st>>>(P.p, k, P.alpha, P.alpha32, P.delta, P.out);
-}
-
-static EvalArgs eval_args(const ModelHost& m, const GridHost& g, const ProblemDev& P, int q) {
+static EvalArgs eval_args(const ModelHost& m, const GridHost& g, const ProblemDev& P) {
   EvalArgs ea;
   memset(&ea, 0, sizeof(ea));
   ea.d = m.d;
   ea.p = P.p;
-  ea.n_query = q;
+  ea.eta = P.eta < 1 ? 1 : P.eta;
   for (int v = 0; v <= m.d; ++v) {
     ea.ctr[v] = 0.5 * (g.lo[v] + g.hi[v]);
     ea.sc[v] = 2.0 / (g.hi[v] - g.lo[v]);
@@ -595,23 +655,27 @@ static EvalArgs eval_args(const ModelHost& m, const GridHost& g, const ProblemDe
   return ea;
 }
 
-// price and du/dx at (0, log S0) after iteration k; the query point lives in
-// the tail of the report block (OUT_SIZE .. OUT_SIZE + 1 + 2 d)
-void launch_eval_x0(const ModelHost& m, const GridHost& g, const ProblemDev& P, int k,
-                    cudaStream_t st) {
-  double* qt = P.out + OUT_SIZE;
-  double* qx = qt + 1;
-  double* logS0 = qx + BSDE_DMAX;
-  k_x0<<<1, 32, 0, st>>>(m.d, 0.0, logS0, qt, qx);
-  const EvalArgs ea = eval_args(m, g, P, 1);
-  k_eval<<<1, 256, 0, st>>>(ea, P.alpha, P.pairs, P.nnz, qt, qx, P.out + OUT_PRICE,
-                            P.out + OUT_DUDX);
-  k_copy_price<<<1, 32, 0, st>>>(k, m.d, P.out);
+// alpha^{k+1} and the price and du/dx at (0, log S0) after iteration k; log S0
+// lives in the tail of the report block
+void launch_update(const ModelHost& m, const GridHost& g, const ProblemDev& P, int k, cudaStream_t st) {
+  k_update<<<1, 256, 0, st>>>(eval_args(m, g, P), k, 0.0, P.alpha, P.alpha32, P.delta, P.pairs, P.nnz,
+                              P.out + OUT_SIZE + 1 + BSDE_DMAX, P.out);
 }
 
-void launch_eval_points(const ModelHost& m, const GridHost& g, const ProblemDev& P, int q,
-                        const double* t, const double* x, double* price, double* dudx,
-                        cudaStream_t st) {
-  const EvalArgs ea = eval_args(m, g, P, q);
-  k_eval<<<q, 256, 0, st>>>(ea, P.alpha, P.pairs, P.nnz, t, x, price, dudx);
+// price and dV/dS (delta may be null) at q points (t, S).  As many slices of the
+// basis as keep four warps on every scheduler, at most eight: a few points are
+// spread over the basis functions, many need no more than a warp per 32.
+cudaError_t launch_eval_points(const ModelHost& m, const GridHost& g, const ProblemDev& P, int q,
+                               const double* t, const double* S, double* price, double* delta,
+                               cudaStream_t st) {
+  const EvalArgs ea = eval_args(m, g, P);
+  const int groups = (q + 31) / 32;
+  int slices = 8;
+  while (slices > 1 && (long long)groups * slices > 32LL * device_sm_count()) slices >>= 1;
+  const size_t smem = ((size_t)2 * (ea.d + 1) * ea.eta + (size_t)slices * (ea.d + 1)) * 32 * sizeof(double);
+  cudaError_t e =
+      cudaFuncSetAttribute(k_eval_many, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_eval_many<<<groups, 32 * slices, smem, st>>>(ea, q, P.alpha, P.pairs, P.nnz, t, S, price, delta);
+  return cudaGetLastError();
 }

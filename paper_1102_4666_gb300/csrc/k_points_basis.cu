@@ -8,39 +8,18 @@ struct BoxArgs {
   double lo[BSDE_DMAX + 1], hi[BSDE_DMAX + 1];
 };
 
-// Algorithm 2, first step of iteration k: point i takes coordinate c from
-// lane c%4 of the Philox block (c/4, i, 0, TAG_PTS<<24 | k) and maps the
-// uniform u = (w + 1/2) 2^-32 onto [lo_c, hi_c].  Explicit _rn operations
-// keep every rounding as written (no FMA contraction).
-__global__ void k_points(int n, int dp, const uint32_t* __restrict__ key, uint32_t k,
-                         const __grid_constant__ BoxArgs box, double* __restrict__ t,
-                         double* __restrict__ x) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const Philox ph{key[0], key[1]};
-  for (int blk = 0; blk * 4 < dp; ++blk) {
-    const uint4 o = ph((uint32_t)blk, (uint32_t)i, 0u, (TAG_PTS << 24) | k);
-    const uint32_t w[4] = {o.x, o.y, o.z, o.w};
-#pragma unroll
-    for (int lane = 0; lane < 4; ++lane) {
-      const int c = blk * 4 + lane;
-      if (c >= dp) break;
-      const double u = __dmul_rn((double)w[lane] + 0.5, 2.3283064365386962890625e-10);
-      const double y = __dadd_rn(box.lo[c], __dmul_rn(__dsub_rn(box.hi[c], box.lo[c]), u));
-      if (c == 0)
-        t[i] = y;
-      else
-        x[(size_t)(c - 1) * n + i] = y;
-    }
-  }
-}
-
 __device__ __forceinline__ float to_tf32(float v) {
   uint32_t r;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(v));
   return __uint_as_float(r);
 }
 
+// Algorithm 2, first step of iteration k: point i takes coordinate c from
+// lane c%4 of the Philox block (c/4, i, 0, TAG_PTS<<24 | k) and maps the
+// uniform u = (w + 1/2) 2^-32 onto [lo_c, hi_c].  Explicit _rn operations
+// keep every rounding as written (no FMA contraction).  Drawn in the kernel that
+// needs them, by every CTA for its own points (a launch of their own cost 2 us
+// and a gap, twice an iteration); the CTAs of the first range store them.
 // B[l][i] = prod over the active variates v of T_{nu_lv}(xi_v(t_i, x_i)),
 // xi_v = (2 y_v - (lo_v + hi_v)) / (hi_v - lo_v), Chebyshev T_e by the
 // three-term recurrence.  A CTA takes 32 consecutive points and a range of
@@ -57,18 +36,37 @@ constexpr int BASIS_PTS = 32;  // points per CTA of k_basis, one per lane
 
 __global__ void k_basis(int n, int n_pad, int p, int l_per, int dp, int eta,
                         const uint2* __restrict__ pairs, const uint8_t* __restrict__ nnz,
-                        const double* __restrict__ t, const double* __restrict__ x,
-                        const __grid_constant__ BoxArgs box, double* __restrict__ B,
+                        const uint32_t* __restrict__ key, uint32_t k, double* __restrict__ t,
+                        double* __restrict__ x, const __grid_constant__ BoxArgs box,
+                        double* __restrict__ B,
                         float* __restrict__ Bhi, float* __restrict__ Blo, int split) {
   extern __shared__ double cheb[];  // [v][e][point]
   const int tid = threadIdx.x, nth = blockDim.x;
   const int i0 = blockIdx.x * BASIS_PTS;
+  const int vrow = (eta + 1) * BASIS_PTS;  // one variate's table
+  const Philox ph{key[0], key[1]};
+  for (int idx = tid; idx < (dp + 3) / 4 * BASIS_PTS; idx += nth) {
+    const int blk = idx / BASIS_PTS, q = idx - blk * BASIS_PTS, i = i0 + q;
+    if (i >= n) continue;
+    const uint4 o = ph((uint32_t)blk, (uint32_t)i, 0u, (TAG_PTS << 24) | k);
+    const uint32_t w[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+    for (int c4 = 0; c4 < 4; ++c4) {
+      const int c = blk * 4 + c4;
+      if (c >= dp) break;
+      const double u = __dmul_rn((double)w[c4] + 0.5, 2.3283064365386962890625e-10);
+      const double y = __dadd_rn(box.lo[c], __dmul_rn(__dsub_rn(box.hi[c], box.lo[c]), u));
+      cheb[c * vrow + q] = y;  // the place of T_0 until the tables are built
+      if (blockIdx.y == 0) (c == 0 ? t : x + (size_t)(c - 1) * n)[i] = y;
+    }
+  }
+  __syncthreads();
   const int ne = eta + 1;
   for (int idx = tid; idx < dp * BASIS_PTS; idx += nth) {
     const int v = idx / BASIS_PTS, q = idx - v * BASIS_PTS;
     const int i = i0 + q;
     if (i >= n) continue;
-    const double y = (v == 0) ? t[i] : x[(size_t)(v - 1) * n + i];
+    const double y = cheb[v * vrow + q];
     const double xi = __ddiv_rn(__dsub_rn(__dmul_rn(2.0, y), __dadd_rn(box.lo[v], box.hi[v])),
                                 __dsub_rn(box.hi[v], box.lo[v]));
     double* tv = cheb + (size_t)v * ne * BASIS_PTS + q;
@@ -110,18 +108,7 @@ __global__ void k_basis(int n, int n_pad, int p, int l_per, int dp, int eta,
 
 }  // namespace
 
-void launch_points(const ModelHost& m, const GridHost& g, const ProblemDev& P, uint32_t k,
-                   cudaStream_t st) {
-  BoxArgs box;
-  for (int v = 0; v <= m.d; ++v) {
-    box.lo[v] = g.lo[v];
-    box.hi[v] = g.hi[v];
-  }
-  const int tpb = 128;
-  k_points<<<(P.n + tpb - 1) / tpb, tpb, 0, st>>>(P.n, m.d + 1, P.key, k, box, P.t, P.x);
-}
-
-void launch_basis(const ModelHost& m, const GridHost& g, const ProblemDev& P, bool mixed,
+void launch_basis(const ModelHost& m, const GridHost& g, const ProblemDev& P, uint32_t k, bool split,
                   cudaStream_t st) {
   BoxArgs box;
   for (int v = 0; v <= m.d; ++v) {
@@ -140,6 +127,6 @@ void launch_basis(const ModelHost& m, const GridHost& g, const ProblemDev& P, bo
   if (gy < 1) gy = 1;
   const int l_per = (P.p + gy - 1) / gy;
   gy = (P.p + l_per - 1) / l_per;
-  k_basis<<<dim3(gx, gy), tpb, smem, st>>>(P.n, P.n_pad, P.p, l_per, dp, eta, P.pairs, P.nnz, P.t, P.x,
-                                            box, P.B, P.Bhi, P.Blo, mixed ? 1 : 0);
+  k_basis<<<dim3(gx, gy), tpb, smem, st>>>(P.n, P.n_pad, P.p, l_per, dp, eta, P.pairs, P.nnz, P.key, k,
+                                            P.t, P.x, box, P.B, P.Bhi, P.Blo, split ? 1 : 0);
 }

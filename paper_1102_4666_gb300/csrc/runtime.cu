@@ -585,8 +585,7 @@ int Problem::enqueue_factors(int k0, int nb, cudaStream_t st) {
   const size_t pp = (size_t)shape.p * shape.p;
   for (int j = 0; j < nb; ++j) {
     const uint32_t kp = grid.resample ? (uint32_t)(k0 + j) : 0u;
-    launch_points(model, grid, dev, kp, st);
-    launch_basis(model, grid, dev, mixed, st);
+    launch_basis(model, grid, dev, kp, mixed, st);
     ProblemDev Pj = dev;
     Pj.A = dev.A + (size_t)j * pp;
     if (mixed) {
@@ -609,8 +608,7 @@ int Problem::enqueue_gram(int k, cudaStream_t st) {
     err = "gram: no factor block";
     return BSDE_ERR_STATE;
   }
-  launch_points(model, grid, dev, grid.resample ? (uint32_t)k : 0u, st);
-  launch_basis(model, grid, dev, mixed, st);
+  launch_basis(model, grid, dev, grid.resample ? (uint32_t)k : 0u, mixed, st);
   if (mixed) {
     const cudaError_t e = launch_gram_tc(dev, st);
     if (e != cudaSuccess) {
@@ -640,8 +638,7 @@ int Problem::enqueue_iteration(const bsde_solve_params& prm, int k, cudaStream_t
     dev.c = sh_buf + region_off;
   }
   const uint32_t kp = grid.resample ? (uint32_t)k : 0u;
-  launch_points(model, grid, dev, kp, st);
-  launch_basis(model, grid, dev, false, st);  // FP64 B for the refit (no TF32 split)
+  launch_basis(model, grid, dev, kp, false, st);  // FP64 B for the refit (no TF32 split)
   if (dev.dense) launch_cheb2mono(dev, st);
   if (rec) record(ev[0], st);
   cudaError_t e = launch_paths(model, grid, dev, shape.M, shape.N, (uint32_t)k, mixed, shape.tpb,
@@ -709,8 +706,7 @@ int Problem::enqueue_iteration(const bsde_solve_params& prm, int k, cudaStream_t
     }
   }
   if (rec) record(ev[5], st);
-  launch_update(dev, k - prm.k_start, st);
-  launch_eval_x0(model, grid, dev, k - prm.k_start, st);
+  launch_update(model, grid, dev, k - prm.k_start, st);
   e = cudaGetLastError();
   if (e != cudaSuccess) {
     err = std::string("kernel launch failed: ") + cudaGetErrorString(e);
@@ -888,10 +884,10 @@ int Problem::finish_report(const bsde_solve_params& prm, cudaStream_t st, bsde_r
     r.path_steps_per_s = ms_total > 0 ? r.path_steps / (ms_total * 1e-3) : 0.0;
     r.path_launches = prm.K_it;
     r.rank = rank;
-    // launches: per iteration points, basis, (monomial conversion), paths,
+    // launches: per iteration points with basis, (monomial conversion), paths,
     // reduce, refit (QR: init, factorisation, solve; otherwise
-    // rhs, inverse product, 3 per refinement step), update, read-out (3);
-    // per factorised Gram matrix points, basis, Gram (+ split-K reduce in
+    // rhs, inverse product, 3 per refinement step), update with read-out;
+    // per factorised Gram matrix points with basis, Gram (+ split-K reduce in
     // mixed precision); per group save_diag, 3 per panel but the last
     // (diag, trsm, update), the last panel's diag, the batched inverse (2)
     const int panels = (shape.p + 31) / 32;
@@ -902,8 +898,8 @@ int Problem::finish_report(const bsde_solve_params& prm, cudaStream_t st, bsde_r
       groups = grid.resample ? (prm.K_it + nfact - 1) / nfact : 1;
       mats = grid.resample ? prm.K_it : 1;
     }
-    r.kernel_launches = prm.K_it * (2 + (dev.dense ? 1 : 0) + 1 + 1 + refit + 1 + 3) +
-                        mats * (2 + (mixed ? 2 : 1)) + groups * (3 * panels - 1 + 2);
+    r.kernel_launches = prm.K_it * (1 + (dev.dense ? 1 : 0) + 1 + 1 + refit + 1) +
+                        mats * (1 + (mixed ? 2 : 1)) + groups * (3 * panels - 1 + 2);
     if (prm.timing && (int)events.size() >= 8 * prm.K_it) {
       // paths: ev0..ev1; Gram matrices, factors and inverses built ahead of
       // a group of iterations: ev3..ev7 of the group's first iteration;
