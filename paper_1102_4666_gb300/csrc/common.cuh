@@ -143,6 +143,41 @@ struct Math<double> {
 };
 
 // ---------------------------------------------------------------------------
+// Programmatic dependent launch: an iteration is a chain of some fifteen small
+// kernels around the path kernel, each a few microseconds long with about one
+// more between two of them.  A kernel launched by launch_pdl may be scheduled
+// while the one before it on the stream still runs; pdl_begin, first thing in
+// the kernel, waits until that one has completed and its writes are visible, and
+// then lets the next one be scheduled in turn (after the wait, so that no more
+// than one waits on the SMs).  Every kernel launched this way must call it in
+// every thread before it touches memory; their pointers are not __restrict__, as
+// a read-only load could be moved ahead of the wait.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_begin() {
+  pdl_wait();
+  pdl_trigger();
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                              A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
+// ---------------------------------------------------------------------------
 // Host-side description of one solve, shared by the launchers.
 // ---------------------------------------------------------------------------
 struct ModelHost {

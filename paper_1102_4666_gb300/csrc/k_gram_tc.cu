@@ -116,6 +116,7 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
 __global__ void __launch_bounds__(128, 1)
     k_gram_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
               const __grid_constant__ GramArgs ga) {
+  pdl_begin();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   // 1024-align the stage ring
   unsigned char* base = reinterpret_cast<unsigned char*>(
@@ -265,11 +266,20 @@ __global__ void __launch_bounds__(128, 1)
   }
 }
 
+// FP32 -> FP64 of normal numbers by their bits: the conversion instruction is as
+// slow as the FP64 addition after it
+__device__ __forceinline__ double to_f64(float f) {
+  const uint32_t b = __float_as_uint(f), e = (b >> 23) & 0xffu;
+  if (e == 0u || e == 255u) return (double)f;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b >> 3) & 0x0fffffffu) + 0x38000000u)), (int)(b << 29));
+}
+
 // A[l1][l2] = sum over splits (FP64, split order) of the partial tiles;
 // diagonal tiles are read on and above their diagonal only, so A is
 // exactly symmetric.
-__global__ void k_gram_reduce(int p, int ntile_side, int splits, const float* __restrict__ part,
-                              double* __restrict__ A) {
+__global__ void k_gram_reduce(int p, int ntile_side, int splits, const float* part,
+                              double* A) {
+  pdl_begin();
   const int tile = blockIdx.y;
   int t = tile, I = 0;
   while (t >= ntile_side - I) {
@@ -282,8 +292,17 @@ __global__ void k_gram_reduce(int p, int ntile_side, int splits, const float* __
   if (I == J && r > c) return;
   const int l1 = I * TILE + r, l2 = J * TILE + c;
   if (l1 >= p || l2 >= p) return;
+  const float* src = part + ((size_t)tile * splits * TILE + r) * TILE + c;
   double s = 0.0;
-  for (int q = 0; q < splits; ++q) s += (double)part[(((size_t)tile * splits + q) * TILE + r) * TILE + c];
+  int q = 0;
+  for (; q + 8 <= splits; q += 8) {  // eight loads in flight, added in split order
+    float f[8];
+#pragma unroll
+    for (int h = 0; h < 8; ++h) f[h] = src[(size_t)(q + h) * TILE * TILE];
+#pragma unroll
+    for (int h = 0; h < 8; ++h) s += to_f64(f[h]);
+  }
+  for (; q < splits; ++q) s += to_f64(src[(size_t)q * TILE * TILE]);
   A[(size_t)l1 * p + l2] = s;
   A[(size_t)l2 * p + l1] = s;
 }
@@ -355,10 +374,10 @@ cudaError_t launch_gram_tc(const ProblemDev& P, cudaStream_t st) {
   cudaError_t e =
       cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_gram_tc<<<tiles * ga.splits, 128, smem, st>>>(mh, ml, ga);
+  launch_pdl(k_gram_tc, tiles * ga.splits, 128, smem, st, mh, ml, ga);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   dim3 grid(TILE * TILE / 256, tiles);
-  k_gram_reduce<<<grid, 256, 0, st>>>(P.p, ga.ntile_side, ga.splits, P.gram_part, P.A);
+  launch_pdl(k_gram_reduce, grid, 256, 0, st, P.p, ga.ntile_side, ga.splits, P.gram_part, P.A);
   return cudaGetLastError();
 }

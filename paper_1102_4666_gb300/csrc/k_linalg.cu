@@ -12,8 +12,9 @@
 namespace {
 
 // eq. chat: c_i = (1/M) sum of the per-chunk sums, in chunk order
-__global__ void k_reduce_c(int i0, int count, int chunks, int M, const double* __restrict__ partial,
-                           double* __restrict__ c) {
+__global__ void k_reduce_c(int i0, int count, int chunks, int M, const double* partial,
+                           double* c) {
+  pdl_begin();
   const int i = i0 + blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= i0 + count) return;
   double s = 0.0;
@@ -27,10 +28,11 @@ __global__ void k_reduce_c(int i0, int count, int chunks, int M, const double* _
 // latency of its loads at small p (35 CTAs of 128 threads with few loads in
 // flight: 5.5 us at n = 2000, this 3.5 us).
 __global__ void __launch_bounds__(256) k_bt_times(int n, int n_pad, int p,
-                                                  const double* __restrict__ B,
-                                                  const double* __restrict__ y,
-                                                  const double* __restrict__ sub,
-                                                  double* __restrict__ out) {
+                                                  const double* B,
+                                                  const double* y,
+                                                  const double* sub,
+                                                  double* out) {
+  pdl_begin();
   __shared__ double ws[8];
   const int l = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -51,9 +53,10 @@ __global__ void __launch_bounds__(256) k_bt_times(int n, int n_pad, int p,
 // v[i] = sum_l B[l][i] x[l]: CTA of 32 points x 8 slices of the basis
 // functions (coalesced rows of B per warp), the slice sums added in order
 __global__ void __launch_bounds__(256) k_b_times(int n, int n_pad, int p,
-                                                 const double* __restrict__ B,
-                                                 const double* __restrict__ x,
-                                                 double* __restrict__ v) {
+                                                 const double* B,
+                                                 const double* x,
+                                                 double* v) {
+  pdl_begin();
   __shared__ double part[8][33];
   const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane;
@@ -89,8 +92,9 @@ __device__ __forceinline__ void lower_tile(int t, int& ti, int& tj) {
 // FP64 Gram A = B B^T on CUDA cores: one lower tile per CTA, written to both
 // triangles.
 __global__ void __launch_bounds__(256) k_gram_f64(int n, int n_pad, int p,
-                                                  const double* __restrict__ B,
-                                                  double* __restrict__ A) {
+                                                  const double* B,
+                                                  double* A) {
+  pdl_begin();
   __shared__ double Rs[T16][33], Cs[T16][33];
   int ti, tj;
   lower_tile(blockIdx.x, ti, tj);
@@ -124,7 +128,8 @@ __global__ void __launch_bounds__(256) k_gram_f64(int n, int n_pad, int p,
 // at Ainv + z p^2.
 
 // original diagonal of A, for the relative pivot test of the factorisation
-__global__ void k_save_diag(const double* __restrict__ A, int p, double* __restrict__ diag0) {
+__global__ void k_save_diag(const double* A, int p, double* diag0) {
+  pdl_begin();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   const size_t z = blockIdx.y;
   if (j < p) diag0[z * p + j] = A[z * p * p + (size_t)j * p + j];
@@ -154,10 +159,11 @@ __device__ __forceinline__ double rsqrt_f64(double a) {
 // column.  Per block: one warp on shared memory 65 us, this 26 us.
 // A pivot below 1e-13 of its original diagonal entry (or not finite) marks the
 // matrix as numerically singular: ST_NOT_PD, and the pivot becomes NaN.
-__global__ void __launch_bounds__(128) k_chol_diag(double* __restrict__ A, int p, int j0,
-                                                   int* __restrict__ status,
-                                                   const double* __restrict__ diag0,
-                                                   double* __restrict__ dinv) {
+__global__ void __launch_bounds__(128) k_chol_diag(double* A, int p, int j0,
+                                                   int* status,
+                                                   const double* diag0,
+                                                   double* dinv) {
+  pdl_begin();
   __shared__ double col[2][32], Ls[32][33], Ei[32][33], di[32];
   const size_t z = blockIdx.y;
   A += z * p * p;
@@ -179,6 +185,7 @@ __global__ void __launch_bounds__(128) k_chol_diag(double* __restrict__ A, int p
   __syncthreads();
 #pragma unroll
   for (int c = 0; c < 32; ++c) {
+    if (c >= nb) break;  // a short last block
     const double colv = col[c & 1][lane], piv = col[c & 1][c];
     // piv > thr and finite, on the bits (no FP64 comparison); thr >= 0
     const long long pb = __double_as_longlong(piv), tb = __shfl_sync(0xffffffffu, thr, c);
@@ -187,8 +194,7 @@ __global__ void __launch_bounds__(128) k_chol_diag(double* __restrict__ A, int p
     const double l = lane > c ? colv * inv : 0.0;
     // the next column first: its owner hands it on
     if (c < 31) {
-      constexpr int one = 1;
-      const int k = (c + one) / 4, w = (c + one) % 4;
+      const int k = (c + 1) / 4, w = (c + 1) % 4;
       const double ls = __shfl_sync(0xffffffffu, l, c + 1);
       if (warp == w) {
         R[k] -= l * ls;
@@ -234,8 +240,9 @@ __device__ __forceinline__ double diag_inv(const double* __restrict__ A, const d
 // Panel step 2: the rows below, L21 = A21 L11^-T: eight rows per CTA, an
 // output per thread (a substitution per row left a warp to 496 dependent steps
 // on its own: 24 us a panel, this 5 us)
-__global__ void __launch_bounds__(256) k_chol_trsm(double* __restrict__ A, int p, int j0,
-                                                   const double* __restrict__ dinv) {
+__global__ void __launch_bounds__(256) k_chol_trsm(double* A, int p, int j0,
+                                                   const double* dinv) {
+  pdl_begin();
   __shared__ double Li[32][33], a[8][33];
   const size_t z = blockIdx.y;
   A += z * p * p;
@@ -252,7 +259,8 @@ __global__ void __launch_bounds__(256) k_chol_trsm(double* __restrict__ A, int p
 }
 
 // trailing update A22 -= L21 L21^T on the lower triangle
-__global__ void __launch_bounds__(256) k_chol_update(double* __restrict__ A, int p, int j0) {
+__global__ void __launch_bounds__(256) k_chol_update(double* A, int p, int j0) {
+  pdl_begin();
   __shared__ double Lr[T16][33], Lc[T16][33];
   A += (size_t)blockIdx.y * p * p;
   int ti, tj;
@@ -285,8 +293,9 @@ __global__ void __launch_bounds__(256) k_chol_update(double* __restrict__ A, int
 // p = 924 (the FP64 pipe's time for p^3 / 3: 4.3 ms) with the factorisation
 // 17.1 -> 9.6 ms, twelve of p = 364 3.20 -> 1.89 ms, one of p = 364 1.74 -> 0.73.
 template <int C>
-__global__ void __launch_bounds__(32 * C) k_tri_inv(double* __restrict__ A, int p,
-                                                    const double* __restrict__ dinv) {
+__global__ void __launch_bounds__(32 * C) k_tri_inv(double* A, int p,
+                                                    const double* dinv) {
+  pdl_begin();
   extern __shared__ double Ms[];  // [row][C], rows padded to blocks of 32
   __shared__ double Lt[32][33], Ac[32][C + 1];
   constexpr int PER = 32 / C;  // tile elements per thread
@@ -340,9 +349,10 @@ __global__ void __launch_bounds__(32 * C) k_tri_inv(double* __restrict__ A, int 
 
 // A^-1 = M^T M: Ainv[a][b] = sum_{i >= max(a, b)} M_ia M_ib, the columns of M
 // being the rows of the upper triangle; lower tiles, written to both triangles
-__global__ void __launch_bounds__(256) k_inv_syrk(const double* __restrict__ A, int p,
-                                                  const double* __restrict__ dinv,
-                                                  double* __restrict__ Ainv) {
+__global__ void __launch_bounds__(256) k_inv_syrk(const double* A, int p,
+                                                  const double* dinv,
+                                                  double* Ainv) {
+  pdl_begin();
   __shared__ double Rs[T16][33], Cs[T16][33];
   const size_t z = blockIdx.y;
   A += z * p * p;
@@ -436,13 +446,14 @@ __device__ __forceinline__ double basis_value(uint2 pr, int nz, int eta, const d
 // CTA (one launch instead of four): the Chebyshev values of the point once in
 // shared memory, threads over basis functions, a fixed shuffle tree.
 __global__ void __launch_bounds__(256) k_update(const __grid_constant__ EvalArgs ea, int k, double t0,
-                                                double* __restrict__ alpha,
-                                                float* __restrict__ alpha32,
-                                                const double* __restrict__ delta,
-                                                const uint2* __restrict__ pairs,
-                                                const uint8_t* __restrict__ nnz,
-                                                const double* __restrict__ logS0,
-                                                double* __restrict__ out) {
+                                                double* alpha,
+                                                float* alpha32,
+                                                const double* delta,
+                                                const uint2* pairs,
+                                                const uint8_t* nnz,
+                                                const double* logS0,
+                                                double* out) {
+  pdl_begin();
   __shared__ double T[(BSDE_DMAX + 1) * 15], dT[(BSDE_DMAX + 1) * 15];
   __shared__ double red[BSDE_DMAX + 3][256];  // row 0: |delta|^2, 1: max |delta|, 2: u, 3..: du/dx_j
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, d = ea.d;
@@ -549,9 +560,10 @@ __global__ void __launch_bounds__(256) k_eval_many(const __grid_constant__ EvalA
 
 // monomial coefficients of u^k (basis of total degree <= 3): beta_m =
 // sum over the CSR row m of coef * alpha_l, in FP64, with an FP32 copy
-__global__ void k_cheb2mono(int pm, const int* __restrict__ row, const int* __restrict__ lidx,
-                            const double* __restrict__ coef, const double* __restrict__ alpha,
-                            double* __restrict__ beta, float* __restrict__ beta32) {
+__global__ void k_cheb2mono(int pm, const int* row, const int* lidx,
+                            const double* coef, const double* alpha,
+                            double* beta, float* beta32) {
+  pdl_begin();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= pm) return;
   double s = 0.0;
@@ -561,8 +573,9 @@ __global__ void k_cheb2mono(int pm, const int* __restrict__ row, const int* __re
 }
 
 // x (+)= Ainv b: warp per row, fixed shuffle order
-__global__ void k_inv_gemv(int p, const double* __restrict__ Ainv, const double* __restrict__ b,
-                           double* __restrict__ x, int accumulate) {
+__global__ void k_inv_gemv(int p, const double* Ainv, const double* b,
+                           double* x, int accumulate) {
+  pdl_begin();
   const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (row >= p) return;
@@ -581,7 +594,7 @@ static void launch_tri_inv(const ProblemDev& P, int nb, cudaStream_t st) {
   const size_t smem = (size_t)((P.p + 31) / 32 * 32) * C * sizeof(double);
   if (smem > 32 * 1024)
     cudaFuncSetAttribute(k_tri_inv<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_tri_inv<C><<<dim3((P.p + C - 1) / C, nb), 32 * C, smem, st>>>(P.A, P.p, P.dinv);
+  launch_pdl(k_tri_inv<C>, dim3((P.p + C - 1) / C, nb), 32 * C, smem, st, P.A, P.p, P.dinv);
 }
 
 // strips of 8 columns when there are enough of them for two CTAs per SM (they
@@ -596,50 +609,50 @@ void launch_inverse(const ProblemDev& P, int nb, cudaStream_t st) {
   else
     launch_tri_inv<1>(P, nb, st);
   const int T = (P.p + T16 - 1) / T16;
-  k_inv_syrk<<<dim3(T * (T + 1) / 2, nb), 256, 0, st>>>(P.A, P.p, P.dinv, P.Ainv);
+  launch_pdl(k_inv_syrk, dim3(T * (T + 1) / 2, nb), 256, 0, st, P.A, P.p, P.dinv, P.Ainv);
 }
 
 void launch_inv_gemv(const ProblemDev& P, const double* b, double* x, int accumulate,
                      cudaStream_t st) {
-  k_inv_gemv<<<(P.p * 32 + 255) / 256, 256, 0, st>>>(P.p, P.Ainv, b, x, accumulate);
+  launch_pdl(k_inv_gemv, (P.p * 32 + 255) / 256, 256, 0, st, P.p, P.Ainv, b, x, accumulate);
 }
 
 void launch_cheb2mono(const ProblemDev& P, cudaStream_t st) {
-  k_cheb2mono<<<(P.pm + 127) / 128, 128, 0, st>>>(P.pm, P.conv_row, P.conv_l, P.conv_c, P.alpha,
+  launch_pdl(k_cheb2mono, (P.pm + 127) / 128, 128, 0, st, P.pm, P.conv_row, P.conv_l, P.conv_c, P.alpha,
                                                    P.beta, P.beta32);
 }
 
 void launch_reduce_c(const ProblemDev& P, int M, cudaStream_t st) {
   const int count = P.shard_n > 0 ? P.shard_n : P.n;
   if (count <= 0) return;
-  k_reduce_c<<<(count + 255) / 256, 256, 0, st>>>(P.shard_i0, count, P.chunks, M, P.partial, P.c);
+  launch_pdl(k_reduce_c, (count + 255) / 256, 256, 0, st, P.shard_i0, count, P.chunks, M, P.partial, P.c);
 }
 
 void launch_gram_f64(const ProblemDev& P, cudaStream_t st) {
   const int T = (P.p + T16 - 1) / T16;
-  k_gram_f64<<<T * (T + 1) / 2, 256, 0, st>>>(P.n, P.n_pad, P.p, P.B, P.A);
+  launch_pdl(k_gram_f64, T * (T + 1) / 2, 256, 0, st, P.n, P.n_pad, P.p, P.B, P.A);
 }
 
 void launch_rhs(const ProblemDev& P, cudaStream_t st) {
-  k_bt_times<<<P.p, 256, 0, st>>>(P.n, P.n_pad, P.p, P.B, P.c, nullptr, P.rhs);
+  launch_pdl(k_bt_times, P.p, 256, 0, st, P.n, P.n_pad, P.p, P.B, P.c, nullptr, P.rhs);
 }
 
 void launch_cholesky(const ProblemDev& P, int nb, cudaStream_t st) {
-  k_save_diag<<<dim3((P.p + 255) / 256, nb), 256, 0, st>>>(P.A, P.p, P.diag0);
+  launch_pdl(k_save_diag, dim3((P.p + 255) / 256, nb), 256, 0, st, P.A, P.p, P.diag0);
   for (int j0 = 0; j0 < P.p; j0 += 32) {
-    k_chol_diag<<<dim3(1, nb), 128, 0, st>>>(P.A, P.p, j0, P.status, P.diag0, P.dinv);
+    launch_pdl(k_chol_diag, dim3(1, nb), 128, 0, st, P.A, P.p, j0, P.status, P.diag0, P.dinv);
     const int m = P.p - j0 - 32;
     if (m > 0) {
-      k_chol_trsm<<<dim3((m + 7) / 8, nb), 256, 0, st>>>(P.A, P.p, j0, P.dinv);
+      launch_pdl(k_chol_trsm, dim3((m + 7) / 8, nb), 256, 0, st, P.A, P.p, j0, P.dinv);
       const int T = (m + T16 - 1) / T16;
-      k_chol_update<<<dim3(T * (T + 1) / 2, nb), 256, 0, st>>>(P.A, P.p, j0);
+      launch_pdl(k_chol_update, dim3(T * (T + 1) / 2, nb), 256, 0, st, P.A, P.p, j0);
     }
   }
 }
 
 void launch_refine_residual(const ProblemDev& P, cudaStream_t st) {
-  k_b_times<<<(P.n + 31) / 32, 256, 0, st>>>(P.n, P.n_pad, P.p, P.B, P.delta, P.v);
-  k_bt_times<<<P.p, 256, 0, st>>>(P.n, P.n_pad, P.p, P.B, P.v, P.rhs, P.res);
+  launch_pdl(k_b_times, (P.n + 31) / 32, 256, 0, st, P.n, P.n_pad, P.p, P.B, P.delta, P.v);
+  launch_pdl(k_bt_times, P.p, 256, 0, st, P.n, P.n_pad, P.p, P.B, P.v, P.rhs, P.res);
 }
 
 static EvalArgs eval_args(const ModelHost& m, const GridHost& g, const ProblemDev& P) {
@@ -658,7 +671,7 @@ static EvalArgs eval_args(const ModelHost& m, const GridHost& g, const ProblemDe
 // alpha^{k+1} and the price and du/dx at (0, log S0) after iteration k; log S0
 // lives in the tail of the report block
 void launch_update(const ModelHost& m, const GridHost& g, const ProblemDev& P, int k, cudaStream_t st) {
-  k_update<<<1, 256, 0, st>>>(eval_args(m, g, P), k, 0.0, P.alpha, P.alpha32, P.delta, P.pairs, P.nnz,
+  launch_pdl(k_update, 1, 256, 0, st, eval_args(m, g, P), k, 0.0, P.alpha, P.alpha32, P.delta, P.pairs, P.nnz,
                               P.out + OUT_SIZE + 1 + BSDE_DMAX, P.out);
 }
 

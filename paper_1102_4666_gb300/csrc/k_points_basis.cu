@@ -35,11 +35,12 @@ __device__ __forceinline__ float to_tf32(float v) {
 constexpr int BASIS_PTS = 32;  // points per CTA of k_basis, one per lane
 
 __global__ void k_basis(int n, int n_pad, int p, int l_per, int dp, int eta,
-                        const uint2* __restrict__ pairs, const uint8_t* __restrict__ nnz,
-                        const uint32_t* __restrict__ key, uint32_t k, double* __restrict__ t,
-                        double* __restrict__ x, const __grid_constant__ BoxArgs box,
-                        double* __restrict__ B,
-                        float* __restrict__ Bhi, float* __restrict__ Blo, int split) {
+                        const uint2* pairs, const uint8_t* nnz,
+                        const uint32_t* key, uint32_t k, double* t,
+                        double* x, const __grid_constant__ BoxArgs box,
+                        double* B,
+                        float* Bhi, float* Blo, int split) {
+  pdl_begin();
   extern __shared__ double cheb[];  // [v][e][point]
   const int tid = threadIdx.x, nth = blockDim.x;
   const int i0 = blockIdx.x * BASIS_PTS;
@@ -127,6 +128,6 @@ void launch_basis(const ModelHost& m, const GridHost& g, const ProblemDev& P, ui
   if (gy < 1) gy = 1;
   const int l_per = (P.p + gy - 1) / gy;
   gy = (P.p + l_per - 1) / l_per;
-  k_basis<<<dim3(gx, gy), tpb, smem, st>>>(P.n, P.n_pad, P.p, l_per, dp, eta, P.pairs, P.nnz, P.key, k,
+  launch_pdl(k_basis, dim3(gx, gy), tpb, smem, st, P.n, P.n_pad, P.p, l_per, dp, eta, P.pairs, P.nnz, P.key, k,
                                             P.t, P.x, box, P.B, P.Bhi, P.Blo, split ? 1 : 0);
 }

@@ -16,10 +16,11 @@
 namespace {
 
 // copy B -> W, c -> y, squared column norms
-__global__ void k_qr_init(int n, int n_pad, int p, const double* __restrict__ B,
-                          const double* __restrict__ c, double* __restrict__ W,
-                          double* __restrict__ y, double* __restrict__ nrm, int* __restrict__ perm,
-                          uint32_t* __restrict__ sync) {
+__global__ void k_qr_init(int n, int n_pad, int p, const double* B,
+                          const double* c, double* W,
+                          double* y, double* nrm, int* perm,
+                          uint32_t* sync) {
+  pdl_begin();
   if (blockIdx.x == 0 && threadIdx.x < 2) sync[threadIdx.x] = 0u;
   const int l = blockIdx.x;  // column (p of them) or the right-hand side (l == p)
   const double* src = (l < p) ? B + (size_t)l * n_pad : c;
@@ -281,11 +282,12 @@ __global__ void __launch_bounds__(QR_THREADS, 1)
 // substitution, delta[perm[j]] = d_j (0 beyond r).  One CTA; blocks of 32
 // columns: warp 0 solves the block's triangle with shuffles, then every thread
 // takes the block's columns off its rows, the last column first.
-__global__ void __launch_bounds__(256) k_qr_solve(int n, int n_pad, int p, const double* __restrict__ W,
-                                                  const double* __restrict__ y,
-                                                  const int* __restrict__ perm,
-                                                  double* __restrict__ delta,
-                                                  double* __restrict__ work, int* __restrict__ rank_out) {
+__global__ void __launch_bounds__(256) k_qr_solve(int n, int n_pad, int p, const double* W,
+                                                  const double* y,
+                                                  const int* perm,
+                                                  double* delta,
+                                                  double* work, int* rank_out) {
+  pdl_begin();
   __shared__ int s_rank;
   __shared__ double xs[32];
   __shared__ const double* cols[32];
@@ -338,7 +340,7 @@ __global__ void __launch_bounds__(256) k_qr_solve(int n, int n_pad, int p, const
 // delta = argmin |c - X delta| by pivoted QR; the workspace (W: p x n_pad,
 // y: n, norms, perm, rank, the barrier's words) is P.qr_*
 void launch_qr_solve(const ProblemDev& P, cudaStream_t st) {
-  k_qr_init<<<P.p + 1, 256, 0, st>>>(P.n, P.n_pad, P.p, P.B, P.c, P.qr_W, P.qr_y, P.qr_nrm,
+  launch_pdl(k_qr_init, P.p + 1, 256, 0, st, P.n, P.n_pad, P.p, P.B, P.c, P.qr_W, P.qr_y, P.qr_nrm,
                                      P.qr_perm, P.qr_sync);
   int n = P.n, n_pad = P.n_pad, p = P.p, steps = P.p < P.n ? P.p : P.n;
   double *W = P.qr_W, *y = P.qr_y, *nrm = P.qr_nrm;
@@ -356,5 +358,5 @@ void launch_qr_solve(const ProblemDev& P, cudaStream_t st) {
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   void* args[] = {&n, &n_pad, &p, &steps, &W, &y, &nrm, &perm, &sync, &status};
   cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(QR_THREADS), args, smem, st);
-  k_qr_solve<<<1, 256, 0, st>>>(n, n_pad, p, W, y, perm, P.delta, P.res, P.qr_rank);
+  launch_pdl(k_qr_solve, 1, 256, 0, st, n, n_pad, p, W, y, perm, P.delta, P.res, P.qr_rank);
 }
