@@ -212,16 +212,43 @@ void Problem::ensure_events(int count) {
   }
 }
 
-// launch shape of the path kernel: threads per CTA and paths per thread,
-// limited by the shared memory of the per-thread Chebyshev tables
-int Problem::choose_launch(int d, int p, int eta, int N, int M, bool mx, bool dense, int& tpb,
-                           int& ppt) {
+// launch shape of the path kernel: threads per CTA, limited by the shared memory
+// of the per-thread Chebyshev tables, and paths per thread.  The dense
+// evaluations (tree: degree of the prefix tree, else 0):
+// * 128 threads (FP64: 64); the degree-6 tree at d = 5 (p up to 924 of straight-
+//   line code under the 80-register cap) shares its instruction fetches better
+//   among eight warps, unless M wastes a quarter of the last round: one launch
+//   at n = 2801, M = 4000 7.66 -> 6.33 ms, M = 1111 2.77 -> 2.06 ms (d <= 4 and
+//   the degree-4 trees at d >= 6 lose 1-4 % with 256);
+// * rounds of paths per CTA: four, or eight for the Horner loops when eight
+//   waves of CTAs remain (a CTA builds its volatility and Philox tables once:
+//   d = 10 16.25 -> 16.16 ms, d = 6 0.858 -> 0.848 ms; the trees but the largest
+//   lose 1 %, as does d = 3 with two waves), fewer when less than one wave would be left (the
+//   smallest solves);
+// * all CTAs alike: M = 1111 as rounds of 4 + 4 + 1 made every third CTA pay its
+//   tables for one round (d = 10 degree 4, n = 3000, 3.42 -> 2.83 ms as 3 + 3 + 3).
+int Problem::choose_launch(int d, int n, int p, int eta, int N, int M, bool mx, bool dense, int tree,
+                           int& tpb, int& ppt) {
   tpb = mx ? 128 : 64;
   while (tpb > 32 && paths_smem_bytes(d, p, eta, N, tpb, mx, dense) > 220 * 1024) tpb >>= 1;
   if (paths_smem_bytes(d, p, eta, N, tpb, mx, dense) > 220 * 1024) return BSDE_ERR_INVALID_ARG;
-  // about 512 paths per CTA, fewer for small M
-  ppt = 4;
-  while (ppt > 1 && (long long)tpb * ppt > 2LL * M) ppt >>= 1;
+  if (!dense) {
+    // about 512 paths per CTA, fewer for small M
+    ppt = 4;
+    while (ppt > 1 && (long long)tpb * ppt > 2LL * M) ppt >>= 1;
+    return BSDE_OK;
+  }
+  const bool big = tree && d <= 5 && p > 600;
+  if (big && 4LL * ((M + 255) / 256 * 256) <= 5LL * M &&
+      paths_smem_bytes(d, p, eta, N, 256, mx, dense) <= 220 * 1024)
+    tpb = 256;
+  const long long rounds = (M + tpb - 1) / tpb;
+  const long long wave = (long long)device_sm_count() * (mx ? 768 / tpb : 512 / tpb);
+  auto ctas = [&](long long t) { return n * ((rounds + t - 1) / t); };
+  long long t = big || (!tree && ctas(8) >= 8 * wave) ? 8 : 4;
+  while (t > 1 && ctas(t) < wave) t >>= 1;
+  const long long chunks = (rounds + t - 1) / t;
+  ppt = (int)((rounds + chunks - 1) / chunks);
   return BSDE_OK;
 }
 
@@ -373,15 +400,10 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
   }
   s.qr = prm.ls_mode == 1;
   s.pm = s.dense ? pm : 0;
-  if (choose_launch(d, s.dense ? pm : p, s.eta, s.N, s.M, mixed, s.dense, s.tpb, s.ppt) != BSDE_OK) {
+  if (choose_launch(d, n, s.dense ? pm : p, s.eta, s.N, s.M, mixed, s.dense, s.tree, s.tpb, s.ppt) !=
+      BSDE_OK) {
     err = "solve: basis and step count too large for the shared-memory tables";
     return BSDE_ERR_INVALID_ARG;
-  }
-  // the large tree evaluations (d >= 6): 8 warps enter each evaluation
-  // together (measured at d = 10, degree 4: 6.8 ms against 7.4 ms with 4)
-  if (s.tree && d >= 6 && s.M >= 512) {
-    s.tpb = 256;
-    s.ppt = 2;
   }
   if (prm.paths_tpb) {
     if (prm.paths_tpb < 32 || prm.paths_tpb > 256 || prm.paths_tpb % 32 ||

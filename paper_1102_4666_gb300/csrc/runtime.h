@@ -110,8 +110,8 @@ class Problem {
   cudaGraphExec_t gexec = nullptr;
   std::string graph_key;
   std::vector<cudaEvent_t> events;  // 8 per iteration when timing
-  int choose_launch(int d, int p, int eta, int N, int M, bool mixed, bool dense, int& tpb,
-                    int& ppt);
+  int choose_launch(int d, int n, int p, int eta, int N, int M, bool mixed, bool dense, int tree,
+                    int& tpb, int& ppt);
   void ensure_events(int count);
   // points, basis and Gram matrix of iterations k0 .. k0 + nb - 1 into the
   // nb slots of the factor block, then their batched factorisation and inverses
