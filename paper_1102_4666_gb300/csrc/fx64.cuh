@@ -68,6 +68,7 @@ FX_FN double from_bits(uint64_t b) {
   return x;
 }
 FX_FN double exp_lib(double x) { return ::exp(x); }
+FX_FN double log_lib(double x) { return ::log(x); }
 FX_FN void load2(const uint64_t* t, uint64_t& a, uint64_t& b) {
   a = t[0];
   b = t[1];
@@ -90,6 +91,7 @@ FX_FN float rcp_seed(float a) {
 FX_FN uint64_t bits(double x) { return (uint64_t)__double_as_longlong(x); }
 FX_FN double from_bits(uint64_t b) { return __longlong_as_double((long long)b); }
 FX_FN double exp_lib(double x) { return ::exp(x); }
+FX_FN double log_lib(double x) { return ::log(x); }
 FX_FN void load2(const uint64_t* t, uint64_t& a, uint64_t& b) {
   const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(t));
   a = v.x;
@@ -259,6 +261,35 @@ FX_FN double exp(double x) {
   const int64_t nt = (b >> 63) ? (int64_t)t : -(int64_t)t;   // e^x = 2^-nt
   const uint64_t E = pow2_neg(((uint64_t)nt & ((1ull << 54) - 1)) << 3);
   return pack(E, -63 - (int)(nt >> 54), 0);
+}
+
+// ln x with an absolute error below 2^-52 (the rounding of the result beyond
+// |ln x| = 2): x = y 2^e, y c = 1 - rho as in neg_log, rho exact from the low 64
+// bits of the product; the library's function for x <= 0, subnormal numbers,
+// NaN and infinities.  Not for relative accuracy next to x = 1.
+FX_FN double log_abs(double x) {
+  const uint64_t b = bits(x);
+  const int ex = (int)(b >> 52);
+  if (ex == 0 || ex >= 0x7ff) return log_lib(x);
+  const uint64_t m = (b & 0xfffffffffffffull) | 0x10000000000000ull;  // y at 2^53
+  uint64_t c, lnc;
+  load2(FX_LOG_TAB + 2 * ((int)(m >> 45) & 127), c, lnc);
+  const uint64_t rho = 0 - m * c;  // at 2^68, below 2^61
+  const uint64_t s = rho << 2;     // 64 rho at 2^64
+  const uint32_t sh = hi32(s);
+  const uint32_t q5 = (uint32_t)FX_LOG_C5 + mulhi32(sh, (uint32_t)FX_LOG_C6);
+  const uint64_t q4 = FX_LOG_C4 + mulhi32(sh, q5);
+  const uint64_t q3 = FX_LOG_C3 + mulhi_32(q4, sh);
+  const uint64_t q2 = FX_LOG_C2 + mulhi_32(q3, sh);
+  const uint64_t P = FX_LOG_C0 + mulhi(s, FX_LOG_C1 + mulhi(s, q2));
+  const uint64_t s2 = wide(sh, sh) + ((uint64_t)mulhi32(sh, lo32(s)) << 1);
+  const uint64_t ny = lnc + (rho >> 9) + (mulhi(s2, P) >> 17);  // -ln y at 2^59, below 2^59
+  const int e = ex - 1022;
+  const uint32_t ae = (uint32_t)(e < 0 ? -e : e);
+  const uint64_t l2 = (wide(ae, hi32(FX_LN2_64)) << 21) + (wide(ae, lo32(FX_LN2_64)) >> 11);  // |e| ln 2 at 2^53
+  const int64_t r = (e < 0 ? -(int64_t)l2 : (int64_t)l2) - (int64_t)((ny + 32) >> 6);
+  if (r == 0) return 0.0;
+  return pack((uint64_t)(r < 0 ? -r : r), -53, r < 0 ? 1u : 0u);
 }
 
 }  // namespace fx64

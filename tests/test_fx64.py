@@ -28,6 +28,7 @@ int t_bm(int n, const uint32_t* a, const uint32_t* b, double k, double* x, doubl
   return 1;
 }
 void t_logistic(int n, const double* y, int ab, double* o) { for (int i = 0; i < n; i++) o[i] = logistic_p1(y[i], ab); }
+void t_lnabs(int n, const double* x, double* o) { for (int i = 0; i < n; i++) o[i] = log_abs(x[i]); }
 void t_exp(int n, const double* x, double* o) { for (int i = 0; i < n; i++) o[i] = fx64::exp(x[i]); }
 }
 '''
@@ -141,3 +142,19 @@ def test_exp(lib):
     o = np.zeros(5)
     lib.t_exp(5, _p(s), _p(o))
     assert o[0] == np.inf and o[1] == 0 and o[2] == np.inf and o[3] == 0 and np.isnan(o[4])
+
+
+def test_log_absolute(lib):
+    rng = np.random.default_rng(6)
+    x = np.concatenate([100 * np.exp(rng.standard_normal(200)), np.exp(rng.uniform(-700, 700, 100)),
+                        [1.0, np.nextafter(1, 2), np.nextafter(1, 0), 2.0, 0.5, 2.2250738585072014e-308, 1.7e308, 100.0],
+                        (128 + np.arange(128)) / 256.0, np.nextafter((129 + np.arange(128)) / 256.0, 0)])
+    o = np.zeros(len(x))
+    lib.t_lnabs(len(x), _p(x), _p(o))
+    for i, v in enumerate(x):
+        want = D(float(v)).ln()
+        assert abs(D(float(o[i])) - want) <= max(abs(want) * D(2) ** -53, D(2) ** -53) + D(2) ** -53, v
+    s = np.array([0.0, np.inf, 5e-324, -1.0])
+    o = np.zeros(4)
+    lib.t_lnabs(4, _p(s), _p(o))
+    assert o[0] == -np.inf and o[1] == np.inf and abs(o[2] - np.log(5e-324)) < 1e-12 and np.isnan(o[3])
