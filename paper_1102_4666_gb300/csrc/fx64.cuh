@@ -200,20 +200,64 @@ FX_FN void trig_quadrant(uint32_t w, uint64_t& sn, uint64_t& cs) {
   cs = neg ? cs + b : cs - b;
 }
 
-// Box-Muller: (z0, z1) = scale sqrt(-2 ln u0) (cos, sin)(2 pi u1) with
-// u = (2 w + 1) 2^-33, rounded once to double
-FX_FN void box_muller(uint32_t w0, uint32_t w1, const Scale& sc, double& z0, double& z1) {
-  int e, at;
+// |z0| and |z1| of a Box-Muller pair, z = sm sqrt(-2 ln u0) (cos, sin)(2 pi u1),
+// u = (2 w + 1) 2^-33, as m 2^(e - 62), with their signs (0 or 1)
+FX_FN void box_muller_parts(uint32_t w0, uint32_t w1, uint64_t sm, uint64_t& m0, uint64_t& m1, int& e,
+                            uint32_t& n0, uint32_t& n1) {
+  int at;
   const uint64_t L = neg_log(w0, at);  // -ln u0 at 2^59 is -2 ln u0 at 2^58
-  const uint64_t S = mulhi(sqrt58(L, e), sc.sm);
+  const uint64_t S = mulhi(sqrt58(L, e), sm);
   e -= (at - 59) >> 1;
   uint64_t sn, cs;
   trig_quadrant(w1, sn, cs);
   const uint32_t qd = w1 >> 30;
-  const uint64_t c = (qd & 1) ? sn : cs, s = (qd & 1) ? cs : sn;
-  e += sc.se - 62;  // S at 2^63 times trig at 2^63, shifted by 64
-  z0 = pack(mulhi(S, c), e, (qd ^ (qd >> 1)) & 1);
-  z1 = pack(mulhi(S, s), e, qd >> 1);
+  m0 = mulhi(S, (qd & 1) ? sn : cs);  // S and the trigonometric factor at 2^63, shifted by 64
+  m1 = mulhi(S, (qd & 1) ? cs : sn);
+  n0 = (qd ^ (qd >> 1)) & 1;
+  n1 = qd >> 1;
+}
+
+// the pair times the scale, rounded once to double
+FX_FN void box_muller(uint32_t w0, uint32_t w1, const Scale& sc, double& z0, double& z1) {
+  uint64_t m0, m1;
+  uint32_t n0, n1;
+  int e;
+  box_muller_parts(w0, w1, sc.sm, m0, m1, e, n0, n1);
+  e += sc.se - 62;
+  z0 = pack(m0, e, n0);
+  z1 = pack(m1, e, n1);
+}
+
+// the pair (sm without the power of two of the scale) as signed numbers at 2^60;
+// |z| < 6.8
+FX_FN void box_muller_fixed(uint32_t w0, uint32_t w1, uint64_t sm, int64_t& z0, int64_t& z1) {
+  uint64_t m0, m1;
+  uint32_t n0, n1;
+  int e;  // at most 3
+  box_muller_parts(w0, w1, sm, m0, m1, e, n0, n1);
+  const int64_t a = (int64_t)((m0 << 1) >> (3 - e)), b = (int64_t)((m1 << 1) >> (3 - e));
+  z0 = n0 ? -a : a;
+  z1 = n1 ? -b : b;
+}
+
+// a b / 2^64 of signed numbers, to within 2
+FX_FN int64_t smulhi(int64_t a, int64_t b) {
+  const uint64_t m = mulhi((uint64_t)(a < 0 ? -a : a), (uint64_t)(b < 0 ? -b : b));
+  return ((a ^ b) < 0) ? -(int64_t)m : (int64_t)m;
+}
+
+// y 2^(se - 58) as a double, to within 2^-58 2^se
+FX_FN double from_fixed58(int64_t y, int se) {
+  return pack((uint64_t)(y < 0 ? -y : y) | 1u, se - 58, y < 0 ? 1u : 0u);
+}
+
+// x at 2^57 when |x| < 32 (exact to 2^-57); false otherwise, NaN included
+FX_FN bool to_fixed57(double x, int64_t& r) {
+  const uint64_t b = bits(x);
+  const int ex = (int)(b >> 52) & 0x7ff;
+  const int64_t v = (int64_t)shr(0x8000000000000000ull | (b << 11), 1029 - (ex > 1027 ? 1027 : ex));
+  r = (int64_t)b < 0 ? -v : v;
+  return ex <= 1027;
 }
 
 // 2^(-f), f = f57 2^-57 in [0, 1), at 2^63: error below 2^-61
@@ -229,14 +273,9 @@ FX_FN uint64_t pow2_neg(uint64_t f57) {
   return T - mulhi(T, m);
 }
 
-// 1 + 1 / (e^{2 y} + 1) in [1, 2], absolute error below 2^-52.9 (the result's
-// rounding); saturates for |y| >= 32 and for infinities
-FX_FN double logistic_p1(double y, bool absolute) {
-  const uint64_t b = bits(y);
-  const int ex = (int)(b >> 52) & 0x7ff;
-  const uint64_t m = 0x8000000000000000ull | (b << 11);
-  const uint64_t v = ex > 1027 ? ~0ull : shr(m, 1027 - ex);  // |y| at 2^59
-  const uint64_t t = mulhi(v, FX_2LOG2E_62);                 // |y| 2 log2(e) at 2^57
+// 1 + r in [1, 2] with r = 1 / (1 + E) (inverse false: 1 - that), E = 2^-t,
+// t at 2^57, t < 128: absolute error below 2^-52.9 (the result's rounding)
+FX_FN double logistic_of(uint64_t t, bool complement) {
   const uint64_t E = shr(pow2_neg(t & ((1ull << 57) - 1)), (int)(t >> 57));
   // q = 1 / (1 + E) in [1/2, 1]: R (1 + e + e^2), e = 1 - (1 + E) R exact to 2^-61
   const uint64_t D = (1ull << 62) + (E >> 1);
@@ -246,8 +285,24 @@ FX_FN double logistic_p1(double y, bool absolute) {
   const int64_t w = e0 + (swide(es, es) >> 43);
   const int64_t Rw = (int64_t)((uint64_t)((int64_t)(int32_t)(w >> 32) * R) + mulhi32(lo32((uint64_t)w), R));
   const uint64_t q = ((uint64_t)R << 32) + ((uint64_t)Rw << 3);  // at 2^63
-  const uint64_t r = ((b >> 63) && !absolute) ? q : (1ull << 63) - q;
+  const uint64_t r = complement ? (1ull << 63) - q : q;
   return from_bits(0x3ff0000000000000ull + ((r + 0x400) >> 11));
+}
+
+// 1 + 1 / (e^{2 y} + 1) in [1, 2] (absolute: of |y|); saturates for |y| >= 32
+// and for infinities
+FX_FN double logistic_p1(double y, bool absolute) {
+  const uint64_t b = bits(y);
+  const int ex = (int)(b >> 52) & 0x7ff;
+  const uint64_t m = 0x8000000000000000ull | (b << 11);
+  const uint64_t v = ex > 1027 ? ~0ull : shr(m, 1027 - ex);  // |y| at 2^59
+  return logistic_of(mulhi(v, FX_2LOG2E_62), !(b >> 63) || absolute);
+}
+
+// the same for y at 2^57, |y| < 64 (saturating beyond 44)
+FX_FN double logistic_p1_fixed(int64_t y, bool absolute) {
+  const uint64_t t = mulhi((uint64_t)(y < 0 ? -y : y), FX_2LOG2E_62);  // at 2^55
+  return logistic_of(t < (1ull << 62) ? t << 2 : ~0ull, y >= 0 || absolute);
 }
 
 // e^x: relative error below 2^-52.5; the library's function for |x| >= 256,

@@ -67,6 +67,10 @@ struct Args {
   R vb;
   R rho;  // constant correlation (dense evaluation)
   alignas(16) R kc[D];  // -2 log2(e) kappa_j: e^{2 (x - kappa)} = 2^{x 2 log2(e) + kc}
+  // FP64 paths: diagonal and column of the constant correlation's factor at
+  // 2^62 and kappa at 2^57, valid when fixed_ok
+  int64_t Ldf[D], Lcf[D], kf[D];
+  int fixed_ok;
   R sj[D], cj[D];  // sin and cos of the asset number j + 1 (sin/tanh volatility, FP64 rows)
   uint32_t k;
   uint32_t key0, key1;  // Philox key
@@ -1003,20 +1007,23 @@ __device__ __forceinline__ void load_state(const float4* p, int stride, R (&X)[D
 // states before and after step s* in Xs and Xn.  With a constant volatility
 // X is linear in the normals, X_n = x0 + n h (r - delta - sigma^2 / 2) +
 // sigma (L sum z): X, Xs and Xn are then the running sums of the normals
-// (0 on entry), one FP64 instruction per asset and step.  Bound by the FP64 pipe (two
-// lanes per SM and clock: 64 issue slots per instruction of a warp): with
-// the normals and the logistic function in fixed point (fx64.cuh) an asset's
-// step takes seven FP64 instructions (constant correlation, tanh
-// volatility) and about 250 integer ones.  The loop runs over the normals
+// (0 on entry), one FP64 instruction per asset and step.
+// Bound by the FP64 pipe (two lanes per SM and clock: 64 issue slots per
+// instruction of a warp), then by instruction issue.  In fixed point (fx64.cuh):
+// the normals, the logistic function of x - kappa, and with a constant
+// correlation the increments y = L z too (FIXED: the host has checked that L
+// and kappa fit, fixed_ok); an asset's step takes four FP64 instructions (tanh
+// volatility) and some 400 integer ones.  The loop runs over the normals
 // themselves, four (one Philox block) a turn, with (step, asset) counted
 // along, and the assets' states in local memory: unrolled over G steps of D
 // assets the fixed-point code would be several times the instruction cache,
 // and its states, normals and copies more registers than there are; a
 // state's load and store are nothing beside the 64-slot instructions.
 // Measured, d = 10 degree 3 (n = 1000, M = 100, N = 60): 11.08 ms a launch
-// with the library's log, sqrt, sincospi and exp, 2.24 ms with this (FP64 pipe
-// 74 % busy, a third of it the evaluation of u^k; issue 39 %).
-template <int VK, bool CC, int D>
+// with the library's log, sqrt, sincospi and exp, 2.15 ms with the normals and
+// the logistic function in fixed point (FP64 pipe 76 % busy), 1.91 ms with
+// the correlation and x - kappa too.
+template <int VK, bool CC, bool FIXED, int D>
 __device__ __forceinline__ void euler_path_f64(const Args<double, D>& a, const double* tab,
                                                const uint4* s_ph, const PhiloxFixed& pz,
                                                const Math<double>::Bm& bmk, double nhh, double h,
@@ -1025,15 +1032,20 @@ __device__ __forceinline__ void euler_path_f64(const Args<double, D>& a, const d
   const int total = a.N * D;
   int s = 0, j = 0;
   const double* row = tab;
-  double pre = 0.0;  // running sum of the constant-correlation factor
-  double zs[D];      // the step's normals so far (general correlation)
+  double pre = 0.0;   // running sum of the constant-correlation factor
+  int64_t pref = 0;   // the same at 2^58
+  double zs[D];       // the step's normals so far (general correlation)
 #pragma unroll 1
   for (int q = 0; q < total; q += 4) {
     const uint4 o = philox_tab(a, pz, s_ph[q >> 2]);
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
       double z[2];
-      Math<double>::box_muller(half ? o.z : o.x, half ? o.w : o.y, z[0], z[1], bmk);
+      int64_t zf[2];
+      if constexpr (FIXED)
+        fx64::box_muller_fixed(half ? o.z : o.x, half ? o.w : o.y, bmk.sc.sm, zf[0], zf[1]);
+      else
+        Math<double>::box_muller(half ? o.z : o.x, half ? o.w : o.y, z[0], z[1], bmk);
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
         if (s < a.N) {
@@ -1042,8 +1054,11 @@ __device__ __forceinline__ void euler_path_f64(const Args<double, D>& a, const d
           if constexpr (VK == VK_CONST) {
             xn = x + z[r];
           } else {
-            double y;
-            if constexpr (CC) {
+            double y, sig;
+            if constexpr (FIXED) {
+              y = fx64::from_fixed58(fx64::smulhi(zf[r], a.Ldf[j]) + pref, bmk.sc.se);
+              pref += fx64::smulhi(zf[r], a.Lcf[j]);
+            } else if constexpr (CC) {
               y = a.Ld[j] * z[r] + pre;
               pre += a.Lc[j] * z[r];
             } else {
@@ -1052,7 +1067,11 @@ __device__ __forceinline__ void euler_path_f64(const Args<double, D>& a, const d
 #pragma unroll 1
               for (int c = 0; c <= j; ++c) y += a.L[j][c] * zs[c];
             }
-            const double sig = sigma_j<VK>(a, row, j, x);
+            int64_t xf;
+            if (FIXED && (VK == VK_TANH || VK == VK_TANH_ABS) && fx64::to_fixed57(x, xf))
+              sig = row[2 * j] + row[2 * j + 1] * fx64::logistic_p1_fixed(xf - a.kf[j], VK == VK_TANH_ABS);
+            else
+              sig = sigma_j<VK>(a, row, j, x);
             xn = sig * (nhh * sig + y) + (h * a.rd[j] + x);
           }
           X[j] = xn;
@@ -1065,6 +1084,7 @@ __device__ __forceinline__ void euler_path_f64(const Args<double, D>& a, const d
             ++s;
             row += a.tab_stride;
             pre = 0.0;
+            pref = 0;
           }
         }
       }
@@ -1240,7 +1260,11 @@ __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
     const R nhh = R(-0.5) * h;
     const PhiloxFixed pz = philox_fix(a, (uint32_t)m, (uint32_t)i, tagZ);
     if constexpr (sizeof(R) == 8) {
-      euler_path_f64<VK, CC>(a, tab, s_ph, pz, bmk, nhh, h, sstar, X, Xs, Xn);
+      // uniform over the CTA: the point's step has a fixed-point scale and the model fits
+      if (CC && VK != VK_CONST && a.fixed_ok && bmk.plain)
+        euler_path_f64<VK, CC, true>(a, tab, s_ph, pz, bmk, nhh, h, sstar, X, Xs, Xn);
+      else
+        euler_path_f64<VK, CC, false>(a, tab, s_ph, pz, bmk, nhh, h, sstar, X, Xs, Xn);
     } else
     for (int s0 = 0; s0 < a.N; s0 += G) {
       R z[G * D];  // normals of G steps, scaled by sqrt(h)
@@ -1597,6 +1621,20 @@ cudaError_t launch(const ModelHost& m, const GridHost& g, const ProblemDev& P, i
       a.L[j][q] = (R)m.L[j * D + q];
       a.Cp[j + 1][q + 1] = (R)m.C[j * D + q];
     }
+  }
+  // rows of L of norm sqrt(2) at most (1 for a correlation matrix): |L z| < 32
+  a.fixed_ok = cc ? 1 : 0;
+  for (int j = 0; j < D && a.fixed_ok; ++j) {
+    double row = 0.0;
+    for (int q = 0; q < D; ++q) row += m.L[j * D + q] * m.L[j * D + q];
+    const double col = j + 1 < D ? m.L[(j + 1) * D + j] : 0.0;
+    if (!(row <= 2.0) || !(std::fabs(m.kappa[j]) < 32.0)) {
+      a.fixed_ok = 0;
+      break;
+    }
+    a.Ldf[j] = std::llrint(std::ldexp(m.L[j * D + j], 62));
+    a.Lcf[j] = std::llrint(std::ldexp(col, 62));
+    a.kf[j] = std::llrint(std::ldexp(m.kappa[j], 57));
   }
   for (int v = 0; v <= D; ++v) {
     a.ctr[v] = (R)(0.5 * (g.lo[v] + g.hi[v]));

@@ -27,6 +27,20 @@ int t_bm(int n, const uint32_t* a, const uint32_t* b, double k, double* x, doubl
   for (int i = 0; i < n; i++) box_muller(a[i], b[i], s, x[i], y[i]);
   return 1;
 }
+int t_bmf(int n, const uint32_t* a, const uint32_t* b, double k, int64_t* x, int64_t* y, double* d) {
+  Scale s;
+  if (!to_scale(k, s)) return 0;
+  for (int i = 0; i < n; i++) {
+    box_muller_fixed(a[i], b[i], s.sm, x[i], y[i]);
+    d[i] = from_fixed58((x[i] >> 2) + smulhi(y[i], (int64_t)3 << 60), s.se);  // x + 0.75 y
+  }
+  return 1;
+}
+void t_logf(int n, const double* y, double k, int ab, double* o) {
+  int64_t kf, yf;
+  to_fixed57(k, kf);
+  for (int i = 0; i < n; i++) o[i] = to_fixed57(y[i], yf) ? logistic_p1_fixed(yf - kf, ab) : -1.0;
+}
 void t_logistic(int n, const double* y, int ab, double* o) { for (int i = 0; i < n; i++) o[i] = logistic_p1(y[i], ab); }
 void t_lnabs(int n, const double* x, double* o) { for (int i = 0; i < n; i++) o[i] = log_abs(x[i]); }
 void t_exp(int n, const double* x, double* o) { for (int i = 0; i < n; i++) o[i] = fx64::exp(x[i]); }
@@ -158,3 +172,35 @@ def test_log_absolute(lib):
     o = np.zeros(4)
     lib.t_lnabs(4, _p(s), _p(o))
     assert o[0] == -np.inf and o[1] == np.inf and abs(o[2] - np.log(5e-324)) < 1e-12 and np.isnan(o[3])
+
+
+@pytest.mark.parametrize("k", [1.0, 0.0123456789, 3.0e100])
+def test_fixed_normals_and_their_sums(lib, k):
+    """x + 3/4 y of a pair: within the truncations of the two products (a few
+    2^-58) and the normals' own error, times the scale, and the last rounding."""
+    a = _words()
+    b = np.roll(a, 17).copy()
+    n = len(a)
+    x, y, d = np.zeros(n, np.int64), np.zeros(n, np.int64), np.zeros(n)
+    assert lib.t_bmf(n, _p(a), _p(b), ctypes.c_double(k), _p(x), _p(y), _p(d)) == 1
+    for i in range(n):
+        r = (-2 * ((2 * int(a[i]) + 1) * D(2) ** -33).ln()).sqrt() * D(k)
+        es, ec = _sincos((2 * int(b[i]) + 1) * PI / 2**32)
+        want = r * ec + r * es * D("0.75")
+        assert abs(D(float(d[i])) - want) <= abs(want) * D(2) ** -53 + D(k) * D(2) ** -52, (int(a[i]), int(b[i]))
+
+
+@pytest.mark.parametrize("absolute", [0, 1])
+def test_fixed_logistic(lib, absolute):
+    k = 4.605170185988092
+    y = np.concatenate([k + np.random.default_rng(3).standard_normal(200) * 4,
+                        [k, 0.0, -0.0, 5e-324, 1e-9, k + 1e-9, 31.9999, -31.9999, 32.0, -32.0, np.inf, np.nan]])
+    o = np.zeros(len(y))
+    lib.t_logf(len(y), _p(y), ctypes.c_double(k), absolute, _p(o))
+    for i, v in enumerate(y):
+        if not abs(v) < 32:
+            assert o[i] == -1.0
+            continue
+        z = D(float(v)) - D(k)
+        want = 1 + 1 / ((2 * (abs(z) if absolute else z)).exp() + 1)
+        assert abs(D(float(o[i])) - want) < D(2) ** -D("52.9"), v
