@@ -441,67 +441,115 @@ __device__ __forceinline__ double basis_value(uint2 pr, int nz, int eta, const d
   return val;
 }
 
+// u and its space derivatives at one point by a CTA of 256 threads, lanes =
+// basis functions: the Chebyshev values of the point once in shared memory (the
+// last warp; coord(v): its coordinate v), coef(l) gives the coefficients, the
+// sums over the threads are taken by one warp per row.  row(0, u) and row(j,
+// du/dx_j) are called by one lane each.
+constexpr int EVAL_ROWS = BSDE_DMAX + 1;
+struct EvalShared {
+  double T[EVAL_ROWS * 15], dT[EVAL_ROWS * 15];
+  double red[EVAL_ROWS][256];
+};
+__device__ __forceinline__ double row_sum(const double* q) {  // 256 values, one warp
+  q += threadIdx.x & 31;
+  double s = ((q[0] + q[32]) + (q[64] + q[96])) + ((q[128] + q[160]) + (q[192] + q[224]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+template <typename Coord, typename Coef, typename Row>
+__device__ __forceinline__ void eval_point(const EvalArgs& ea, const uint2* pairs, const uint8_t* nnz,
+                                           EvalShared& sh, Coord&& coord, Coef&& coef, Row&& row) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, d = ea.d;
+  if (warp == 7 && lane <= d)
+    cheb_column((coord(lane) - ea.ctr[lane]) * ea.sc[lane], ea.eta, sh.T + lane * ea.eta,
+                sh.dT + lane * ea.eta, 1);
+  for (int j = 1; j <= d; ++j) sh.red[j][tid] = 0.0;
+  __syncthreads();
+  double u = 0.0;
+  for (int l = tid; l < ea.p; l += 256) {
+    const double al = coef(l);
+    u += al * basis_value(pairs[l], nnz[l], ea.eta, sh.T, sh.dT, 1,
+                          [&](int v, double gd) { sh.red[v][tid] += al * gd; });
+  }
+  sh.red[0][tid] = u;
+  __syncthreads();
+  for (int r = warp; r <= d; r += 8) {
+    const double s = row_sum(sh.red[r]);
+    if (lane == 0) row(r, r == 0 ? s : s * ea.sc[r]);
+  }
+}
+
 // alpha += delta; ||delta||_2, ||delta||_inf into the report block; FP32 copy;
 // then the read-out of Section 5.3 at (0, log S0): price V = u and du/dx.  One
-// CTA (one launch instead of four): the Chebyshev values of the point once in
-// shared memory, threads over basis functions, a fixed shuffle tree.
+// CTA, one launch.
 __global__ void __launch_bounds__(256) k_update(const __grid_constant__ EvalArgs ea, int k, double t0,
-                                                double* alpha,
-                                                float* alpha32,
-                                                const double* delta,
-                                                const uint2* pairs,
-                                                const uint8_t* nnz,
-                                                const double* logS0,
-                                                double* out) {
+                                                double* alpha, float* alpha32, const double* delta,
+                                                const uint2* pairs, const uint8_t* nnz,
+                                                const double* logS0, double* out) {
   pdl_begin();
-  __shared__ double T[(BSDE_DMAX + 1) * 15], dT[(BSDE_DMAX + 1) * 15];
-  __shared__ double red[BSDE_DMAX + 3][256];  // row 0: |delta|^2, 1: max |delta|, 2: u, 3..: du/dx_j
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, d = ea.d;
-  // the last warp tabulates
-  if (warp == 7 && lane <= d) {
-    const double z = ((lane == 0 ? t0 : logS0[lane - 1]) - ea.ctr[lane]) * ea.sc[lane];
-    cheb_column(z, ea.eta, T + lane * ea.eta, dT + lane * ea.eta, 1);
-  }
-  for (int j = 0; j < d; ++j) red[3 + j][tid] = 0.0;
-  __syncthreads();
-  double a2 = 0.0, ai = 0.0, u = 0.0;
-  for (int l = tid; l < ea.p; l += 256) {
-    const double dl = delta[l];
-    const double al = alpha[l] + dl;
-    alpha[l] = al;
-    if (alpha32) alpha32[l] = (float)al;
-    a2 += dl * dl;
-    ai = fmax(ai, fabs(dl));
-    u += al * basis_value(pairs[l], nnz[l], ea.eta, T, dT, 1,
-                          [&](int v, double gd) { red[2 + v][tid] += al * gd; });
-  }
-  red[0][tid] = a2;
-  red[1][tid] = ai;
-  red[2][tid] = u;
-  __syncthreads();
-  for (int r = warp; r < 3 + d; r += 8) {
-    const double* q = red[r] + lane;
-    double s;
-    if (r == 1) {
-      s = q[0];
-      for (int w = 32; w < 256; w += 32) s = fmax(s, q[w]);
+  __shared__ EvalShared sh;
+  __shared__ double w2[8], wi[8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool it = k >= 0 && k < 64;
+  double a2 = 0.0, ai = 0.0;
+  eval_point(
+      ea, pairs, nnz, sh, [&](int v) { return v == 0 ? t0 : logS0[v - 1]; },
+      [&](int l) {
+        const double dl = delta[l];
+        const double al = alpha[l] + dl;
+        alpha[l] = al;
+        if (alpha32) alpha32[l] = (float)al;
+        a2 += dl * dl;
+        ai = fmax(ai, fabs(dl));
+        return al;
+      },
+      [&](int j, double s) {
+        if (j > 0) {
+          out[OUT_DUDX + j - 1] = s;
+        } else {
+          out[OUT_PRICE] = s;
+          if (it) out[OUT_PRICE_IT + k] = s;
+        }
+      });
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s = fmax(s, __shfl_xor_sync(0xffffffffu, s, o));
-    } else {
-      s = ((q[0] + q[32]) + (q[64] + q[96])) + ((q[128] + q[160]) + (q[192] + q[224]));
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    }
-    const bool it = k >= 0 && k < 64;
-    if (lane != 0) continue;
-    if (r == 0 && it) out[OUT_RES2 + k] = sqrt(s);
-    if (r == 1 && it) out[OUT_RESI + k] = s;
-    if (r == 2) {
-      out[OUT_PRICE] = s;
-      if (it) out[OUT_PRICE_IT + k] = s;
-    }
-    if (r >= 3) out[OUT_DUDX + r - 3] = s * ea.sc[r - 2];
+  for (int o = 16; o > 0; o >>= 1) {
+    a2 += __shfl_xor_sync(0xffffffffu, a2, o);
+    ai = fmax(ai, __shfl_xor_sync(0xffffffffu, ai, o));
   }
+  if (lane == 0) {
+    w2[warp] = a2;
+    wi[warp] = ai;
+  }
+  __syncthreads();
+  if (tid == 0 && it) {
+    for (int w = 1; w < 8; ++w) {
+      a2 += w2[w];
+      ai = fmax(ai, wi[w]);
+    }
+    out[OUT_RES2 + k] = sqrt(a2);
+    out[OUT_RESI + k] = ai;
+  }
+}
+
+// u and dV/dS (delta may be null) at a few query points, one CTA each
+__global__ void __launch_bounds__(256) k_eval_few(const __grid_constant__ EvalArgs ea,
+                                                  const double* alpha, const uint2* pairs,
+                                                  const uint8_t* nnz, const double* qt, const double* S,
+                                                  double* price, double* delta) {
+  __shared__ EvalShared sh;
+  const size_t q = blockIdx.x;
+  const double* Sq = S + q * ea.d;
+  eval_point(
+      ea, pairs, nnz, sh, [&](int v) { return v == 0 ? qt[q] : fx64::log_abs(Sq[v - 1]); },
+      [&](int l) { return alpha[l]; },
+      [&](int j, double s) {
+        if (j == 0)
+          price[q] = s;
+        else if (delta)
+          delta[q * ea.d + j - 1] = s / Sq[j - 1];
+      });
 }
 
 // u and du/dx at query points, threads = queries: CTA of 32 points x slices of
@@ -716,13 +764,19 @@ void launch_update(const ModelHost& m, const GridHost& g, const ProblemDev& P, i
                               P.out + OUT_SIZE + 1 + BSDE_DMAX, P.out);
 }
 
-// price and dV/dS (delta may be null) at q points (t, S).  As many slices of the
-// basis as keep four warps on every scheduler, at most eight: a few points are
-// spread over the basis functions, many need no more than a warp per 32.
+// price and dV/dS (delta may be null) at q points (t, S).  Up to eight points per
+// SM: a CTA per point, as a warp of k_eval_many takes as long for one point as for
+// 32 (the call with 600 points at d = 10, p = 1001 115 us; 620 points in the
+// other form 196 us, 1500 points 212 us); more: as many slices of the basis as
+// keep eight warps on every scheduler, at most eight.
 cudaError_t launch_eval_points(const ModelHost& m, const GridHost& g, const ProblemDev& P, int q,
                                const double* t, const double* S, double* price, double* delta,
                                cudaStream_t st) {
   const EvalArgs ea = eval_args(m, g, P);
+  if (q <= 8 * device_sm_count()) {
+    k_eval_few<<<q, 256, 0, st>>>(ea, P.alpha, P.pairs, P.nnz, t, S, price, delta);
+    return cudaGetLastError();
+  }
   const int groups = (q + 31) / 32;
   int slices = 8;
   while (slices > 1 && (long long)groups * slices > 32LL * device_sm_count()) slices >>= 1;

@@ -14,7 +14,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("d,eta,q,m", [(1, 1, 1.0, 1), (1, 6, 1.0, 33), (2, 15, 1.0, 31), (3, 0, 1.0, 5), (4, 5, 0.7, 64),
-                                       (5, 6, 1.0, 257), (10, 3, 1.0, 40000), (10, 4, 1.0, 3), (10, 5, 0.6, 100)])
+                                       (5, 6, 1.0, 257), (10, 3, 1.0, 40000), (10, 4, 1.0, 3), (10, 5, 0.6, 100),
+                                       (3, 2, 1.0, 1249), (5, 6, 0.8, 2000), (10, 2, 1.0, 1217), (2, 0, 1.0, 3000)])
 def test_eval_against_oracle(d, eta, q, m):
     import paper_1102_4666_gb300 as G
     n = 2 * len(O.multi_index_set(d + 1, eta, q)) + 2
