@@ -1227,8 +1227,11 @@ __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
   // serve the others.  The loop then runs the same number of paths on every
   // thread of the CTA; threads past the last path compute one that is
   // discarded.  (Measured: d = 10 degree 4 16.1 -> 7.4 ms, d = 5 degree 4
-  // 4.02 -> 3.75 ms; the degree-3 loops at d = 10 lose 2 % with it.)
-  constexpr bool SYNC_EVAL = EV == EV_DENSE4 || EV >= EV_TREE4;
+  // 4.02 -> 3.75 ms; the degree-3 loops at d = 10 lose 2 % with it.)  In FP64
+  // the degree-3 loops at d >= 8 are as long (d = 10, n = 1000, M = 2000, N = 20:
+  // 13.87 -> 11.72 ms; d = 6 loses 5 %).
+  constexpr bool SYNC_EVAL =
+      EV == EV_DENSE4 || EV >= EV_TREE4 || (sizeof(R) == 8 && EV == EV_DENSE3 && D >= 8);
   for (int jp = 0; jp < a.ppt; ++jp) {
     const int m = chunk * ppc + jp * tpb + tid;
     if constexpr (SYNC_EVAL) {

@@ -215,7 +215,11 @@ void Problem::ensure_events(int count) {
 // launch shape of the path kernel: threads per CTA, limited by the shared memory
 // of the per-thread Chebyshev tables, and paths per thread.  The dense
 // evaluations (tree: degree of the prefix tree, else 0):
-// * 128 threads (FP64: 64); the degree-6 tree at d = 5 (p up to 924 of straight-
+// * FP64: 128 threads (64 for M <= 64), one round: its code is several times the
+//   instruction cache and warps that start together share the fetches (d = 10,
+//   n = 1000, M = 2000, N = 20: 64 threads and 4 rounds 16.97 ms, 128 and 4 16.13,
+//   128 and 1 13.87; d = 5 degree 4 3.43 -> 3.12, d = 3 1.93 -> 1.85);
+// * FP32: 128 threads; the degree-6 tree at d = 5 (p up to 924 of straight-
 //   line code under the 80-register cap) shares its instruction fetches better
 //   among eight warps, unless M wastes a quarter of the last round: one launch
 //   at n = 2801, M = 4000 7.66 -> 6.33 ms, M = 1111 2.77 -> 2.06 ms (d <= 4 and
@@ -238,12 +242,17 @@ int Problem::choose_launch(int d, int n, int p, int eta, int N, int M, bool mx, 
     while (ppt > 1 && (long long)tpb * ppt > 2LL * M) ppt >>= 1;
     return BSDE_OK;
   }
+  if (!mx) {
+    tpb = M > 64 ? 128 : 64;
+    ppt = 1;
+    return paths_smem_bytes(d, p, eta, N, tpb, mx, dense) > 220 * 1024 ? BSDE_ERR_INVALID_ARG : BSDE_OK;
+  }
   const bool big = tree && d <= 5 && p > 600;
   if (big && 4LL * ((M + 255) / 256 * 256) <= 5LL * M &&
       paths_smem_bytes(d, p, eta, N, 256, mx, dense) <= 220 * 1024)
     tpb = 256;
   const long long rounds = (M + tpb - 1) / tpb;
-  const long long wave = (long long)device_sm_count() * (mx ? 768 / tpb : 512 / tpb);
+  const long long wave = (long long)device_sm_count() * (768 / tpb);
   auto ctas = [&](long long t) { return n * ((rounds + t - 1) / t); };
   long long t = big || (!tree && ctas(8) >= 8 * wave) ? 8 : 4;
   while (t > 1 && ctas(t) < wave) t >>= 1;
