@@ -226,6 +226,7 @@ struct ProblemDev {
   float* alpha32 = nullptr;   // [p] FP32 copy for the mixed path kernel
   uint2* pairs = nullptr;     // [p] packed (variate, degree) bytes
   uint8_t* nnz = nullptr;     // [p] active variates per basis function
+  uint2* prog = nullptr;      // [p] the basis as a tree (build_eval_program), for the table evaluation
   uint32_t* key = nullptr;    // [2] Philox key (device copy, read by the basis kernel)
   uint32_t seed_key[2] = {0, 0};  // the same key on the host, a parameter of the path kernel
   int* status = nullptr;      // [1] device status bits

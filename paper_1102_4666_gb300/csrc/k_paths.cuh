@@ -78,7 +78,7 @@ struct Args {
   const double* pt;
   const double* px;
   const R* alpha;
-  const uint2* pairs;
+  const uint2* pairs;  // constant correlation: the tree of build_eval_program
   const uint8_t* nnz;
   double* partial;
 };
@@ -306,6 +306,72 @@ __device__ __forceinline__ void term(const R* __restrict__ tb, int S, int eta, i
     g += al * gen;
     uT += al * valT;
   }
+}
+
+// The table evaluation with a constant correlation rho: the basis as a tree
+// (build_eval_program), a node being a function and its children the products
+// with one more, later variate, so that Q_N = alpha_N + sum_c T_c Q_c is the
+// part of u under N, divided by N's own factors.  With W = st st^T C, C = rho off
+// the diagonal, each node carries for Q: V the value, S the derivative along st,
+// G the generator (drift, half the diffusion) and the value at maturity; folding
+// child c with the factor T_e(z_v) into its parent takes
+//   V += T V_c;  S += T S_c + s T' V_c;  G += T G_c + (b T' + s^2 T''/2) V_c + rho s T' S_c
+// (a leaf's V_c is its coefficient, S_c = G_c = 0): four multiply-adds for a
+// leaf and ten operations for a node, instead of products over all the factors of every
+// function on its own.  The nodes are visited children first; the sums of the
+// open nodes, one per depth, stay in registers.  Four tables per variate and
+// degree instead of five leave room for more CTAs: FP64 at d = 5 degree 6 was held
+// to one warp per scheduler.  One launch against products function by function
+// (with the steps' arithmetic of the time): FP64 d = 5 degree 6 (n = 2000, M = 64)
+// 12.3 -> 3.7 ms, d = 8 degree 4 9.0 -> 2.9; FP32 d = 10 degree 5 q = 0.6 3.89 ->
+// 3.30, d = 3 degree 8 1.72 -> 1.16.
+template <typename R>
+struct TreeSums {
+  R V[BSDE_NNZ_MAX + 2], G[BSDE_NNZ_MAX + 2], S[BSDE_NNZ_MAX + 2], E[BSDE_NNZ_MAX + 2];
+};
+template <int K, typename R>
+__device__ __forceinline__ void fold(TreeSums<R>& s, bool leaf, R al, R t, R a1, R s1, R rho, R tT) {
+  if (leaf) {
+    s.V[K] += t * al;
+    s.G[K] += a1 * al;
+    s.S[K] += s1 * al;
+    s.E[K] += tT * al;
+  } else {
+    const R v = al + s.V[K + 1], e = al + s.E[K + 1];
+    s.V[K] += t * v;
+    s.G[K] += t * s.G[K + 1] + a1 * v + s1 * (rho * s.S[K + 1]);
+    s.S[K] += t * s.S[K + 1] + s1 * v;
+    s.E[K] += tT * e;
+    s.V[K + 1] = s.G[K + 1] = s.S[K + 1] = s.E[K + 1] = R(0);
+  }
+}
+template <typename R>
+__device__ __forceinline__ void eval_program(const R* __restrict__ tb, int stride, int eta, int tpb, int tid,
+                                             const uint2* __restrict__ prog, int p,
+                                             const R* __restrict__ alpha, R rho, R& u, R& gen, R& uT) {
+  TreeSums<R> s;
+#pragma unroll
+  for (int k = 0; k < BSDE_NNZ_MAX + 2; ++k) s.V[k] = s.G[k] = s.S[k] = s.E[k] = R(0);
+  for (int i = 0; i + 1 < p; ++i) {
+    const uint2 w = prog[i];
+    const R* f = tb + ((int)(w.y & 15u) * eta + (int)((w.y >> 4) & 15u) - 1) * tpb + tid;
+    const R al = alpha[w.x], t = f[0], a1 = f[stride], s1 = f[2 * stride], tT = f[3 * stride];
+    const bool leaf = (w.y >> 12) != 0u;
+    switch ((w.y >> 8) & 15u) {
+      case 1: fold<1>(s, leaf, al, t, a1, s1, rho, tT); break;
+      case 2: fold<2>(s, leaf, al, t, a1, s1, rho, tT); break;
+      case 3: fold<3>(s, leaf, al, t, a1, s1, rho, tT); break;
+      case 4: fold<4>(s, leaf, al, t, a1, s1, rho, tT); break;
+      case 5: fold<5>(s, leaf, al, t, a1, s1, rho, tT); break;
+      case 6: fold<6>(s, leaf, al, t, a1, s1, rho, tT); break;
+      case 7: fold<7>(s, leaf, al, t, a1, s1, rho, tT); break;
+      default: fold<8>(s, leaf, al, t, a1, s1, rho, tT); break;
+    }
+  }
+  const R c = alpha[prog[p - 1].x];
+  u = c + s.V[1];
+  gen = s.G[1];
+  uT = c + s.E[1];
 }
 
 // u^k, (d_t + L^N) u^k at z (the reduced (tau, X_tau)) and u^k at zT (the
@@ -1134,7 +1200,7 @@ __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
     s_nnz = smem_raw + off;
     off += ((size_t)a.p + 15) & ~(size_t)15;
     cheb = reinterpret_cast<R*>(smem_raw + off);
-    off += (size_t)5 * S * sizeof(R);
+    off += (size_t)(CC ? 4 : 5) * S * sizeof(R);
     off = (off + 15) & ~(size_t)15;
   }
   double* red = reinterpret_cast<double*>(smem_raw + off);          // 32
@@ -1442,26 +1508,36 @@ __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
           }
           const int base = (v * a.eta + e - 1) * tpb;
           tb[base] = t1;
-          tb[base + S] = bt * d1;
-          tb[base + 2 * S] = st * d1;
-          tb[base + 3 * S] = st * st * e1;
-          tb[base + 4 * S] = T1;
+          if constexpr (CC) {
+            tb[base + S] = bt * d1 + R(0.5) * (st * st * e1);
+            tb[base + 2 * S] = st * d1;
+            tb[base + 3 * S] = T1;
+          } else {
+            tb[base + S] = bt * d1;
+            tb[base + 2 * S] = st * d1;
+            tb[base + 3 * S] = st * st * e1;
+            tb[base + 4 * S] = T1;
+          }
         }
       }
-      const R* tbr = cheb;
-      for (int l = 0; l < a.p; ++l) {
-        const R al = s_alpha[l];
-        const uint2 pr = s_pairs[l];
-        switch (s_nnz[l]) {
-          case 0: term<0, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
-          case 1: term<1, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
-          case 2: term<2, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
-          case 3: term<3, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
-          case 4: term<4, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
-          case 5: term<5, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
-          case 6: term<6, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
-          case 7: term<7, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
-          default: term<8, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
+      if constexpr (CC) {
+        eval_program<R>(cheb, S, a.eta, tpb, tid, s_pairs, a.p, s_alpha, a.rho, u, gsum, uT);
+      } else {
+        const R* tbr = cheb;
+        for (int l = 0; l < a.p; ++l) {
+          const R al = s_alpha[l];
+          const uint2 pr = s_pairs[l];
+          switch (s_nnz[l]) {
+            case 0: term<0, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
+            case 1: term<1, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
+            case 2: term<2, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
+            case 3: term<3, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
+            case 4: term<4, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
+            case 5: term<5, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
+            case 6: term<6, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
+            case 7: term<7, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
+            default: term<8, R>(tbr, S, a.eta, tpb, tid, pr, s_cp, DP, al, u, gsum, uT); break;
+          }
         }
       }
     }
@@ -1515,7 +1591,7 @@ constexpr bool paths_lr() {
 // dynamic shared memory of the path kernel; dense: p is the number of
 // monomial coefficients and there are no per-thread tables
 inline size_t smem_bytes(int d, int p, int eta, int N, int tpb, size_t rsize, bool dense,
-                         int tab_stride, bool pairs, bool xcopy) {
+                         int tab_stride, bool pairs, bool xcopy, int tables = 5) {
   const int dp = d + 1;
   // the volatility table, 16-byte aligned; the coefficients (twice when
   // `pairs`: the prefix-tree evaluation with FP32 paths reads them in pairs)
@@ -1526,7 +1602,7 @@ inline size_t smem_bytes(int d, int p, int eta, int N, int tpb, size_t rsize, bo
   if (!dense) {
     off += (size_t)p * sizeof(uint2);
     off += ((size_t)p + 15) & ~(size_t)15;
-    off += (size_t)5 * dp * eta * tpb * rsize;
+    off += (size_t)tables * dp * eta * tpb * rsize;
     off = (off + 15) & ~(size_t)15;
   }
   off += 32 * sizeof(double);
@@ -1671,7 +1747,7 @@ cudaError_t launch(const ModelHost& m, const GridHost& g, const ProblemDev& P, i
     a.alpha = reinterpret_cast<const R*>(P.alpha32);
   else
     a.alpha = reinterpret_cast<const R*>(P.alpha);
-  a.pairs = P.pairs;
+  a.pairs = cc ? P.prog : P.pairs;
   a.nnz = P.nnz;
   a.partial = P.partial;
   const bool dense = P.dense;
@@ -1685,7 +1761,8 @@ cudaError_t launch(const ModelHost& m, const GridHost& g, const ProblemDev& P, i
   const size_t smem = smem_bytes(D, a.p, a.eta, N, tpb, sizeof(R), dense, a.tab_stride,
                                 dense && sizeof(R) == 4,
                                 dense && copy_smem(P.tree > 0 ? EV_TREE4 : P.dense4 ? EV_DENSE4 : EV_DENSE3,
-                                                   sizeof(R) == 4, D));
+                                                   sizeof(R) == 4, D),
+                                cc ? 4 : 5);
   const int vk = (m.vol_kind == 0)   ? VK_CONST
                  : (m.vol_kind == 1) ? VK_TANH_ABS
                  : (m.vol_kind == 3) ? VK_DUPIRE

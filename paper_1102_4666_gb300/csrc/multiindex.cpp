@@ -65,6 +65,43 @@ bool pack_multi_indices(const std::vector<std::vector<int>>& nus, std::vector<ui
   return true;
 }
 
+void build_eval_program(const std::vector<std::vector<int>>& nus, std::vector<uint32_t>& prog) {
+  std::map<std::vector<int>, int> at;
+  for (size_t l = 0; l < nus.size(); ++l) at[nus[l]] = (int)l;
+  std::vector<std::vector<int>> kids(nus.size());
+  std::vector<uint32_t> word(nus.size(), 0u);
+  for (size_t l = 0; l < nus.size(); ++l) {
+    std::vector<int> parent = nus[l];
+    int last = -1;
+    uint32_t depth = 0;
+    for (int v = 0; v < (int)parent.size(); ++v)
+      if (parent[v] > 0) {
+        last = v;
+        ++depth;
+      }
+    if (last < 0) continue;  // the constant
+    word[l] = (uint32_t)last | ((uint32_t)parent[last] << 4) | (depth << 8);
+    parent[last] = 0;
+    kids[at[parent]].push_back((int)l);
+  }
+  prog.clear();
+  prog.reserve(2 * nus.size());
+  // post-order with an explicit stack of (function, next child)
+  std::vector<std::pair<int, size_t>> stack;
+  if (!nus.empty()) stack.push_back({at[std::vector<int>(nus[0].size(), 0)], 0});
+  while (!stack.empty()) {
+    const int l = stack.back().first;
+    if (stack.back().second < kids[l].size()) {
+      const int k = kids[l][stack.back().second++];
+      stack.push_back({k, 0});
+    } else {
+      prog.push_back((uint32_t)l);
+      prog.push_back(word[l] | (kids[l].empty() ? 1u << 12 : 0u));
+      stack.pop_back();
+    }
+  }
+}
+
 // Chebyshev -> monomial map of a basis of total degree <= 3 or 4.  Monomials
 // in the order constant, z_a, z_a z_b (a <= b), z_a z_b z_c (a <= b <= c)
 // and, for a degree-4 basis, z_a z_b z_c z_e (a <= b <= c <= e), each group

@@ -11,6 +11,12 @@ std::vector<std::vector<int>> build_multi_indices(int dp, int eta, double q);
 // pack each multi-index as (variate << 4 | degree) bytes in increasing
 // variate order, two 32-bit words per basis function; false when a variate
 // or degree exceeds 15 or more than 8 variates are active
+// The basis as a tree, each function's parent being the function without its
+// last active variate (both kinds of index set contain it): two words per
+// function, all of a function's children before it (the constant last):
+// {basis index, variate | degree << 4 | depth << 8 | leaf << 12}
+void build_eval_program(const std::vector<std::vector<int>>& nus, std::vector<uint32_t>& prog);
+
 bool pack_multi_indices(const std::vector<std::vector<int>>& nus, std::vector<uint32_t>& pairs_xy,
                         std::vector<uint8_t>& nnz, int& max_deg);
 

@@ -96,6 +96,12 @@ extern "C" BSDE_API int bsde_corrections_noalloc(
       set_msg(errbuf, errbuf_len, "corrections_noalloc: basis needs more than 8 active variates");
       return BSDE_ERR_INVALID_ARG;
     }
+    std::vector<uint32_t> prog;
+    build_eval_program(nus, prog);
+    bool const_corr = true;
+    for (int i = 0; i < m.d; ++i)
+      for (int j = 0; j < m.d; ++j)
+        if (i != j && m.C[i * m.d + j] != m.C[m.d > 1 ? 1 : 0]) const_corr = false;
     const int p = (int)nus.size();
     const bool mixed = precision == BSDE_PREC_MIXED;
     const int eta_t = max_deg < 1 ? 1 : max_deg;
@@ -140,6 +146,7 @@ extern "C" BSDE_API int bsde_corrections_noalloc(
     P.key = (uint32_t*)s;
     P.status = (int*)(s + 16);
     P.pairs = (uint2*)(s + 256);
+    P.prog = P.pairs;
     P.nnz = (uint8_t*)(s + 256 + (size_t)NOALLOC_MAX_P * 8);
     P.alpha32 = (float*)(s + 256 + (size_t)NOALLOC_MAX_P * 9 + 256);
     P.partial = (double*)(s + TABLE_BYTES);
@@ -151,7 +158,9 @@ extern "C" BSDE_API int bsde_corrections_noalloc(
     // every scratch word the kernels read is rewritten here; the partial
     // sums are all overwritten by the path kernel before they are read
     e = cudaMemcpyAsync(P.key, key, sizeof(key), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(P.pairs, pairs.data(), (size_t)p * 8, cudaMemcpyHostToDevice, st);
+    // the path kernel reads the basis from the same place in either form
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(P.pairs, const_corr ? prog.data() : pairs.data(), (size_t)p * 8, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(P.nnz, nnz.data(), (size_t)p, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && mixed) {
       k_to_f32<<<(p + 127) / 128, 128, 0, st>>>(p, alpha_dev, P.alpha32);

@@ -215,7 +215,7 @@ void Problem::ensure_events(int count) {
 // launch shape of the path kernel: threads per CTA, limited by the shared memory
 // of the per-thread Chebyshev tables, and paths per thread.  The dense
 // evaluations (tree: degree of the prefix tree, else 0):
-// * FP64: 128 threads (64 for M <= 64), one round: its code is several times the
+// * FP64: 128 threads (fewer for M <= 64), one round: its code is several times the
 //   instruction cache and warps that start together share the fetches (d = 10,
 //   n = 1000, M = 2000, N = 20: 64 threads and 4 rounds 16.97 ms, 128 and 4 16.13,
 //   128 and 1 13.87; d = 5 degree 4 3.43 -> 3.12, d = 3 1.93 -> 1.85);
@@ -236,16 +236,18 @@ int Problem::choose_launch(int d, int n, int p, int eta, int N, int M, bool mx, 
   tpb = mx ? 128 : 64;
   while (tpb > 32 && paths_smem_bytes(d, p, eta, N, tpb, mx, dense) > 220 * 1024) tpb >>= 1;
   if (paths_smem_bytes(d, p, eta, N, tpb, mx, dense) > 220 * 1024) return BSDE_ERR_INVALID_ARG;
+  while (tpb > 32 && tpb / 2 >= M) tpb >>= 1;
   if (!dense) {
-    // about 512 paths per CTA, fewer for small M
-    ppt = 4;
+    // FP32: about 512 paths per CTA, fewer for small M; FP64: one round (d = 3
+    // degree 5 2.41 -> 2.21 ms)
+    ppt = mx ? 4 : 1;
     while (ppt > 1 && (long long)tpb * ppt > 2LL * M) ppt >>= 1;
     return BSDE_OK;
   }
   if (!mx) {
-    tpb = M > 64 ? 128 : 64;
     ppt = 1;
-    return paths_smem_bytes(d, p, eta, N, tpb, mx, dense) > 220 * 1024 ? BSDE_ERR_INVALID_ARG : BSDE_OK;
+    if (M > 64 && paths_smem_bytes(d, p, eta, N, 128, mx, dense) <= 220 * 1024) tpb = 128;
+    return BSDE_OK;
   }
   const bool big = tree && d <= 5 && p > 600;
   if (big && 4LL * ((M + 255) / 256 * 256) <= 5LL * M &&
@@ -345,6 +347,7 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
       return BSDE_ERR_INVALID_ARG;
     }
     eta_used = mdeg;
+    build_eval_program(nus, prog);
     coeffs_valid = false;
     // monomial (dense) evaluation: Horner loops for total degree <= 3 (any
     // d) or 4 (d <= 5); with FP32 paths, the prefix-tree recursion for
@@ -494,6 +497,7 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
     P.rhs = (double*)take((size_t)p * 8 * 4);
     P.delta = P.rhs + p;
     P.res = P.rhs + 2 * p;
+    P.prog = (uint2*)(P.rhs + 3 * p);
     P.v = (double*)take((size_t)(n > p ? n : p) * 8);
     P.alpha = (double*)take((size_t)p * 8);
     P.alpha32 = (float*)take((size_t)p * 4);
@@ -572,6 +576,8 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
   // tables, read-out point, key
   cudaError_t e = cudaMemcpyAsync(dev.pairs, pairs.data(), (size_t)p * 8, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(dev.nnz, nnz.data(), (size_t)p, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess && !dev.dense)
+    e = cudaMemcpyAsync(dev.prog, prog.data(), (size_t)p * 8, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && dev.dense) {
     e = cudaMemcpyAsync(dev.conv_row, conv_row.data(), conv_row.size() * 4, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)

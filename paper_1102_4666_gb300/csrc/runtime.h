@@ -39,6 +39,7 @@ class Problem {
   Shape shape;
   ProblemDev dev;
   std::vector<uint32_t> pairs;
+  std::vector<uint32_t> prog;  // the basis as a tree (build_eval_program)
   std::vector<uint8_t> nnz;
   std::vector<std::vector<int>> nus;
   int eta_used = 0;  // largest single-variate degree present
