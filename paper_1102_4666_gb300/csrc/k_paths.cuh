@@ -30,6 +30,8 @@
 // CTA reduces them by a fixed warp-shuffle tree into partial[i][chunk], so
 // the result does not depend on scheduling.
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace paths {
@@ -1315,6 +1317,10 @@ __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
     // is over the lanes that reach a copy together, and a lane whose copy is
     // due always votes for itself, so it is never skipped
     constexpr bool VOTE = copy_vote(EV, D) && !XCOPY;
+    // one predicated store a step into the slot that s asks for, instead of one
+    // before and one after it, where a step is a whole group (d = 4 degree 4 2.27 ->
+    // 2.21 ms a launch, d = 8 degree 3 4.34 -> 4.32; d = 6 loses 2 %)
+    constexpr bool MERGED = G == 1;
     constexpr bool REBUILD = sizeof(R) == 4 && VOTE;
     const int g_hit = sstar - sstar % G;  // first step of the group that contains s*
     constexpr bool ZSUM = sizeof(R) == 8 && VK == VK_CONST;  // states are sums of normals
@@ -1334,52 +1340,71 @@ __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
         euler_path_f64<VK, CC, true>(a, tab, s_ph, pz, bmk, nhh, h, sstar, X, Xs, Xn);
       else
         euler_path_f64<VK, CC, false>(a, tab, s_ph, pz, bmk, nhh, h, sstar, X, Xs, Xn);
-    } else
-    for (int s0 = 0; s0 < a.N; s0 += G) {
-      R z[G * D];  // normals of G steps, scaled by sqrt(h)
-      const uint32_t blk0 = (uint32_t)(s0 / G) * (uint32_t)NB;
+    } else {
+      if constexpr (XCOPY && MERGED) store_state<D>(s_xc + tid, tpb, X);
+      auto group = [&](int s0, auto tail) {
+        R z[G * D];  // normals of G steps, scaled by sqrt(h)
+        const uint32_t blk0 = (uint32_t)(s0 / G) * (uint32_t)NB;
 #pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        const uint4 o = philox_tab(a, pz, s_ph[blk0 + b]);
-        Math<R>::box_muller(o.x, o.y, z[4 * b + 0], z[4 * b + 1], bmk);
-        Math<R>::box_muller(o.z, o.w, z[4 * b + 2], z[4 * b + 3], bmk);
-      }
-      if constexpr (REBUILD) {
-        const bool hit = (s0 == g_hit);
-        const bool any_hit = VOTE ? __any_sync(__activemask(), hit) : true;
-        if (any_hit) {
-#pragma unroll
-          for (int j = 0; j < D; ++j)
-            if (hit) Xg[j] = X[j];
+        for (int b = 0; b < NB; ++b) {
+          const uint4 o = philox_tab(a, pz, s_ph[blk0 + b]);
+          Math<R>::box_muller(o.x, o.y, z[4 * b + 0], z[4 * b + 1], bmk);
+          Math<R>::box_muller(o.z, o.w, z[4 * b + 2], z[4 * b + 3], bmk);
         }
-      }
+        if constexpr (REBUILD) {
+          const bool hit = (s0 == g_hit);
+          const bool any_hit = VOTE ? __any_sync(__activemask(), hit) : true;
+          if (any_hit) {
 #pragma unroll
-      for (int gs = 0; gs < G; ++gs) {
-        const int s = s0 + gs;
-        if (s < a.N) {
-          if constexpr (REBUILD) {
-            euler_step<VK, CC, G>(a, tab + s * a.tab_stride, z, gs, nhh, h, X);
-          } else if constexpr (XCOPY) {
-            const bool hit = (s == sstar);
-            if (hit) store_state<D>(s_xc + tid, tpb, X);
-            euler_step<VK, CC, G>(a, tab + s * a.tab_stride, z, gs, nhh, h, X);
-            if (hit) store_state<D>(s_xc + (size_t)NQ * tpb + tid, tpb, X);
-          } else {
-            const bool hit = (s == sstar);
-            const bool any_hit = VOTE ? __any_sync(__activemask(), hit) : true;
-            if (any_hit) {
+            for (int j = 0; j < D; ++j)
+              if (hit) Xg[j] = X[j];
+          }
+        }
 #pragma unroll
-              for (int j = 0; j < D; ++j)
-                if (hit) Xs[j] = X[j];
-            }
-            euler_step<VK, CC, G>(a, tab + s * a.tab_stride, z, gs, nhh, h, X);
-            if (any_hit) {
+        for (int gs = 0; gs < G; ++gs) {
+          const int s = s0 + gs;
+          if (!decltype(tail)::value || s < a.N) {
+            if constexpr (REBUILD) {
+              euler_step<VK, CC, G>(a, tab + s * a.tab_stride, z, gs, nhh, h, X);
+            } else if constexpr (XCOPY) {
+              if constexpr (MERGED) {
+                euler_step<VK, CC, G>(a, tab + s * a.tab_stride, z, gs, nhh, h, X);
+                const unsigned rel = (unsigned)(s - sstar + 1);
+                if (rel <= 1u) store_state<D>(s_xc + (rel ? NQ * tpb : 0) + tid, tpb, X);
+              } else {
+                const bool hit = (s == sstar);
+                if (hit) store_state<D>(s_xc + tid, tpb, X);
+                euler_step<VK, CC, G>(a, tab + s * a.tab_stride, z, gs, nhh, h, X);
+                if (hit) store_state<D>(s_xc + (size_t)NQ * tpb + tid, tpb, X);
+              }
+            } else {
+              const bool hit = (s == sstar);
+              const bool any_hit = VOTE ? __any_sync(__activemask(), hit) : true;
+              if (any_hit) {
 #pragma unroll
-              for (int j = 0; j < D; ++j)
-                if (hit) Xn[j] = X[j];
+                for (int j = 0; j < D; ++j)
+                  if (hit) Xs[j] = X[j];
+              }
+              euler_step<VK, CC, G>(a, tab + s * a.tab_stride, z, gs, nhh, h, X);
+              if (any_hit) {
+#pragma unroll
+                for (int j = 0; j < D; ++j)
+                  if (hit) Xn[j] = X[j];
+              }
             }
           }
         }
+      };
+      // whole groups without a test per step; the last, partial one is a second
+      // copy of the code, which pays up to 28 normals a group (d = 5 degree 4 3.26 ->
+      // 3.24 ms a launch, d = 6 0.854 -> 0.843, d = 1 0.170 -> 0.162, d = 4 full
+      // correlation 0.214 -> 0.205; d = 9, 36 normals: 5.31 -> 5.67 with it)
+      if constexpr (G * D <= 28) {
+        const int full = G > 1 ? a.N - a.N % G : a.N;
+        for (int s0 = 0; s0 < full; s0 += G) group(s0, std::false_type{});
+        if (G > 1 && full < a.N) group(full, std::true_type{});
+      } else {
+        for (int s0 = 0; s0 < a.N; s0 += G) group(s0, std::true_type{});
       }
     }
 
