@@ -349,9 +349,9 @@ int bsde_eval_price_delta(bsde_ctx* c, int q, const double* t, const double* S, 
     if (!set_device(c)) return fail(c, BSDE_ERR_CUDA, "eval: cudaSetDevice failed");
     const int d = P.model.d;
     // the logarithms and the division by S are the kernel's
-    bool positive = true;
-    for (size_t e = 0; e < (size_t)q * d; ++e) positive = positive && S[e] > 0.0;
-    if (!positive) return fail(c, BSDE_ERR_INVALID_ARG, "eval: prices must be positive");
+    int bad = 0;  // no early exit, so that the loop vectorises
+    for (size_t e = 0; e < (size_t)q * d; ++e) bad |= S[e] > 0.0 ? 0 : 1;
+    if (bad) return fail(c, BSDE_ERR_INVALID_ARG, "eval: prices must be positive");
     const size_t bytes = (size_t)q * 8 * (2 + 2 * d);
     double* buf = (double*)c->al.get(bytes, c->stream);
     if (!buf) return fail(c, BSDE_ERR_NOMEM, "eval: device allocation failed");

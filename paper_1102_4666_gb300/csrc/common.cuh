@@ -265,8 +265,8 @@ struct ProblemDev {
 #define ST_BADARG 4
 
 // launchers (one translation unit each)
-// the points of iteration k and their basis matrix (split: with the operands of
-// the tensor-core Gram matrix)
+// the points of iteration k and their basis matrix (split: only the operands of
+// the tensor-core Gram matrix instead)
 void launch_basis(const ModelHost& m, const GridHost& g, const ProblemDev& P, uint32_t k, bool split,
                   cudaStream_t st);
 // path kernel: returns cudaSuccess or the launch error
@@ -275,6 +275,9 @@ cudaError_t launch_paths(const ModelHost& m, const GridHost& g, const ProblemDev
 void launch_reduce_c(const ProblemDev& P, int M, cudaStream_t st);
 void launch_gram_f64(const ProblemDev& P, cudaStream_t st);
 cudaError_t launch_gram_tc(const ProblemDev& P, cudaStream_t st);
+int gram_fused_batch(int d, int p, int eta);
+cudaError_t launch_gram_fused(const ModelHost& m, const GridHost& g, const ProblemDev& P, uint32_t k0,
+                              uint32_t kstep, int nb, double* A, cudaStream_t st);
 // K splits of the tensor-core Gram (want > 0: that many, capped by the
 // K-blocks; 0: one wave of the device's SMs) and the bytes of its partial tiles
 int gram_tc_splits(int p_pad, int n_pad, int want);

@@ -25,7 +25,7 @@
 // kernel, so the result is deterministic.
 #include <cuda.h>
 
-#include "common.cuh"
+#include "basis.cuh"
 
 namespace {
 
@@ -307,6 +307,143 @@ __global__ void k_gram_reduce(int p, int ntile_side, int splits, const float* pa
   A[(size_t)l2 * p + l1] = s;
 }
 
+// The Gram matrices of several iterations in one launch, for bases of one tile
+// (p <= 128): CTA (split, iteration) draws its points, forms their basis values
+// and stores the TF32 operands straight into shared memory in the swizzled
+// layout of the descriptors, so that neither the operands nor the points pass
+// through memory and an iteration costs no launches of its own.  The same
+// products in the same order as k_basis with k_gram_tc.  Only the p x p
+// corner of the accumulator is stored.  Ten iterations at p = 35, n = 2000: three
+// launches each took 0.13 ms of a 1.67 ms solve more than the two launches now.
+struct FusedArgs {
+  int n, p, dp, eta, splits, kblocks;
+  uint32_t k0, kstep;  // iteration of matrix z: k0 + z kstep
+  const uint2* pairs;
+  const uint8_t* nnz;
+  const uint32_t* key;
+  float* part;  // [iteration][split][p][p]
+  int* status;
+  BoxArgs box;
+};
+
+__global__ void __launch_bounds__(128) k_gram_fused(const __grid_constant__ FusedArgs fa) {
+  pdl_begin();
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* base = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  double* cheb = reinterpret_cast<double*>(base + 2 * TILE_BYTES);
+  __shared__ uint64_t s_bar;
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_ok;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int split = blockIdx.x, z = blockIdx.y;
+  const int kb0 = (int)(((long long)split * fa.kblocks) / fa.splits);
+  const int kb1 = (int)(((long long)(split + 1) * fa.kblocks) / fa.splits);
+  const uint32_t bar = smem_u32(&s_bar);
+  if (tid == 0) {
+    s_ok = 1;
+    mbar_init(bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&s_tmem)),
+                 "r"(TILE));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  // rows past the basis stay zero
+  for (int q = fa.p * (KBLK / 4) + tid; q < TILE * (KBLK / 4); q += 128) {
+    reinterpret_cast<float4*>(base)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    reinterpret_cast<float4*>(base + TILE_BYTES)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = s_tmem;
+  const uint32_t op_hi = smem_u32(base), op_lo = op_hi + TILE_BYTES;
+  for (int kb = kb0; kb < kb1; ++kb) {
+    const int i0 = kb * KBLK, i = i0 + lane;
+    basis_tables(fa.n, i0, fa.dp, fa.eta, fa.key, fa.k0 + (uint32_t)z * fa.kstep, fa.box, cheb,
+                 [](int, int, double) {});
+    if (kb > kb0) {
+      // the operands of the block before have been read (issued work: the wait ends)
+      if (tid == 0 && !mbar_wait(bar, (uint32_t)((kb - kb0 - 1) & 1), DRAIN_LIMIT)) s_ok = 0;
+      __syncthreads();
+    }
+    for (int l = warp; l < fa.p; l += 4) {
+      const float b32 = i < fa.n ? __double2float_rn(basis_at(fa.pairs[l], fa.nnz[l], fa.eta, cheb)) : 0.f;
+      const float hi = to_tf32(b32);
+      // 128-byte rows, their 16-byte chunks permuted by the row within its atom of 8
+      const int off = l * 128 + ((((lane >> 2) ^ (l & 7)) << 4) | ((lane & 3) << 2));
+      *reinterpret_cast<float*>(base + off) = hi;
+      *reinterpret_cast<float*>(base + TILE_BYTES + off) = to_tf32(b32 - hi);
+    }
+    // the stores are visible to the tensor core's reads
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    if (tid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int kk = 0; kk < KBLK / 8; ++kk) {
+        const uint32_t off = kk * 32;  // 8 tf32 = 32 bytes along K
+        mma_tf32(tmem, sdesc(op_hi + off), sdesc(op_hi + off), kb > kb0 || kk > 0);
+        mma_tf32(tmem, sdesc(op_hi + off), sdesc(op_lo + off), 1);
+        mma_tf32(tmem, sdesc(op_lo + off), sdesc(op_hi + off), 1);
+      }
+      mma_commit(bar);
+    }
+  }
+  if (tid == 0 && !mbar_wait(bar, (uint32_t)((kb1 - kb0 - 1) & 1), DRAIN_LIMIT)) s_ok = 0;
+  __syncthreads();
+  const bool ok = s_ok != 0;
+  if (tid == 0 && !ok) atomicOr(fa.status, ST_TIMEOUT);
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const int row = warp * 32 + lane;
+  float* dst = fa.part + (((size_t)z * fa.splits + split) * fa.p + row) * fa.p;
+  for (int c0 = 0; c0 < fa.p; c0 += 8) {
+    uint32_t r[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+    if (ok) {  // CTA-uniform: tcgen05.ld is a warp-collective instruction
+      const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                   : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                     "=r"(r[6]), "=r"(r[7])
+                   : "r"(taddr));
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    }
+    if (row < fa.p)
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+        if (c0 + c < fa.p) dst[c0 + c] = __uint_as_float(r[c]);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TILE));
+  }
+}
+
+// A_z = the FP64 sum over the splits, in their order; both triangles from the upper one
+__global__ void k_gram_fused_reduce(int p, int splits, const float* part, double* A) {
+  pdl_begin();
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  const size_t z = blockIdx.y, pp = (size_t)p * p;
+  const int l1 = e / p, l2 = e - l1 * p;
+  if (l1 >= p || l1 > l2) return;
+  const float* src = part + z * splits * pp + e;
+  double s = 0.0;
+  int q = 0;
+  for (; q + 8 <= splits; q += 8) {
+    float f[8];
+#pragma unroll
+    for (int h = 0; h < 8; ++h) f[h] = src[(size_t)(q + h) * pp];
+#pragma unroll
+    for (int h = 0; h < 8; ++h) s += to_f64(f[h]);
+  }
+  for (; q < splits; ++q) s += to_f64(src[(size_t)q * pp]);
+  A[z * pp + (size_t)l1 * p + l2] = s;
+  A[z * pp + (size_t)l2 * p + l1] = s;
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
                                   const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -380,4 +517,49 @@ cudaError_t launch_gram_tc(const ProblemDev& P, cudaStream_t st) {
   dim3 grid(TILE * TILE / 256, tiles);
   launch_pdl(k_gram_reduce, grid, 256, 0, st, P.p, ga.ntile_side, ga.splits, P.gram_part, P.A);
   return cudaGetLastError();
+}
+
+// matrices per launch of the fused kernel: as many as the partial tiles' buffer
+// (one 128 x 128 tile per split) holds as p x p corners; 0 when the basis has
+// more than one tile or its Chebyshev tables are too large for four CTAs per SM
+int gram_fused_batch(int d, int p, int eta) {
+  const size_t cheb = (size_t)(d + 1) * ((eta < 1 ? 1 : eta) + 1) * BASIS_PTS * sizeof(double);
+  if (p > TILE || cheb > 20 * 1024) return 0;
+  const int g = TILE * TILE / (p * p);
+  return g < 1024 ? g : 1024;
+}
+
+// the Gram matrices of the iterations k0 .. k0 + nb - 1 (kstep 0: of k0) into A
+cudaError_t launch_gram_fused(const ModelHost& m, const GridHost& g, const ProblemDev& P, uint32_t k0,
+                              uint32_t kstep, int nb, double* A, cudaStream_t st) {
+  const int batch = gram_fused_batch(m.d, P.p, P.eta);
+  if (batch < 1 || P.n_pad % KBLK != 0 || !P.gram_part) return cudaErrorInvalidValue;
+  FusedArgs fa;
+  fa.n = P.n;
+  fa.p = P.p;
+  fa.dp = m.d + 1;
+  fa.eta = P.eta < 1 ? 1 : P.eta;
+  fa.splits = P.gram_splits > 0 ? P.gram_splits : gram_tc_splits(P.p_pad, P.n_pad, 0);
+  fa.kblocks = P.n_pad / KBLK;
+  fa.kstep = kstep;
+  fa.pairs = P.pairs;
+  fa.nnz = P.nnz;
+  fa.key = P.key;
+  fa.part = P.gram_part;
+  fa.status = P.status;
+  fa.box = box_args(m, g);
+  // at least 55 KB: four CTAs per SM, whose accumulators fill the tensor memory
+  size_t smem = 1024 + 2 * (size_t)TILE_BYTES + (size_t)fa.dp * (fa.eta + 1) * BASIS_PTS * sizeof(double);
+  if (smem < 55 * 1024) smem = 55 * 1024;
+  cudaError_t e =
+      cudaFuncSetAttribute(k_gram_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  for (int z = 0; z < nb && e == cudaSuccess; z += batch) {
+    const int c = nb - z < batch ? nb - z : batch;
+    fa.k0 = k0 + (uint32_t)z * kstep;
+    e = launch_pdl(k_gram_fused, dim3(fa.splits, c), 128, smem, st, fa);
+    if (e == cudaSuccess)
+      e = launch_pdl(k_gram_fused_reduce, dim3((P.p * P.p + 255) / 256, c), 256, 0, st, P.p, fa.splits,
+                     P.gram_part, A + (size_t)z * P.p * P.p);
+  }
+  return e;
 }

@@ -620,7 +620,16 @@ static void record(cudaEvent_t e, cudaStream_t st) {
 // the stored inverse plus FP64 refinement.
 int Problem::enqueue_factors(int k0, int nb, cudaStream_t st) {
   const size_t pp = (size_t)shape.p * shape.p;
-  for (int j = 0; j < nb; ++j) {
+  const bool fused = mixed && gram_fused_batch(model.d, shape.p, shape.eta) > 0;
+  if (fused) {
+    const cudaError_t e = launch_gram_fused(model, grid, dev, grid.resample ? (uint32_t)k0 : 0u,
+                                            grid.resample ? 1u : 0u, nb, dev.A, st);
+    if (e != cudaSuccess) {
+      err = std::string("tensor-core Gram launch failed: ") + cudaGetErrorString(e);
+      return BSDE_ERR_CUDA;
+    }
+  }
+  for (int j = 0; j < nb && !fused; ++j) {
     const uint32_t kp = grid.resample ? (uint32_t)(k0 + j) : 0u;
     launch_basis(model, grid, dev, kp, mixed, st);
     ProblemDev Pj = dev;
@@ -645,9 +654,11 @@ int Problem::enqueue_gram(int k, cudaStream_t st) {
     err = "gram: no factor block";
     return BSDE_ERR_STATE;
   }
-  launch_basis(model, grid, dev, grid.resample ? (uint32_t)k : 0u, mixed, st);
+  const uint32_t kp = grid.resample ? (uint32_t)k : 0u;
+  const bool fused = mixed && gram_fused_batch(model.d, shape.p, shape.eta) > 0;
+  if (!fused) launch_basis(model, grid, dev, kp, mixed, st);
   if (mixed) {
-    const cudaError_t e = launch_gram_tc(dev, st);
+    const cudaError_t e = fused ? launch_gram_fused(model, grid, dev, kp, 0u, 1, dev.A, st) : launch_gram_tc(dev, st);
     if (e != cudaSuccess) {
       err = std::string("tensor-core Gram launch failed: ") + cudaGetErrorString(e);
       return BSDE_ERR_CUDA;
@@ -925,7 +936,7 @@ int Problem::finish_report(const bsde_solve_params& prm, cudaStream_t st, bsde_r
     // reduce, refit (QR: init, factorisation, solve; otherwise
     // rhs, inverse product, 3 per refinement step), update with read-out;
     // per factorised Gram matrix points with basis, Gram (+ split-K reduce in
-    // mixed precision); per group save_diag, 3 per panel but the last
+    // mixed precision; fused and batched for one-tile bases); per group save_diag, 3 per panel but the last
     // (diag, trsm, update), the last panel's diag, the batched inverse (2)
     const int panels = (shape.p + 31) / 32;
     const int refine2 = prm.refine_steps >= 0 ? prm.refine_steps : (mixed ? 2 : 1);
@@ -935,8 +946,17 @@ int Problem::finish_report(const bsde_solve_params& prm, cudaStream_t st, bsde_r
       groups = grid.resample ? (prm.K_it + nfact - 1) / nfact : 1;
       mats = grid.resample ? prm.K_it : 1;
     }
+    const int batch = mixed ? gram_fused_batch(model.d, shape.p, shape.eta) : 0;
+    int gram_launches = mats * (1 + (mixed ? 2 : 1));
+    if (batch > 0) {
+      gram_launches = 0;
+      for (int left = mats; left > 0; left -= nfact) {
+        const int c = left < nfact ? left : nfact;
+        gram_launches += 2 * ((c + batch - 1) / batch);
+      }
+    }
     r.kernel_launches = prm.K_it * (1 + (dev.dense ? 1 : 0) + 1 + 1 + refit + 1) +
-                        mats * (1 + (mixed ? 2 : 1)) + groups * (3 * panels - 1 + 2);
+                        gram_launches + groups * (3 * panels - 1 + 2);
     if (prm.timing && (int)events.size() >= 8 * prm.K_it) {
       // paths: ev0..ev1; Gram matrices, factors and inverses built ahead of
       // a group of iterations: ev3..ev7 of the group's first iteration;
