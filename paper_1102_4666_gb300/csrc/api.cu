@@ -282,6 +282,12 @@ int bsde_basis_size(int d, int eta, double q, int* p_out) {
   if (d < 1 || d > BSDE_MAX_D || eta < 0 || eta > 15 || !(q > 0.0) || q > 1.0 || !p_out)
     return BSDE_ERR_INVALID_ARG;
   try {
+    if (q == 1.0) {  // C(d + 1 + eta, eta): no list of them, each product is exact
+      long long c = 1;
+      for (int e = 1; e <= eta; ++e) c = c * (d + 1 + e) / e;
+      *p_out = (int)c;
+      return BSDE_OK;
+    }
     *p_out = (int)build_multi_indices(d + 1, eta, q).size();
     return BSDE_OK;
   } catch (...) {

@@ -196,6 +196,8 @@ int bsde_set_grid_impl(GridHost& g, int d, int n, const double* lo, const double
 Problem::~Problem() {
   destroy_graph();
   for (auto e : events) cudaEventDestroy(e);
+  if (ev0) cudaEventDestroy(ev0);
+  if (ev1) cudaEventDestroy(ev1);
 }
 
 void Problem::destroy_graph() {
@@ -336,10 +338,11 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
     err = "solve: the path kernel is compiled for d = 1..10";
     return BSDE_ERR_INVALID_ARG;
   }
-  // basis (cached per (d, eta, q))
-  const auto nu_new = build_multi_indices(d + 1, prm.eta, prm.q);
-  if (nu_new != nus) {
-    nus = nu_new;
+  // basis, built anew only for another (d, eta, q)
+  if (nus.empty() || d != basis_d || prm.eta != basis_eta || prm.q != basis_q) {
+    basis_d = 0;
+    tables_dirty = true;
+    nus = build_multi_indices(d + 1, prm.eta, prm.q);
     int mdeg = 0;
     if (!pack_multi_indices(nus, pairs, nnz, mdeg)) {
       err = "solve: basis needs more than 8 active variates or a degree above 15";
@@ -369,6 +372,9 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
       pm = -1;
     }
     if (pm < 0) pm = 0;
+    basis_d = d;
+    basis_eta = prm.eta;
+    basis_q = prm.q;
   }
   const int p = (int)nus.size();
   const int n = grid.n;
@@ -527,6 +533,7 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
     }
     dev = P;
     coeffs_valid = false;
+    tables_dirty = true;
     nfact = 0;  // the factor block is laid out for p again below
   }
   // factor block: kept across solves (and across reallocations of the main
@@ -573,33 +580,46 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
     dev.shard_i0 = i0;
     dev.shard_n = i1 - i0;
   }
-  // tables, read-out point, key
-  cudaError_t e = cudaMemcpyAsync(dev.pairs, pairs.data(), (size_t)p * 8, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dev.nnz, nnz.data(), (size_t)p, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && !dev.dense)
-    e = cudaMemcpyAsync(dev.prog, prog.data(), (size_t)p * 8, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && dev.dense) {
-    e = cudaMemcpyAsync(dev.conv_row, conv_row.data(), conv_row.size() * 4, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(dev.conv_l, conv_l.data(), conv_l.size() * 4, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(dev.conv_c, conv_c.data(), conv_c.size() * 8, cudaMemcpyHostToDevice, st);
+  // the basis tables and the read-out point stay in the arena from call to call
+  // and are uploaded when they change; the key and a cleared status every time.
+  // The sources are members: a copy from pageable memory may still be reading
+  // them when this returns (the tables' vectors are waited for, as the next
+  // call may reallocate them).
+  cudaError_t e = cudaSuccess;
+  auto upload = [&](void* dst, const void* src, size_t bytes) {
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+  };
+  bool point = tables_dirty;
+  for (int j = 0; j < d; ++j) {
+    const double v = std::log(model.S0[j]);
+    point = point || v != up_point[j];
+    up_point[j] = v;
   }
-  double logS0[BSDE_DMAX];
-  for (int j = 0; j < d; ++j) logS0[j] = std::log(model.S0[j]);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(dev.out + OUT_SIZE + 1 + BSDE_DMAX, logS0, (size_t)d * 8,
-                        cudaMemcpyHostToDevice, st);
-  uint32_t key[2] = {(uint32_t)(prm.seed & 0xffffffffu), (uint32_t)(prm.seed >> 32)};
-  dev.seed_key[0] = key[0];
-  dev.seed_key[1] = key[1];
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dev.key, key, 8, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(dev.status, 0, sizeof(int), st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // key/logS0 live on this stack
+  if (point) upload(dev.out + OUT_SIZE + 1 + BSDE_DMAX, up_point, (size_t)d * 8);
+  up_key[0] = (uint32_t)(prm.seed & 0xffffffffu);
+  up_key[1] = (uint32_t)(prm.seed >> 32);
+  up_key[2] = up_key[3] = up_key[4] = 0u;  // word 4 is the status
+  dev.seed_key[0] = up_key[0];
+  dev.seed_key[1] = up_key[1];
+  upload(dev.key, up_key, sizeof(up_key));
+  if (tables_dirty) {
+    upload(dev.pairs, pairs.data(), (size_t)p * 8);
+    upload(dev.nnz, nnz.data(), (size_t)p);
+    if (dev.dense) {
+      upload(dev.conv_row, conv_row.data(), conv_row.size() * 4);
+      upload(dev.conv_l, conv_l.data(), conv_l.size() * 4);
+      upload(dev.conv_c, conv_c.data(), conv_c.size() * 8);
+    } else {
+      upload(dev.prog, prog.data(), (size_t)p * 8);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  }
   if (e != cudaSuccess) {
+    tables_dirty = true;
     err = std::string("solve: upload failed: ") + cudaGetErrorString(e);
     return BSDE_ERR_CUDA;
   }
+  tables_dirty = false;
   return BSDE_OK;
 }
 
@@ -876,25 +896,22 @@ int Problem::complete(const bsde_solve_params& prm, cudaStream_t st, cudaEvent_t
 
 int Problem::solve(const bsde_solve_params& prm, Allocator& al, size_t budget, cudaStream_t st,
                    bsde_report* rep) {
-  cudaEvent_t e0, e1;
-  if (cudaEventCreate(&e0) != cudaSuccess) return BSDE_ERR_CUDA;
-  if (cudaEventCreate(&e1) != cudaSuccess) {
-    cudaEventDestroy(e0);
+  if ((!ev0 && cudaEventCreate(&ev0) != cudaSuccess) || (!ev1 && cudaEventCreate(&ev1) != cudaSuccess)) {
+    cudaGetLastError();
+    err = "solve: cudaEventCreate failed";
     return BSDE_ERR_CUDA;
   }
-  int rc = start(prm, al, budget, st, e0, e1);
-  if (rc == BSDE_OK) rc = complete(prm, st, e0, e1, rep);
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  return rc;
+  const int rc = start(prm, al, budget, st, ev0, ev1);
+  return rc == BSDE_OK ? complete(prm, st, ev0, ev1, rep) : rc;
 }
 
 int Problem::finish_report(const bsde_solve_params& prm, cudaStream_t st, bsde_report* rep,
                            float ms_total) {
-  std::vector<double> out(OUT_SIZE);
-  int status = 0, rank = shape.p;
-  cudaError_t e = cudaMemcpyAsync(out.data(), dev.out, OUT_SIZE * 8, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&status, dev.status, sizeof(int), cudaMemcpyDeviceToHost, st);
+  // the status (a word of the key's block) and the report block behind it in one copy
+  const size_t lead = (size_t)((char*)dev.out - (char*)dev.status);
+  std::vector<double> buf((lead + 7) / 8 + OUT_SIZE);
+  int rank = shape.p;
+  cudaError_t e = cudaMemcpyAsync(buf.data(), dev.status, lead + OUT_SIZE * 8, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess && shape.qr)
     e = cudaMemcpyAsync(&rank, dev.qr_rank, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -902,6 +919,9 @@ int Problem::finish_report(const bsde_solve_params& prm, cudaStream_t st, bsde_r
     err = std::string("solve: report copy failed: ") + cudaGetErrorString(e);
     return BSDE_ERR_CUDA;
   }
+  int status = 0;
+  memcpy(&status, buf.data(), sizeof(int));
+  const double* out = reinterpret_cast<const double*>((const char*)buf.data() + lead);
   int rc = BSDE_OK;
   if (status & ST_NOT_PD) {
     err = "solve: the Gram matrix is not positive definite (Cholesky pivot <= 0)";
@@ -990,6 +1010,7 @@ void Problem::release(Allocator& al, cudaStream_t st) {
   fact_bytes = 0;
   nfact = 0;
   dev = ProblemDev();
+  tables_dirty = true;
   alloc_shape = Shape();
   coeffs_valid = false;
 }

@@ -109,6 +109,13 @@ class Problem {
   int nfact = 0;
   // graph of a whole solve
   cudaGraphExec_t gexec = nullptr;
+  cudaEvent_t ev0 = nullptr, ev1 = nullptr;  // around a synchronous solve
+  // (d, eta, q) of `nus`; what prepare() uploads, and whether the arena lacks the tables
+  int basis_d = 0, basis_eta = -1;
+  double basis_q = 0.0;
+  bool tables_dirty = true;
+  double up_point[BSDE_DMAX] = {0};
+  uint32_t up_key[5] = {0};
   std::string graph_key;
   std::vector<cudaEvent_t> events;  // 8 per iteration when timing
   int choose_launch(int d, int n, int p, int eta, int N, int M, bool mixed, bool dense, int tree,
