@@ -295,7 +295,10 @@ cudaError_t launch_eval_points(const ModelHost& m, const GridHost& g, const Prob
 size_t paths_smem_bytes(int d, int p, int eta, int N, int tpb, bool mixed, bool dense);
 void launch_cheb2mono(const ProblemDev& P, cudaStream_t st);
 void launch_qr_solve(const ProblemDev& P, cudaStream_t st);
-void launch_inverse(const ProblemDev& P, int nb, cudaStream_t st);
+void launch_inverse(const ProblemDev& P, int nb, bool full, cudaStream_t st);  // full: A^-1, else M = L^-1 only
+// x (+)= M^T (M b) from the M in A's upper triangle; overwrites P.v
+void launch_factor_solve(const ProblemDev& P, const double* b, double* x, int accumulate,
+                         cudaStream_t st);
 void launch_inv_gemv(const ProblemDev& P, const double* b, double* x, int accumulate, cudaStream_t st);
 int paths_supported_d(int d);
 // peer exchange of a sharded solve: push this rank's block [i0, i0 + count)

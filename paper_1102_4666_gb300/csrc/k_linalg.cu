@@ -285,13 +285,13 @@ __global__ void __launch_bounds__(256) k_chol_update(double* A, int p, int j0) {
 }
 
 // M = L^-1 by block columns, transposed into the upper triangle of A: CTA
-// (strip, z) computes C columns of M from their diagonal block down,
+// (z, strip) computes C columns of M from their diagonal block down,
 //   M_I = -L_II^-1 sum_{K < I} L_IK M_K,
 // keeping the strip in shared memory; warp = column, lane = row.  The strips of
-// the first columns are the longest and start first.  With k_inv_syrk p^3 / 3
-// multiply-adds instead of the 2 p^3 / 3 of p substitutions: ten matrices of
-// p = 924 (the FP64 pipe's time for p^3 / 3: 4.3 ms) with the factorisation
-// 17.1 -> 9.6 ms, twelve of p = 364 3.20 -> 1.89 ms, one of p = 364 1.74 -> 0.73.
+// the first columns are the longest and start first, those of every matrix
+// before the next shorter ones (matrix by matrix the long strips of the last one
+// ended the launch: ten of p = 924 3.3 -> 2.5 ms; p^3 / 6 is 2.1).  p^3 / 6 multiply-adds, with k_inv_syrk
+// p^3 / 3 instead of the 2 p^3 / 3 of p substitutions.
 template <int C>
 __global__ void __launch_bounds__(32 * C) k_tri_inv(double* A, int p,
                                                     const double* dinv) {
@@ -299,10 +299,10 @@ __global__ void __launch_bounds__(32 * C) k_tri_inv(double* A, int p,
   extern __shared__ double Ms[];  // [row][C], rows padded to blocks of 32
   __shared__ double Lt[32][33], Ac[32][C + 1];
   constexpr int PER = 32 / C;  // tile elements per thread
-  const size_t z = blockIdx.y;
+  const size_t z = blockIdx.x;
   A += z * p * p;
   dinv += z * p;
-  const int c0 = blockIdx.x * C, J = c0 >> 5, T = (p + 31) >> 5;
+  const int c0 = blockIdx.y * C, J = c0 >> 5, T = (p + 31) >> 5;
   const int lane = threadIdx.x & 31, col = threadIdx.x >> 5;
   const int cg = c0 + col;
   // element e of the tile (I, K): row (threadIdx.x >> 5) + e C, column lane
@@ -676,6 +676,49 @@ __global__ void k_inv_gemv(int p, const double* Ainv, const double* b,
   if (lane == 0) x[row] = accumulate ? x[row] + s : s;
 }
 
+// The two halves of A^-1 b = M^T (M b), M in the upper triangle of A.  y = M b:
+// CTA of 256 threads for eight entries, thread = (term mod 32, entry), so that a
+// row of A is read in whole sectors and every SM has a part of the p^2 / 2
+// multiply-adds (32 entries per CTA would leave one SM 7 us of them at p = 924).
+__global__ void __launch_bounds__(256) k_m_times(int p, const double* A, const double* dinv,
+                                                 const double* b, double* y) {
+  pdl_begin();
+  __shared__ double ws[8][8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i = blockIdx.x * 8 + (threadIdx.x & 7);
+  double s = 0.0;
+  if (i < p) {
+    const int a0 = threadIdx.x >> 3;
+#pragma unroll 8
+    for (int a = a0; a < i; a += 32) s += A[(size_t)a * p + i] * b[a];
+    if ((i & 31) == a0) s += dinv[i] * b[i];
+  }
+  s += __shfl_xor_sync(0xffffffffu, s, 8);
+  s += __shfl_xor_sync(0xffffffffu, s, 16);
+  if (lane < 8) ws[warp][lane] = s;
+  __syncthreads();
+  if (threadIdx.x < 8 && i < p) {
+    const int c = threadIdx.x;
+    y[i] = ((ws[0][c] + ws[1][c]) + (ws[2][c] + ws[3][c])) + ((ws[4][c] + ws[5][c]) + (ws[6][c] + ws[7][c]));
+  }
+}
+
+// x (+)= M^T y: warp per row, fixed shuffle order
+__global__ void __launch_bounds__(256) k_mt_times(int p, const double* A, const double* dinv,
+                                                  const double* y, double* x, int accumulate) {
+  pdl_begin();
+  const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (row >= p) return;
+  const double* a = A + (size_t)row * p;
+  double s = lane == 0 ? dinv[row] * y[row] : 0.0;
+#pragma unroll 8
+  for (int c = row + 1 + lane; c < p; c += 32) s += a[c] * y[c];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) x[row] = accumulate ? x[row] + s : s;
+}
+
 }  // namespace
 
 template <int C>
@@ -683,13 +726,13 @@ static void launch_tri_inv(const ProblemDev& P, int nb, cudaStream_t st) {
   const size_t smem = (size_t)((P.p + 31) / 32 * 32) * C * sizeof(double);
   if (smem > 32 * 1024)
     cudaFuncSetAttribute(k_tri_inv<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  launch_pdl(k_tri_inv<C>, dim3((P.p + C - 1) / C, nb), 32 * C, smem, st, P.A, P.p, P.dinv);
+  launch_pdl(k_tri_inv<C>, dim3(nb, (P.p + C - 1) / C), 32 * C, smem, st, P.A, P.p, P.dinv);
 }
 
 // strips of 8 columns when there are enough of them for two CTAs per SM (they
 // read the factor half as often as strips of 4) and their p x 8 values fit the
 // shared memory, else of 4, or 1 for the largest bases
-void launch_inverse(const ProblemDev& P, int nb, cudaStream_t st) {
+void launch_inverse(const ProblemDev& P, int nb, bool full, cudaStream_t st) {
   const size_t col = (size_t)((P.p + 31) / 32 * 32) * sizeof(double), room = 208 * 1024;
   if ((long long)((P.p + 7) / 8) * nb >= 2LL * device_sm_count() && 8 * col <= room)
     launch_tri_inv<8>(P, nb, st);
@@ -697,6 +740,7 @@ void launch_inverse(const ProblemDev& P, int nb, cudaStream_t st) {
     launch_tri_inv<4>(P, nb, st);
   else
     launch_tri_inv<1>(P, nb, st);
+  if (!full) return;
   const int T = (P.p + T16 - 1) / T16;
   launch_pdl(k_inv_syrk, dim3(T * (T + 1) / 2, nb), 256, 0, st, P.A, P.p, P.dinv, P.Ainv);
 }
@@ -704,6 +748,12 @@ void launch_inverse(const ProblemDev& P, int nb, cudaStream_t st) {
 void launch_inv_gemv(const ProblemDev& P, const double* b, double* x, int accumulate,
                      cudaStream_t st) {
   launch_pdl(k_inv_gemv, (P.p * 32 + 255) / 256, 256, 0, st, P.p, P.Ainv, b, x, accumulate);
+}
+
+void launch_factor_solve(const ProblemDev& P, const double* b, double* x, int accumulate,
+                         cudaStream_t st) {
+  launch_pdl(k_m_times, (P.p + 7) / 8, 256, 0, st, P.p, P.A, P.dinv, b, P.v);
+  launch_pdl(k_mt_times, (P.p + 7) / 8, 256, 0, st, P.p, P.A, P.dinv, P.v, x, accumulate);
 }
 
 void launch_cheb2mono(const ProblemDev& P, cudaStream_t st) {

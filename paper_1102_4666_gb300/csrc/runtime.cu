@@ -632,13 +632,27 @@ static void record(cudaEvent_t e, cudaStream_t st) {
                            cs == cudaStreamCaptureStatusActive ? cudaEventRecordExternal : cudaEventRecordDefault);
 }
 
+int Problem::refinements(const bsde_solve_params& prm) const {
+  return prm.refine_steps >= 0 ? prm.refine_steps : (mixed ? 2 : 1);
+}
+
+// Whether A^-1 = M^T M is formed, or M^T (M b) applied as two products.  Forming it
+// is p^3 / 6 multiply-adds, 0.6 of them per ps, for each matrix; a second product
+// costs 4 us (its launch, mostly) each time the matrix is used, so with three uses
+// the line is at p = 378.  Ten matrices of p = 924: 2.3 ms for A^-1; the solve as a
+// whole 32.7 -> 29.4 ms with the other order of k_tri_inv's strips.  With fixed points one matrix serves every
+// iteration, however a user splits them into calls.
+bool Problem::full_inverse(const bsde_solve_params& prm) const {
+  return !grid.resample || (double)shape.p * shape.p * shape.p < (1.0 + refinements(prm)) * 18e6;
+}
+
 // The Gram matrix of iteration k depends only on the points of iteration k,
 // which depend only on (seed, k): the matrices of a group of iterations are
 // built and factorised together before the group's path kernels, batched
 // over the group (blockIdx.y of the factorisation kernels).  The path kernel
 // then runs alone on the device, and the refit after it is a product with
 // the stored inverse plus FP64 refinement.
-int Problem::enqueue_factors(int k0, int nb, cudaStream_t st) {
+int Problem::enqueue_factors(const bsde_solve_params& prm, int k0, int nb, cudaStream_t st) {
   const size_t pp = (size_t)shape.p * shape.p;
   const bool fused = mixed && gram_fused_batch(model.d, shape.p, shape.eta) > 0;
   if (fused) {
@@ -665,7 +679,7 @@ int Problem::enqueue_factors(int k0, int nb, cudaStream_t st) {
     }
   }
   launch_cholesky(dev, nb, st);
-  launch_inverse(dev, nb, st);
+  launch_inverse(dev, nb, full_inverse(prm), st);
   return BSDE_OK;
 }
 
@@ -763,14 +777,16 @@ int Problem::enqueue_iteration(const bsde_solve_params& prm, int k, cudaStream_t
     launch_qr_solve(dev, st);
   } else {
     ProblemDev Ps = dev;
+    Ps.A = dev.A + (size_t)slot * shape.p * shape.p;
     Ps.Ainv = dev.Ainv + (size_t)slot * shape.p * shape.p;
+    Ps.dinv = dev.dinv + (size_t)slot * shape.p;
+    const auto apply = full_inverse(prm) ? launch_inv_gemv : launch_factor_solve;
     launch_rhs(dev, st);
     if (rec) record(ev[4], st);
-    launch_inv_gemv(Ps, dev.rhs, dev.delta, 0, st);
-    const int refine = prm.refine_steps >= 0 ? prm.refine_steps : (mixed ? 2 : 1);
-    for (int r = 0; r < refine; ++r) {
+    apply(Ps, dev.rhs, dev.delta, 0, st);
+    for (int r = 0; r < refinements(prm); ++r) {
       launch_refine_residual(dev, st);
-      launch_inv_gemv(Ps, dev.res, dev.delta, 1, st);
+      apply(Ps, dev.res, dev.delta, 1, st);
     }
   }
   if (rec) record(ev[5], st);
@@ -801,7 +817,7 @@ int Problem::enqueue_block(const bsde_solve_params& prm, int k0, int count, cuda
       // iteration (zero for the others); the QR refit records its own
       if (!shape.qr && e) record(e[3], st);
       if (!shape.qr && j == 0 && (grid.resample || it == 0)) {
-        const int rc = enqueue_factors(k0 + it, grid.resample ? g : 1, st);
+        const int rc = enqueue_factors(prm, k0 + it, grid.resample ? g : 1, st);
         if (rc != BSDE_OK) return rc;
       }
       if (!shape.qr && e) {
@@ -957,10 +973,11 @@ int Problem::finish_report(const bsde_solve_params& prm, cudaStream_t st, bsde_r
     // rhs, inverse product, 3 per refinement step), update with read-out;
     // per factorised Gram matrix points with basis, Gram (+ split-K reduce in
     // mixed precision; fused and batched for one-tile bases); per group save_diag, 3 per panel but the last
-    // (diag, trsm, update), the last panel's diag, the batched inverse (2)
+    // (diag, trsm, update), the last panel's diag, the batched inverse (2; one
+    // where its second factor is applied in each solve instead)
     const int panels = (shape.p + 31) / 32;
-    const int refine2 = prm.refine_steps >= 0 ? prm.refine_steps : (mixed ? 2 : 1);
-    const int refit = shape.qr ? 3 : (2 + 3 * refine2);
+    const int full = full_inverse(prm) ? 1 : 0, refine2 = refinements(prm);
+    const int refit = shape.qr ? 3 : (2 + 3 * refine2 + (1 - full) * (1 + refine2));
     int groups = 0, mats = 0;
     if (!shape.qr) {
       groups = grid.resample ? (prm.K_it + nfact - 1) / nfact : 1;
@@ -976,7 +993,7 @@ int Problem::finish_report(const bsde_solve_params& prm, cudaStream_t st, bsde_r
       }
     }
     r.kernel_launches = prm.K_it * (1 + (dev.dense ? 1 : 0) + 1 + 1 + refit + 1) +
-                        gram_launches + groups * (3 * panels - 1 + 2);
+                        gram_launches + groups * (3 * panels - 1 + 1 + full);
     if (prm.timing && (int)events.size() >= 8 * prm.K_it) {
       // paths: ev0..ev1; Gram matrices, factors and inverses built ahead of
       // a group of iterations: ev3..ev7 of the group's first iteration;

@@ -123,7 +123,9 @@ class Problem {
   void ensure_events(int count);
   // points, basis and Gram matrix of iterations k0 .. k0 + nb - 1 into the
   // nb slots of the factor block, then their batched factorisation and inverses
-  int enqueue_factors(int k0, int nb, cudaStream_t st);
+  int enqueue_factors(const bsde_solve_params& prm, int k0, int nb, cudaStream_t st);
+  int refinements(const bsde_solve_params& prm) const;
+  bool full_inverse(const bsde_solve_params& prm) const;
   // one iteration k -> k + 1 whose Gram inverse is in slot `slot`
   int enqueue_iteration(const bsde_solve_params& prm, int k, cudaStream_t st, cudaEvent_t* ev,
                         int slot);
