@@ -1395,14 +1395,25 @@ __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
           }
         }
       };
-      // whole groups without a test per step; the last, partial one is a second
-      // copy of the code, which pays up to 28 normals a group (d = 5 degree 4 3.26 ->
-      // 3.24 ms a launch, d = 6 0.854 -> 0.843, d = 1 0.170 -> 0.162, d = 4 full
-      // correlation 0.214 -> 0.205; d = 9, 36 normals: 5.31 -> 5.67 with it)
-      if constexpr (G * D <= 28) {
-        const int full = G > 1 ? a.N - a.N % G : a.N;
+      // Whole groups without a test per step (d = 5 degree 3 2.32 -> 2.22 ms a launch
+      // at N = 49, d = 3 1.41 -> 1.36, d = 1 degree 6 0.170 -> 0.162, d = 4 full
+      // correlation 0.214 -> 0.205).  The last, partial group is a second copy of the
+      // code, which the warps of an SM fetch once a round: where a step is long that
+      // costs what the tests of 25 to 40 steps do (N = 11: d = 5 degree 4 1.00 ->
+      // 1.05, degree 5 1.81 -> 1.89; N = 13: d = 7 1.22 -> 1.34).  So there only where
+      // it paid at N = 50 (d = 5 degree 4 2.48 -> 2.45, d = 3 degree 6 1.81 -> 1.77),
+      // and from 40 steps on.
+      constexpr bool ANY_N = G == 1 || D <= 2 || (EV == EV_DENSE3 && G * D <= 20);
+      constexpr bool LONG_N = (EV == EV_DENSE4 && D == 5) || (EV == EV_TREE6 && D == 3);
+      const int full = G > 1 ? a.N - a.N % G : a.N;
+      if constexpr (ANY_N) {
         for (int s0 = 0; s0 < full; s0 += G) group(s0, std::false_type{});
         if (G > 1 && full < a.N) group(full, std::true_type{});
+      } else if constexpr (LONG_N) {
+        int s0 = 0;
+        if (a.N >= 40)
+          for (; s0 < full; s0 += G) group(s0, std::false_type{});
+        for (; s0 < a.N; s0 += G) group(s0, std::true_type{});
       } else {
         for (int s0 = 0; s0 < a.N; s0 += G) group(s0, std::true_type{});
       }
