@@ -266,9 +266,10 @@ struct ProblemDev {
 
 // launchers (one translation unit each)
 // the points of iteration k and their basis matrix (split: only the operands of
-// the tensor-core Gram matrix instead)
+// the tensor-core Gram matrix instead; early: right after launch_refit, may write
+// them while the refit runs)
 void launch_basis(const ModelHost& m, const GridHost& g, const ProblemDev& P, uint32_t k, bool split,
-                  cudaStream_t st);
+                  bool early, cudaStream_t st);
 // path kernel: returns cudaSuccess or the launch error
 cudaError_t launch_paths(const ModelHost& m, const GridHost& g, const ProblemDev& P, int M, int N,
                          uint32_t k, bool mixed, int tpb, int ppt, cudaStream_t st);
@@ -288,6 +289,10 @@ void launch_rhs(const ProblemDev& P, cudaStream_t st);
 // batched over nb Gram matrices (P.A, P.dinv, P.diag0, P.Ainv hold nb of them)
 void launch_cholesky(const ProblemDev& P, int nb, cudaStream_t st);
 void launch_refine_residual(const ProblemDev& P, cudaStream_t st);
+// small bases: the refit, the update and the next monomial coefficients in one launch
+bool refit_small(int n, int p);
+cudaError_t launch_refit(const ModelHost& m, const GridHost& g, const ProblemDev& P, int M, bool reduce,
+                         int refine, int k, cudaStream_t st);
 void launch_update(const ModelHost& m, const GridHost& g, const ProblemDev& P, int k, cudaStream_t st);
 cudaError_t launch_eval_points(const ModelHost& m, const GridHost& g, const ProblemDev& P, int q,
                                const double* t, const double* S, double* price, double* delta,

@@ -7,7 +7,13 @@
 // with an optional FP64 iterative refinement of the normal equations.
 // Also: the per-point reduction of eq. chat, the coefficient update and the
 // price / delta read-out of Section 5.3.
+#include <atomic>
+
+#include <cooperative_groups.h>
+
 #include "common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -533,6 +539,205 @@ __global__ void __launch_bounds__(256) k_update(const __grid_constant__ EvalArgs
   }
 }
 
+// The whole refit of one iteration for a small basis by one cluster: the mean
+// corrections, B^T c, A^-1, the refinement steps, alpha + delta (CTA 0, with its
+// norms), the read-out (the last CTA) and the monomial coefficients for the next
+// iteration's paths (the others).  CTA r keeps the points [r nl, r nl + nl) of B in
+// shared memory and A^-1 beside them; of a sum over the points every CTA forms its
+// part, which all of them read through distributed shared memory and add in rank
+// order; the p x p products every CTA takes for itself.  The last CTA has no points:
+// it tabulates the basis and its derivatives at the read-out point meanwhile.
+// Bound by latency and the two-lane FP64 pipe: of 21 us at n = 2000, p = 35 the loads
+// take 3, a product with B 1.4 to 2 (five of them), one with A^-1 1.1 and an exchange
+// 1.5 (three of each).
+// Once B is in shared memory the next kernel on the stream may start, so that the
+// next iteration's points and basis are written meanwhile (launch_basis, early).
+constexpr int REFIT_P = 64;
+struct RefitArgs {
+  int n, n_pad, p, nl, ldb, chunks, M, refine, k, pm;
+  const double *B, *Ainv, *partial;
+  double *c, *alpha;
+  float* alpha32;
+  const uint2* pairs;
+  const uint8_t* nnz;
+  const double* logS0;
+  double* out;
+  const int *conv_row, *conv_l;
+  const double* conv_c;
+  double* beta;
+  float* beta32;
+};
+
+__device__ __forceinline__ void copy8_async(double* dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+__global__ void __launch_bounds__(256) k_refit(const __grid_constant__ EvalArgs ea,
+                                               const __grid_constant__ RefitArgs a) {
+  pdl_wait();
+  extern __shared__ double rf[];
+  __shared__ double part[2][REFIT_P], vec[REFIT_P], prod[REFIT_P], delta[REFIT_P], al[REFIT_P];
+  __shared__ double T[EVAL_ROWS * 15], dT[EVAL_ROWS * 15], at[EVAL_ROWS][REFIT_P + 1];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, p = a.p;
+  const int rank = (int)cluster.block_rank(), ranks = (int)cluster.num_blocks();
+  const int i0 = rank * a.nl, cnt = max(0, min(a.nl, a.n - i0));
+  double* As = rf;                      // [c][l], symmetric
+  double* Bs = As + p * p;              // [l][i], rows of odd length
+  double* ys = Bs + (size_t)p * a.ldb;  // at this CTA's points: c, then B delta
+  double* red = ys + a.nl;              // 256
+  double first[4];  // the loads that the sums wait for go first
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    first[q] = tid < cnt && q < a.chunks ? a.partial[(size_t)(i0 + tid) * a.chunks + q] : 0.0;
+  for (int i = tid; i < p * p; i += 256) copy8_async(As + i, a.Ainv + i);
+  for (int l = warp; l < p; l += 8)
+    for (int i = lane; i < cnt; i += 32)
+      copy8_async(Bs + (size_t)l * a.ldb + i, a.B + (size_t)l * a.n_pad + i0 + i);
+  if (tid < p) al[tid] = a.alpha[tid];
+  for (int i = tid; i < cnt; i += 256) {
+    double c;
+    if (a.chunks > 0) {
+      double s = 0.0;
+      for (int q = 0; q < a.chunks; ++q)
+        s += i == tid && q < 4 ? (q == 0 ? first[0] : q == 1 ? first[1] : q == 2 ? first[2] : first[3])
+                               : a.partial[(size_t)(i0 + i) * a.chunks + q];
+      c = s / (double)a.M;
+      a.c[i0 + i] = c;
+    } else {
+      c = a.c[i0 + i];
+    }
+    ys[i] = c;
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  pdl_trigger();
+  if (rank == ranks - 1) {
+    // at[0][l] = B_l and at[j][l] = dB_l / dx_j at (0, log S0)
+    if (warp == 7 && lane <= ea.d)
+      cheb_column(((lane == 0 ? 0.0 : a.logS0[lane - 1]) - ea.ctr[lane]) * ea.sc[lane], ea.eta,
+                  T + lane * ea.eta, dT + lane * ea.eta, 1);
+    for (int i = tid; i < (ea.d + 1) * (REFIT_P + 1); i += 256) at[0][i] = 0.0;
+    __syncthreads();
+    if (tid < p)
+      at[0][tid] = basis_value(a.pairs[tid], a.nnz[tid], ea.eta, T, dT, 1,
+                               [&](int v, double gd) { at[v][tid] = gd * ea.sc[v]; });
+  }
+  // dst[l] = sum_{i < len} m[l sl + i si] x[i], thread = (l, i mod parts): rows of
+  // odd length or columns, so without bank conflicts
+  const int parts = min(8, 256 / p), q = tid / p, l = tid - q * p;
+  auto product = [&](const double* m, int sl, int si, const double* x, int len, double* dst) {
+    if (q < parts) {
+      double s0 = 0.0, s1 = 0.0;
+      int i = q;
+      m += l * sl;
+      for (; i + parts < len; i += 2 * parts) {
+        s0 += m[i * si] * x[i];
+        s1 += m[(i + parts) * si] * x[i + parts];
+      }
+      if (i < len) s0 += m[i * si] * x[i];
+      red[q * p + l] = s0 + s1;
+    }
+    __syncthreads();
+    if (tid < p) {
+      double v[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = e < parts ? red[e * p + tid] : 0.0;
+      dst[tid] = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+    }
+  };
+  double rhs = 0.0;
+  for (int r = 0;; ++r) {
+    // B^T y over the cluster.  The parts' buffer alternates: a CTA may write its
+    // next part while others still read this one
+    product(Bs, a.ldb, 1, ys, cnt, part[r & 1]);
+    cluster.sync();
+    if (tid < p) {
+      double v[16];
+#pragma unroll
+      for (int e = 0; e < 16; ++e) v[e] = e < ranks ? cluster.map_shared_rank(part[r & 1], e)[tid] : 0.0;
+#pragma unroll
+      for (int w = 1; w < 16; w *= 2)
+#pragma unroll
+        for (int e = 0; e < 16; e += 2 * w) v[e] += v[e + w];
+      if (r == 0) rhs = v[0];
+      vec[tid] = r == 0 ? rhs : rhs - v[0];
+    }
+    __syncthreads();
+    if (r == a.refine) break;
+    product(As, 1, p, vec, p, prod);
+    if (tid < p) delta[tid] = r == 0 ? prod[tid] : delta[tid] + prod[tid];
+    __syncthreads();
+    // two threads a point
+    for (int j0 = 0; j0 < cnt; j0 += 128) {
+      const int i = j0 + (tid & 127), h = tid >> 7, half = (p + 1) / 2, l1 = h ? p : half;
+      double s0 = 0.0, s1 = 0.0;
+      if (i < cnt) {
+        int m = h * half;
+        for (; m + 1 < l1; m += 2) {
+          s0 += Bs[m * a.ldb + i] * delta[m];
+          s1 += Bs[(m + 1) * a.ldb + i] * delta[m + 1];
+        }
+        if (m < l1) s0 += Bs[m * a.ldb + i] * delta[m];
+      }
+      red[tid] = s0 + s1;
+      __syncthreads();
+      if (h == 0 && i < cnt) ys[i] = red[tid] + red[tid + 128];
+      __syncthreads();
+    }
+  }
+  auto left = cluster.barrier_arrive();  // no CTA's parts are read after this
+  product(As, 1, p, vec, p, prod);
+  if (tid < p) {
+    const double dl = a.refine == 0 ? prod[tid] : delta[tid] + prod[tid];
+    delta[tid] = dl;
+    al[tid] += dl;
+  }
+  __syncthreads();
+  if (rank == 0) {
+    if (tid < p) {
+      a.alpha[tid] = al[tid];
+      if (a.alpha32) a.alpha32[tid] = (float)al[tid];
+    }
+    if (warp == 7 && a.k >= 0 && a.k < 64) {
+      const double d0 = lane < p ? delta[lane] : 0.0, d1 = lane + 32 < p ? delta[lane + 32] : 0.0;
+      double a2 = d0 * d0 + d1 * d1, ai = fmax(fabs(d0), fabs(d1));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        a2 += __shfl_xor_sync(0xffffffffu, a2, o);
+        ai = fmax(ai, __shfl_xor_sync(0xffffffffu, ai, o));
+      }
+      if (lane == 0) {
+        a.out[OUT_RES2 + a.k] = sqrt(a2);
+        a.out[OUT_RESI + a.k] = ai;
+      }
+    }
+  } else if (rank == ranks - 1) {
+    for (int r = warp; r <= ea.d; r += 8) {
+      double s = (lane < p ? al[lane] * at[r][lane] : 0.0) + (lane + 32 < p ? al[lane + 32] * at[r][lane + 32] : 0.0);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) {
+        if (r > 0) {
+          a.out[OUT_DUDX + r - 1] = s;
+        } else {
+          a.out[OUT_PRICE] = s;
+          if (a.k >= 0 && a.k < 64) a.out[OUT_PRICE_IT + a.k] = s;
+        }
+      }
+    }
+  } else {
+    for (int m = (rank - 1) * 256 + tid; m < a.pm; m += (ranks - 2) * 256) {
+      double s = 0.0;
+      for (int e = a.conv_row[m]; e < a.conv_row[m + 1]; ++e) s += a.conv_c[e] * al[a.conv_l[e]];
+      a.beta[m] = s;
+      a.beta32[m] = (float)s;
+    }
+  }
+  cluster.barrier_wait(std::move(left));
+}
+
 // u and dV/dS (delta may be null) at a few query points, one CTA each
 __global__ void __launch_bounds__(256) k_eval_few(const __grid_constant__ EvalArgs ea,
                                                   const double* alpha, const uint2* pairs,
@@ -812,6 +1017,77 @@ static EvalArgs eval_args(const ModelHost& m, const GridHost& g, const ProblemDe
 void launch_update(const ModelHost& m, const GridHost& g, const ProblemDev& P, int k, cudaStream_t st) {
   launch_pdl(k_update, 1, 256, 0, st, eval_args(m, g, P), k, 0.0, P.alpha, P.alpha32, P.delta, P.pairs, P.nnz,
                               P.out + OUT_SIZE + 1 + BSDE_DMAX, P.out);
+}
+
+// Whether the refit is k_refit's: a small basis whose B fits the cluster's shared
+// memory and is not more than its 16 SMs are worth.  An iteration with hardly any
+// paths as eleven launches and so: n = 200, p = 15 32.7 and 21.1 us, n = 2000, p = 35
+// 49.4 and 39.5, n = 2600, p = 56 (the line) 60.5 and 55.0, n = 20000, p = 6 92.7 and
+// 89.1, n = 37000, p = 3 141 and 145 (the means of that many points).
+constexpr long long REFIT_NP = 150000;
+constexpr int REFIT_SMEM = 203 * 1024;  // of p^2 + (p + 1) nl + ... at eight CTAs
+bool refit_small(int n, int p) { return p <= REFIT_P && n <= 16384 && (long long)n * (p + 1) <= REFIT_NP; }
+
+static cudaLaunchConfig_t refit_config(int n, int p, int ranks, cudaLaunchAttribute* at, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = ranks;
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  const int nl = (n + ranks - 2) / (ranks - 1);  // the last CTA has no points
+  cfg.gridDim = ranks;
+  cfg.blockDim = 256;
+  cfg.dynamicSmemBytes = ((size_t)p * p + (size_t)p * (nl | 1) + nl + 256) * sizeof(double);
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// CTAs of the cluster: sixteen where the device can hold one of the largest
+// admitted size, else the portable eight (asked for once per device)
+static int refit_ranks() {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 8;
+  int r = known[dev].load(std::memory_order_relaxed);
+  if (r == 0) {
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = refit_config((int)(REFIT_NP / (REFIT_P + 1)), REFIT_P, 16, &at, nullptr);
+    int held = 0;
+    r = 8;
+    if (cudaFuncSetAttribute(k_refit, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(k_refit, cudaFuncAttributeMaxDynamicSharedMemorySize, REFIT_SMEM) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&held, k_refit, &cfg) == cudaSuccess && held > 0)
+      r = 16;
+    else
+      cudaGetLastError();
+    known[dev].store(r, std::memory_order_relaxed);
+  }
+  return r;
+}
+
+// c: reduced here from P.partial when reduce is set, else given
+cudaError_t launch_refit(const ModelHost& m, const GridHost& g, const ProblemDev& P, int M, bool reduce,
+                         int refine, int k, cudaStream_t st) {
+  RefitArgs a;
+  memset(&a, 0, sizeof(a));
+  a.n = P.n; a.n_pad = P.n_pad; a.p = P.p;
+  a.chunks = reduce ? P.chunks : 0;
+  a.M = M; a.refine = refine; a.k = k;
+  a.pm = P.dense ? P.pm : 0;
+  a.B = P.B; a.Ainv = P.Ainv; a.partial = P.partial; a.c = P.c;
+  a.alpha = P.alpha; a.alpha32 = P.alpha32; a.pairs = P.pairs; a.nnz = P.nnz;
+  a.logS0 = P.out + OUT_SIZE + 1 + BSDE_DMAX;
+  a.out = P.out;
+  a.conv_row = P.conv_row; a.conv_l = P.conv_l; a.conv_c = P.conv_c;
+  a.beta = P.beta; a.beta32 = P.beta32;
+  const int ranks = refit_ranks();
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t cfg = refit_config(P.n, P.p, ranks, &at, st);
+  a.nl = (P.n + ranks - 2) / (ranks - 1);
+  a.ldb = a.nl | 1;
+  cudaError_t e = cudaFuncSetAttribute(k_refit, cudaFuncAttributeMaxDynamicSharedMemorySize, REFIT_SMEM);
+  return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, k_refit, eval_args(m, g, P), a) : e;
 }
 
 // price and dV/dS (delta may be null) at q points (t, S).  Up to eight points per

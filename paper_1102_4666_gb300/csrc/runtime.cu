@@ -665,7 +665,7 @@ int Problem::enqueue_factors(const bsde_solve_params& prm, int k0, int nb, cudaS
   }
   for (int j = 0; j < nb && !fused; ++j) {
     const uint32_t kp = grid.resample ? (uint32_t)(k0 + j) : 0u;
-    launch_basis(model, grid, dev, kp, mixed, st);
+    launch_basis(model, grid, dev, kp, mixed, false, st);
     ProblemDev Pj = dev;
     Pj.A = dev.A + (size_t)j * pp;
     if (mixed) {
@@ -690,7 +690,7 @@ int Problem::enqueue_gram(int k, cudaStream_t st) {
   }
   const uint32_t kp = grid.resample ? (uint32_t)k : 0u;
   const bool fused = mixed && gram_fused_batch(model.d, shape.p, shape.eta) > 0;
-  if (!fused) launch_basis(model, grid, dev, kp, mixed, st);
+  if (!fused) launch_basis(model, grid, dev, kp, mixed, false, st);
   if (mixed) {
     const cudaError_t e = fused ? launch_gram_fused(model, grid, dev, kp, 0u, 1, dev.A, st) : launch_gram_tc(dev, st);
     if (e != cudaSuccess) {
@@ -708,8 +708,9 @@ int Problem::enqueue_gram(int k, cudaStream_t st) {
   return BSDE_OK;
 }
 
+// follows: nothing was launched since the iteration before it
 int Problem::enqueue_iteration(const bsde_solve_params& prm, int k, cudaStream_t st,
-                               cudaEvent_t* ev, int slot) {
+                               cudaEvent_t* ev, int slot, bool follows) {
   const bool rec = ev != nullptr;
   // peer exchange: this iteration's corrections live in the half of the
   // buffers that belongs to its exchange number
@@ -720,8 +721,10 @@ int Problem::enqueue_iteration(const bsde_solve_params& prm, int k, cudaStream_t
     dev.c = sh_buf + region_off;
   }
   const uint32_t kp = grid.resample ? (uint32_t)k : 0u;
-  launch_basis(model, grid, dev, kp, false, st);  // FP64 B for the refit (no TF32 split)
-  if (dev.dense) launch_cheb2mono(dev, st);
+  const bool one = !shape.qr && refit_small(shape.n, shape.p);  // the refit in one launch
+  // FP64 B for the refit (no TF32 split), while the refit before it still runs
+  launch_basis(model, grid, dev, kp, false, one && follows, st);
+  if (dev.dense && !(one && follows)) launch_cheb2mono(dev, st);
   if (rec) record(ev[0], st);
   cudaError_t e = launch_paths(model, grid, dev, shape.M, shape.N, (uint32_t)k, mixed, shape.tpb,
                                shape.ppt, st);
@@ -730,7 +733,7 @@ int Problem::enqueue_iteration(const bsde_solve_params& prm, int k, cudaStream_t
     return BSDE_ERR_CUDA;
   }
   if (rec) record(ev[1], st);
-  launch_reduce_c(dev, shape.M, st);
+  if (!one || sh_n > 1) launch_reduce_c(dev, shape.M, st);
   if (sh_n > 1) {
     // every rank's block of corrections into the exchange buffer
     e = cudaGetLastError();
@@ -775,6 +778,15 @@ int Problem::enqueue_iteration(const bsde_solve_params& prm, int k, cudaStream_t
     if (rec) record(ev[7], st);
     if (rec) record(ev[4], st);
     launch_qr_solve(dev, st);
+  } else if (one) {
+    ProblemDev Ps = dev;
+    Ps.Ainv = dev.Ainv + (size_t)slot * shape.p * shape.p;
+    if (rec) record(ev[4], st);
+    e = launch_refit(model, grid, Ps, shape.M, sh_n == 1, refinements(prm), k - prm.k_start, st);
+    if (e != cudaSuccess) {
+      err = std::string("refit launch failed: ") + cudaGetErrorString(e);
+      return BSDE_ERR_CUDA;
+    }
   } else {
     ProblemDev Ps = dev;
     Ps.A = dev.A + (size_t)slot * shape.p * shape.p;
@@ -790,7 +802,7 @@ int Problem::enqueue_iteration(const bsde_solve_params& prm, int k, cudaStream_t
     }
   }
   if (rec) record(ev[5], st);
-  launch_update(model, grid, dev, k - prm.k_start, st);
+  if (!one) launch_update(model, grid, dev, k - prm.k_start, st);
   e = cudaGetLastError();
   if (e != cudaSuccess) {
     err = std::string("kernel launch failed: ") + cudaGetErrorString(e);
@@ -824,7 +836,7 @@ int Problem::enqueue_block(const bsde_solve_params& prm, int k0, int count, cuda
         record(e[6], st);
         record(e[7], st);
       }
-      const int rc = enqueue_iteration(prm, k0 + it + j, st, e, grid.resample ? j : 0);
+      const int rc = enqueue_iteration(prm, k0 + it + j, st, e, grid.resample ? j : 0, j > 0);
       if (rc != BSDE_OK) return rc;
     }
     it += g;
@@ -992,7 +1004,12 @@ int Problem::finish_report(const bsde_solve_params& prm, cudaStream_t st, bsde_r
         gram_launches += 2 * ((c + batch - 1) / batch);
       }
     }
-    r.kernel_launches = prm.K_it * (1 + (dev.dense ? 1 : 0) + 1 + 1 + refit + 1) +
+    // small bases: basis, paths, refit an iteration, the conversion once a group
+    const bool one = !shape.qr && refit_small(shape.n, shape.p);
+    const int conv = dev.dense ? 1 : 0;
+    const int iterations = one ? prm.K_it * (3 + (sh_n > 1 ? 1 : 0)) + groups * conv
+                               : prm.K_it * (1 + conv + 1 + 1 + refit + 1);
+    r.kernel_launches = iterations +
                         gram_launches + groups * (3 * panels - 1 + 1 + full);
     if (prm.timing && (int)events.size() >= 8 * prm.K_it) {
       // paths: ev0..ev1; Gram matrices, factors and inverses built ahead of

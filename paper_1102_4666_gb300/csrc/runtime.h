@@ -128,7 +128,8 @@ class Problem {
   bool full_inverse(const bsde_solve_params& prm) const;
   // one iteration k -> k + 1 whose Gram inverse is in slot `slot`
   int enqueue_iteration(const bsde_solve_params& prm, int k, cudaStream_t st, cudaEvent_t* ev,
-                        int slot);
+                        int slot,
+                        bool follows);
 };
 
 int bsde_set_model_impl(ModelHost& m, const bsde_sigma* sigma, double r, const bsde_payoff* payoff,
