@@ -34,14 +34,14 @@ CONFIG = "c4"
 FP32_LANES = 128  # FP32 lanes per SM (sm_103a)
 # DRAM bytes (read + write) of one path-kernel launch per point, from an ncu
 # capture of the same kernel on the d = 10 workload with n = 800 points
-# (146.2 KB read, 0 B written: the partial sums stay in L2), scaled to a
+# (139.0 KB read, 0 B written: the partial sums stay in L2), scaled to a
 # launch over n points (the kernel reads the points and coefficients and
 # writes one partial sum per (point, chunk), both proportional to n).
-PATH_TRAFFIC_BYTES_PER_POINT = (134656.0 + 0.0) / 800.0
+PATH_TRAFFIC_BYTES_PER_POINT = (139008.0 + 0.0) / 800.0
 # instruction issue of the same capture: instructions per path-step and
 # instructions issued per SM cycle (of 4), and the MUFU (XU) pipe's share
-PATH_ISSUE = {"instructions_per_path_step": 251.2, "ipc": 2.44, "ipc_peak": 4.0, "xu_pipe_busy": 0.682,
-              "fma_heavy_pipe_busy": 0.648}
+PATH_ISSUE = {"instructions_per_path_step": 252.1, "ipc": 2.455, "ipc_peak": 4.0, "xu_pipe_busy": 0.684,
+              "fma_heavy_pipe_busy": 0.656}
 
 
 def env_rank():

@@ -19,11 +19,11 @@
 // Brownian bridge.  u^k and its derivatives at (tau, X_tau) and u^k(T, X_T)
 // come from per-thread Chebyshev tables in shared memory (layout
 // [slot][thread], conflict-free), or from the monomial coefficients beta of
-// u^k (converted from the Chebyshev coefficients once per iteration, constant
-// correlation only): Horner loops for total degree <= 3 (EV_DENSE3) and for
-// degree 4 at d <= 5 (EV_DENSE4), a compile-time recursion over the prefix
-// tree of variate multisets for degree 4 at d >= 6 and degrees 5 and 6 at
-// d <= 5 (EV_TREE4..6, FP32 paths); every index is a compile-time constant,
+// u^k (converted from the Chebyshev coefficients once per iteration): Horner
+// loops for total degree <= 3 (EV_DENSE3) and for degree 4 at d <= 5
+// (EV_DENSE4), a compile-time recursion over the prefix tree of variate
+// multisets for degree 4 at d >= 6 and degrees 5 and 6 at d <= 5 (EV_TREE4..6,
+// FP32 paths, constant correlation); every index is a compile-time constant,
 // so u and its derivatives stay in registers.  The warps of a CTA enter the
 // larger of these evaluations together (a barrier before them) to share
 // their instruction fetches.  Per-path samples are accumulated in FP64; the

@@ -105,7 +105,8 @@ extern "C" BSDE_API int bsde_corrections_noalloc(
     const int p = (int)nus.size();
     const bool mixed = precision == BSDE_PREC_MIXED;
     const int eta_t = max_deg < 1 ? 1 : max_deg;
-    // launch shape of the path kernel, as the context runtime chooses it
+    // launch shape of the path kernel: about 512 paths per CTA, which bounds the
+    // partial sums in the static array
     int tpb = mixed ? 128 : 64;
     while (tpb > 32 && paths_smem_bytes(m.d, p, eta_t, N_steps, tpb, mixed, false) > 220 * 1024) tpb >>= 1;
     int ppt = 4;

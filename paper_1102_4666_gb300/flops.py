@@ -77,9 +77,9 @@ def eval_dense3_flops(d):
 
 def path_flops(d, vol="tanh"):
     """FP32 flops and MUFU operations of the once-per-path work besides
-    eval_dense3: the random time, the Brownian bridge to X_tau (general
-    triangular L times the bridge normals, sigma and drift frozen at the
-    step s*), the reduced coordinates of both evaluation points, the two
+    eval_dense3: the random time, the Brownian bridge to X_tau (the
+    correlated bridge normals by the prefix sum of the step, sigma and drift
+    frozen at the step s*), the reduced coordinates of both evaluation points, the two
     basket values, the penalised driver and the sample a_m.  Returns
     (flops, mufu)."""
     nbb = (d + 3) // 4            # Philox blocks of bridge normals
@@ -89,7 +89,7 @@ def path_flops(d, vol="tanh"):
     bb = 3                        # theta (1 - theta) h, then sqrt
     per_asset = 0
     for j in range(d):
-        per_asset += 2 * (j + 1)  # y = sum_{q <= j} L_jq zb_q
+        per_asset += 2 * 2        # y = Ld_j zb_j + pre; pre += Lc_j zb_j
         per_asset += 5 if vol == "tanh" else 0   # sigma at (t_s*, X_s*)
         per_asset += 3            # drift = rd - sig^2 / 2
         per_asset += 6            # Xtau = Xs + theta (Xn - Xs) + sig bb y
