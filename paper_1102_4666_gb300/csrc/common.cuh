@@ -143,15 +143,20 @@ struct Math<double> {
 };
 
 // ---------------------------------------------------------------------------
-// Programmatic dependent launch: an iteration is a chain of some fifteen small
-// kernels around the path kernel, each a few microseconds long with about one
-// more between two of them.  A kernel launched by launch_pdl may be scheduled
-// while the one before it on the stream still runs; pdl_begin, first thing in
-// the kernel, waits until that one has completed and its writes are visible, and
-// then lets the next one be scheduled in turn (after the wait, so that no more
-// than one waits on the SMs).  Every kernel launched this way must call it in
-// every thread before it touches memory; their pointers are not __restrict__, as
-// a read-only load could be moved ahead of the wait.
+// Programmatic dependent launch: the refit is a chain of some ten small kernels,
+// each a few microseconds long with about one more between two of them.  A kernel
+// launched by launch_pdl may be scheduled while the one before it on the stream
+// still runs; pdl_begin, first thing in the kernel, waits until that one has
+// completed and its writes are visible, and then lets the next one be scheduled in
+// turn (after the wait, so that no more than one waits on the SMs).  Every kernel
+// launched this way must call it in every thread before it touches memory; their
+// pointers are not __restrict__, as a read-only load could be moved ahead of the
+// wait.  Only grids of at most a CTA per SM are launched so, and not the Gram and
+// batched factorisation kernels: waiting CTAs in numbers hold up the kernels they wait for
+// (Gram and factors of a solve with everything launched early and without: d = 7,
+// p = 165, ten matrices 1.30 and 0.61 ms, p = 210 1.35 and 0.72, p = 364 2.46 and
+// 1.76, p = 924 7.3 and 6.4; the refits at p = 364 0.54 and 0.50 ms, but p = 66
+// 0.32 and 0.33).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() {
@@ -161,9 +166,10 @@ __device__ __forceinline__ void pdl_begin() {
   pdl_wait();
   pdl_trigger();
 }
+int device_sm_count();
 template <typename... P, typename... A>
-inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                              A&&... args) {
+inline cudaError_t launch_kernel(bool early, void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
+                                 cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -173,8 +179,14 @@ inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t 
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                              A&&... args) {
+  const bool few = (unsigned long long)grid.x * grid.y * grid.z <= (unsigned long long)device_sm_count();
+  return launch_kernel(few, kern, grid, block, smem, st, static_cast<A&&>(args)...);
 }
 
 // ---------------------------------------------------------------------------

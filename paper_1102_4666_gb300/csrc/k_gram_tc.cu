@@ -511,11 +511,11 @@ cudaError_t launch_gram_tc(const ProblemDev& P, cudaStream_t st) {
   cudaError_t e =
       cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  launch_pdl(k_gram_tc, tiles * ga.splits, 128, smem, st, mh, ml, ga);
+  launch_kernel(false, k_gram_tc, tiles * ga.splits, 128, smem, st, mh, ml, ga);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   dim3 grid(TILE * TILE / 256, tiles);
-  launch_pdl(k_gram_reduce, grid, 256, 0, st, P.p, ga.ntile_side, ga.splits, P.gram_part, P.A);
+  launch_kernel(false, k_gram_reduce, grid, 256, 0, st, P.p, ga.ntile_side, ga.splits, P.gram_part, P.A);
   return cudaGetLastError();
 }
 
@@ -556,9 +556,9 @@ cudaError_t launch_gram_fused(const ModelHost& m, const GridHost& g, const Probl
   for (int z = 0; z < nb && e == cudaSuccess; z += batch) {
     const int c = nb - z < batch ? nb - z : batch;
     fa.k0 = k0 + (uint32_t)z * kstep;
-    e = launch_pdl(k_gram_fused, dim3(fa.splits, c), 128, smem, st, fa);
+    e = launch_kernel(false, k_gram_fused, dim3(fa.splits, c), 128, smem, st, fa);
     if (e == cudaSuccess)
-      e = launch_pdl(k_gram_fused_reduce, dim3((P.p * P.p + 255) / 256, c), 256, 0, st, P.p, fa.splits,
+      e = launch_kernel(false, k_gram_fused_reduce, dim3((P.p * P.p + 255) / 256, c), 256, 0, st, P.p, fa.splits,
                      P.gram_part, A + (size_t)z * P.p * P.p);
   }
   return e;

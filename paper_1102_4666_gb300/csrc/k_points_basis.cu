@@ -62,7 +62,7 @@ void launch_basis(const ModelHost& m, const GridHost& g, const ProblemDev& P, ui
   if (gy < 1) gy = 1;
   const int l_per = (P.p + gy - 1) / gy;
   gy = (P.p + l_per - 1) / l_per;
-  launch_pdl(k_basis, dim3(gx, gy), tpb, smem, st, P.n, P.n_pad, P.p, l_per, dp, eta, P.pairs, P.nnz,
+  launch_kernel(early, k_basis, dim3(gx, gy), tpb, smem, st, P.n, P.n_pad, P.p, l_per, dp, eta, P.pairs, P.nnz,
              P.key, k, P.t, P.x, box_args(m, g), P.B, P.Bhi, P.Blo, split ? 1 : 0,
              early ? 1 : 0);
 }
