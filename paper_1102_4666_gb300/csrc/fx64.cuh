@@ -157,13 +157,17 @@ FX_FN uint64_t neg_log(uint32_t w, int& sc) {
 }
 
 // sqrt of A (at 2^58), as S 2^(e - 63), S in [2^62, 2^63]: two Newton steps
-// on exact residuals from an FP32 seed (relative error of the seed up to
-// 2^-21; after the steps 2^-42 and 2^-61)
+// on exact residuals from an FP32 seed.  The seed may be off by 2^-22 (the
+// instruction: 2^-22.9), so that the residual a - s0^2 stays below 2^-20 and its
+// leading 32 bits fit the product; after the steps 2^-42 and 2^-61.  Next to
+// a = 1 a seed rounded up gives s0 = 1, which has no place at 2^32: s0 is held at
+// 1 - 2^-32 then.
 FX_FN uint64_t sqrt58(uint64_t A, int& e) {
   const int e2 = clz(A) & ~1;
   const uint64_t a = A << e2;  // [1/4, 1) at 2^64
   const int32_t rs = f2i(rsqrt_seed(u2f(hi32(a)) * 2.3283064365386963e-10f) * 1073741824.0f);  // at 2^30
-  const uint32_t s0 = mulhi32(hi32(a), (uint32_t)rs) << 2;                                     // at 2^32
+  const uint32_t s30 = mulhi32(hi32(a), (uint32_t)rs);                                         // at 2^30
+  const uint32_t s0 = s30 >= (1u << 30) ? 0xffffffffu : s30 << 2;                              // at 2^32
   const int64_t e0 = (int64_t)(a - wide(s0, s0));
   const uint64_t s1 = ((uint64_t)s0 << 31) + (uint64_t)(swide((int32_t)(e0 >> 13), rs) >> 19);  // at 2^63
   const uint64_t t1 = s1 >> 16;                                                                 // at 2^47
