@@ -141,16 +141,6 @@ __global__ void k_save_diag(const double* A, int p, double* diag0) {
   if (j < p) diag0[z * p + j] = A[z * p * p + (size_t)j * p + j];
 }
 
-// 1 / sqrt(a) for normal positive a: the 20-bit FP64 approximation and one
-// third-order step (relative error below 2^-52), four dependent FP64
-// instructions instead of a square root and a division
-__device__ __forceinline__ double rsqrt_f64(double a) {
-  double r;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-  const double e = fma(-(a * r), r, 1.0);
-  return fma(r * e, fma(0.375, e, 0.5), r);
-}
-
 // Right-looking blocked Cholesky, panel width 32, lower factor in place; the
 // upper triangle of A, no longer needed, takes the transposed inverse of the
 // factor (its diagonal is dinv).
@@ -196,7 +186,7 @@ __global__ void __launch_bounds__(128) k_chol_diag(double* A, int p, int j0,
     // piv > thr and finite, on the bits (no FP64 comparison); thr >= 0
     const long long pb = __double_as_longlong(piv), tb = __shfl_sync(0xffffffffu, thr, c);
     const bool ok = pb > tb && pb < 0x7ff0000000000000ll;
-    const double inv = ok ? rsqrt_f64(piv) : nan("");
+    const double inv = ok ? rsqrt(piv) : nan("");
     const double l = lane > c ? colv * inv : 0.0;
     // the next column first: its owner hands it on
     if (c < 31) {

@@ -79,26 +79,6 @@ __device__ __forceinline__ long long qr_key(double a) {
   return b > 0x7ff0000000000000ll ? -1ll : b;
 }
 
-// 1 / a and sqrt(a) for normal a from the 20-bit FP64 approximations and
-// Newton steps (relative error below 2^-52): a tenth of the instructions of
-// the correctly rounded sequences, whose latency every step would wait for
-__device__ __forceinline__ double qr_rcp(double a) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-  r = fma(r, fma(-a, r, 1.0), r);
-  r = fma(r, fma(-a, r, 1.0), r);
-  return r;
-}
-__device__ __forceinline__ double qr_sqrt(double a) {
-  double r;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-  double s = a * r;
-  const double h = 0.5 * r;
-  s = fma(h, fma(-s, s, a), s);
-  s = fma(h, fma(-s, s, a), s);
-  return s;
-}
-
 // The whole factorisation in one cooperative launch, one CTA per SM at most.
 // CTA b owns the columns b, b + CTAs, ... of W (the right-hand side is column
 // p) and keeps them up to date.  Columns stay where they are; pos[] holds the
@@ -189,14 +169,13 @@ __global__ void __launch_bounds__(QR_THREADS, 1)
       for (int i = j + 1 + tid; i < n; i += QR_THREADS) v[i] = __ldcg(x + i);
     }
     // beta, v_0 = x_0 - beta and 1 / (beta (beta - x_0)), in the two warps that
-    // use them; a column that is zero (to the range of the approximations) is
-    // left as it is
+    // use them; a column of squared norm below 2^-963 is zero and left as it is
     double beta = x0, v0 = 0.0, kap = 0.0;
     if (warp < 2 && !(best >= 0 && best < 0x03c0000000000000ll)) {  // norm >= 2^-963 or NaN
-      const double nx = qr_sqrt(best < 0 ? nan("") : __longlong_as_double(best));
+      const double nx = sqrt(best < 0 ? nan("") : __longlong_as_double(best));
       beta = x0 <= 0.0 ? nx : -nx;
       v0 = x0 - beta;
-      kap = qr_rcp(-beta * v0);
+      kap = -1.0 / (beta * v0);
     }
     // H on the columns of this CTA, two at a time
     int q = 0;
@@ -314,7 +293,7 @@ __global__ void __launch_bounds__(256) k_qr_solve(int n, int n_pad, int p, const
         if (lane < c) tri[c][lane] = cols[c][c0 + lane];
       __syncwarp();
       double w = lane < nb ? work[c0 + lane] : 0.0;
-      const double dg = lane < nb ? qr_rcp(col[c0 + lane]) : 1.0;
+      const double dg = lane < nb ? 1.0 / col[c0 + lane] : 1.0;
       for (int c = nb - 1; c >= 0; --c) {
         if (lane == c) w *= dg;
         const double xc = __shfl_sync(0xffffffffu, w, c);
