@@ -83,7 +83,9 @@ __device__ __forceinline__ long long qr_key(double a) {
 // CTA b owns the columns b, b + CTAs, ... of W (the right-hand side is column
 // p) and keeps them up to date.  Columns stay where they are; pos[] holds the
 // logical order.  Step j:
-//   1. every CTA finds the pivot from the norms in memory; its norm is that of
+//   1. every CTA finds the pivot from the norms in memory (of two sets in turn:
+//      a CTA ahead of the others writes those of step j + 1 while they still
+//      choose from those of step j); its norm is that of
 //      the rows from j on, so beta = -sign(x_0) sqrt(norm) needs no further
 //      pass, and with the reflector left unscaled, v = (x_0 - beta, x_1, ...),
 //      H = I - v v^T / (beta (beta - x_0)), none but the pivot column's load;
@@ -129,10 +131,12 @@ __global__ void __launch_bounds__(QR_THREADS, 1)
   __syncthreads();
   for (int j = 0; j < steps; ++j) {
     // pivot: the largest remaining norm, the first logical column on ties
+    const double* norms = nrm + (j & 1) * p;
+    double* next_norms = nrm + ((j & 1) ^ 1) * p;
     long long best = -1;
     int bi = p;
     for (int l = j + tid; l < p; l += QR_THREADS) {
-      const long long t = qr_key(__ldcg(nrm + pos[l]));
+      const long long t = qr_key(__ldcg(norms + pos[l]));
       if (t > best) {
         best = t;
         bi = l;
@@ -223,8 +227,8 @@ __global__ void __launch_bounds__(QR_THREADS, 1)
       }
       __syncthreads();  // the first sums have been read
       qr_sum2(q0, q1, 1.0, buf);
-      if (tid == 0 && l0 < p) nrm[l0] = q0;
-      if (tid == 0 && m == 2 && l1 < p) nrm[l1] = q1;
+      if (tid == 0 && l0 < p) next_norms[l0] = q0;
+      if (tid == 0 && m == 2 && l1 < p) next_norms[l1] = q1;
       __syncthreads();
     }
     // grid barrier; every wait is bounded
