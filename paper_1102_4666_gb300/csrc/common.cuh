@@ -167,6 +167,18 @@ __device__ __forceinline__ void pdl_begin() {
   pdl_trigger();
 }
 int device_sm_count();
+
+// A kernel's limit of dynamic shared memory is the device's, not a launch's: set to
+// the size of each launch, a thread with a smaller basis could lower it between
+// another thread's call and launch, which was then refused.  So every kernel has
+// one limit, what its largest launch may ask for, known when it is compiled.
+template <int BYTES, typename K>
+inline cudaError_t smem_limit(K kern) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, BYTES);
+}
+constexpr int SMEM_PER_CTA = 227 * 1024;  // static and dynamic together
+constexpr int PATHS_SMEM = 220 * 1024;    // of the path kernels
+
 template <typename... P, typename... A>
 inline cudaError_t launch_kernel(bool early, void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
                                  cudaStream_t st, A&&... args) {

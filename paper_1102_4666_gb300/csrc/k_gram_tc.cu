@@ -507,9 +507,8 @@ cudaError_t launch_gram_tc(const ProblemDev& P, cudaStream_t st) {
   ga.part = P.gram_part;
   ga.status = P.status;
   const int tiles = ga.ntile_side * (ga.ntile_side + 1) / 2;
-  const size_t smem = 1024 + (size_t)STAGES * STAGE_BYTES + 64;
-  cudaError_t e =
-      cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr int smem = 1024 + STAGES * STAGE_BYTES + 64;
+  cudaError_t e = smem_limit<smem>(k_gram_tc);
   if (e != cudaSuccess) return e;
   launch_kernel(false, k_gram_tc, tiles * ga.splits, 128, smem, st, mh, ml, ga);
   e = cudaGetLastError();
@@ -548,11 +547,11 @@ cudaError_t launch_gram_fused(const ModelHost& m, const GridHost& g, const Probl
   fa.part = P.gram_part;
   fa.status = P.status;
   fa.box = box_args(m, g);
-  // at least 55 KB: four CTAs per SM, whose accumulators fill the tensor memory
-  size_t smem = 1024 + 2 * (size_t)TILE_BYTES + (size_t)fa.dp * (fa.eta + 1) * BASIS_PTS * sizeof(double);
-  if (smem < 55 * 1024) smem = 55 * 1024;
-  cudaError_t e =
-      cudaFuncSetAttribute(k_gram_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // operands and tables of at most 20 KB (gram_fused_batch) in 55 KB: four CTAs per SM,
+  // whose accumulators fill the tensor memory
+  constexpr int smem = 55 * 1024;
+  static_assert(1024 + 2 * TILE_BYTES + 20 * 1024 <= smem, "operands and tables");
+  cudaError_t e = smem_limit<smem>(k_gram_fused);
   for (int z = 0; z < nb && e == cudaSuccess; z += batch) {
     const int c = nb - z < batch ? nb - z : batch;
     fa.k0 = k0 + (uint32_t)z * kstep;

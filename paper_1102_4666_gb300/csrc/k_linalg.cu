@@ -923,8 +923,8 @@ static bool factor_early(const ProblemDev& P, int nb) { return nb == 1 && P.p <=
 template <int C>
 static void launch_tri_inv(const ProblemDev& P, int nb, cudaStream_t st) {
   const size_t smem = (size_t)((P.p + 31) / 32 * 32) * C * sizeof(double);
-  if (smem > 32 * 1024)
-    cudaFuncSetAttribute(k_tri_inv<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr int fixed = (32 * 33 + 32 * (C + 1)) * (int)sizeof(double);  // its static part
+  if (smem > 32 * 1024) smem_limit<SMEM_PER_CTA - fixed>(k_tri_inv<C>);
   launch_kernel(factor_early(P, nb), k_tri_inv<C>, dim3(nb, (P.p + C - 1) / C), 32 * C, smem, st, P.A, P.p, P.dinv);
 }
 
@@ -1050,7 +1050,7 @@ static int refit_ranks() {
     int held = 0;
     r = 8;
     if (cudaFuncSetAttribute(k_refit, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-        cudaFuncSetAttribute(k_refit, cudaFuncAttributeMaxDynamicSharedMemorySize, REFIT_SMEM) == cudaSuccess &&
+        smem_limit<REFIT_SMEM>(k_refit) == cudaSuccess &&
         cudaOccupancyMaxActiveClusters(&held, k_refit, &cfg) == cudaSuccess && held > 0)
       r = 16;
     else
@@ -1080,7 +1080,7 @@ cudaError_t launch_refit(const ModelHost& m, const GridHost& g, const ProblemDev
   const cudaLaunchConfig_t cfg = refit_config(P.n, P.p, ranks, &at, st);
   a.nl = (P.n + ranks - 2) / (ranks - 1);
   a.ldb = a.nl | 1;
-  cudaError_t e = cudaFuncSetAttribute(k_refit, cudaFuncAttributeMaxDynamicSharedMemorySize, REFIT_SMEM);
+  cudaError_t e = smem_limit<REFIT_SMEM>(k_refit);
   return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, k_refit, eval_args(m, g, P), a) : e;
 }
 
@@ -1101,8 +1101,8 @@ cudaError_t launch_eval_points(const ModelHost& m, const GridHost& g, const Prob
   int slices = 8;
   while (slices > 1 && (long long)groups * slices > 32LL * device_sm_count()) slices >>= 1;
   const size_t smem = ((size_t)2 * (ea.d + 1) * ea.eta + (size_t)slices * (ea.d + 1)) * 32 * sizeof(double);
-  cudaError_t e =
-      cudaFuncSetAttribute(k_eval_many, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr int most = (2 * EVAL_ROWS * 15 + 8 * EVAL_ROWS) * 32 * (int)sizeof(double);
+  cudaError_t e = smem_limit<most>(k_eval_many);
   if (e != cudaSuccess) return e;
   k_eval_many<<<groups, 32 * slices, smem, st>>>(ea, q, P.alpha, P.pairs, P.nnz, t, S, price, delta);
   return cudaGetLastError();

@@ -1656,7 +1656,7 @@ inline size_t smem_bytes(int d, int p, int eta, int N, int tpb, size_t rsize, bo
 template <typename R, int D>
 cudaError_t launch_kernel(void (*kern)(Args<R, D>), const Args<R, D>& a, unsigned grid, int tpb,
                           size_t smem, cudaStream_t st) {
-  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t err = smem_limit<PATHS_SMEM>(kern);
   if (err != cudaSuccess) return err;
   // not by launch_pdl: its instructions in every one of some 10^4 short CTAs cost 3 %
   kern<<<grid, tpb, smem, st>>>(a);

@@ -53,8 +53,7 @@ void launch_basis(const ModelHost& m, const GridHost& g, const ProblemDev& P, ui
   const int dp = m.d + 1, eta = P.eta < 1 ? 1 : P.eta;
   const int tpb = 128;
   const size_t smem = (size_t)dp * (eta + 1) * BASIS_PTS * sizeof(double);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_basis, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > 48 * 1024) smem_limit<(BSDE_DMAX + 1) * 16 * BASIS_PTS * (int)sizeof(double)>(k_basis);
   const int gx = (P.n + BASIS_PTS - 1) / BASIS_PTS;
   const int want = (2 * device_sm_count() + gx - 1) / gx;
   int gy = (P.p + 31) / 32;

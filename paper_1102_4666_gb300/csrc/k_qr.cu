@@ -338,7 +338,7 @@ void launch_qr_solve(const ProblemDev& P, cudaStream_t st) {
   const void* kern = keep    ? (const void*)k_qr_factor<true, true>
                      : stage ? (const void*)k_qr_factor<true, false>
                              : (const void*)k_qr_factor<false, false>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  smem_limit<SMEM_PER_CTA - 5 * 1024>(kern);  // less the static part
   void* args[] = {&n, &n_pad, &p, &steps, &W, &y, &nrm, &perm, &sync, &status};
   cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(QR_THREADS), args, smem, st);
   launch_pdl(k_qr_solve, 1, 256, 0, st, n, n_pad, p, W, y, perm, P.delta, P.res, P.qr_rank);

@@ -108,12 +108,12 @@ extern "C" BSDE_API int bsde_corrections_noalloc(
     // launch shape of the path kernel: about 512 paths per CTA, which bounds the
     // partial sums in the static array
     int tpb = mixed ? 128 : 64;
-    while (tpb > 32 && paths_smem_bytes(m.d, p, eta_t, N_steps, tpb, mixed, false) > 220 * 1024) tpb >>= 1;
+    while (tpb > 32 && paths_smem_bytes(m.d, p, eta_t, N_steps, tpb, mixed, false) > PATHS_SMEM) tpb >>= 1;
     int ppt = 4;
     while (ppt > 1 && (long long)tpb * ppt > 2LL * M) ppt >>= 1;
     const long long chunks = (M + tpb * ppt - 1) / (tpb * ppt);
     if (p > NOALLOC_MAX_P || (long long)n * chunks > (long long)PARTIAL_MAX ||
-        paths_smem_bytes(m.d, p, eta_t, N_steps, tpb, mixed, false) > 220 * 1024) {
+        paths_smem_bytes(m.d, p, eta_t, N_steps, tpb, mixed, false) > PATHS_SMEM) {
       char msg[256];
       snprintf(msg, sizeof(msg),
                "corrections_noalloc: problem exceeds the static scratch (p = %d, limit %d; "

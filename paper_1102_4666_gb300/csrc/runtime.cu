@@ -236,8 +236,8 @@ void Problem::ensure_events(int count) {
 int Problem::choose_launch(int d, int n, int p, int eta, int N, int M, bool mx, bool dense, int tree,
                            int& tpb, int& ppt) {
   tpb = mx ? 128 : 64;
-  while (tpb > 32 && paths_smem_bytes(d, p, eta, N, tpb, mx, dense) > 220 * 1024) tpb >>= 1;
-  if (paths_smem_bytes(d, p, eta, N, tpb, mx, dense) > 220 * 1024) return BSDE_ERR_INVALID_ARG;
+  while (tpb > 32 && paths_smem_bytes(d, p, eta, N, tpb, mx, dense) > PATHS_SMEM) tpb >>= 1;
+  if (paths_smem_bytes(d, p, eta, N, tpb, mx, dense) > PATHS_SMEM) return BSDE_ERR_INVALID_ARG;
   while (tpb > 32 && tpb / 2 >= M) tpb >>= 1;
   if (!dense) {
     // FP32: about 512 paths per CTA, fewer for small M; FP64: one round (d = 3
@@ -248,12 +248,12 @@ int Problem::choose_launch(int d, int n, int p, int eta, int N, int M, bool mx, 
   }
   if (!mx) {
     ppt = 1;
-    if (M > 64 && paths_smem_bytes(d, p, eta, N, 128, mx, dense) <= 220 * 1024) tpb = 128;
+    if (M > 64 && paths_smem_bytes(d, p, eta, N, 128, mx, dense) <= PATHS_SMEM) tpb = 128;
     return BSDE_OK;
   }
   const bool big = tree && d <= 5 && p > 600;
   if (big && 4LL * ((M + 255) / 256 * 256) <= 5LL * M &&
-      paths_smem_bytes(d, p, eta, N, 256, mx, dense) <= 220 * 1024)
+      paths_smem_bytes(d, p, eta, N, 256, mx, dense) <= PATHS_SMEM)
     tpb = 256;
   const long long rounds = (M + tpb - 1) / tpb;
   const long long wave = (long long)device_sm_count() * (768 / tpb);
@@ -425,7 +425,7 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
   }
   if (prm.paths_tpb) {
     if (prm.paths_tpb < 32 || prm.paths_tpb > 256 || prm.paths_tpb % 32 ||
-        paths_smem_bytes(d, s.dense ? pm : p, s.eta, s.N, prm.paths_tpb, mixed, s.dense) > 220 * 1024) {
+        paths_smem_bytes(d, s.dense ? pm : p, s.eta, s.N, prm.paths_tpb, mixed, s.dense) > PATHS_SMEM) {
       err = "solve: paths_tpb must be a multiple of 32 in 32..256 within the shared memory";
       return BSDE_ERR_INVALID_ARG;
     }
