@@ -338,11 +338,18 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
     err = "solve: the path kernel is compiled for d = 1..10";
     return BSDE_ERR_INVALID_ARG;
   }
-  // basis, built anew only for another (d, eta, q)
-  if (nus.empty() || d != basis_d || prm.eta != basis_eta || prm.q != basis_q) {
+  // basis, built anew only for another (d, eta, q); two values of q may have the
+  // same functions, and the coefficients stay then
+  std::vector<std::vector<int>> nu_new;
+  bool same = !nus.empty() && d == basis_d && prm.eta == basis_eta && prm.q == basis_q;
+  if (!same) {
+    nu_new = build_multi_indices(d + 1, prm.eta, prm.q);
+    same = !nus.empty() && nu_new == nus;
+  }
+  if (!same) {
     basis_d = 0;
     tables_dirty = true;
-    nus = build_multi_indices(d + 1, prm.eta, prm.q);
+    nus.swap(nu_new);
     int mdeg = 0;
     if (!pack_multi_indices(nus, pairs, nnz, mdeg)) {
       err = "solve: basis needs more than 8 active variates or a degree above 15";
@@ -372,10 +379,10 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
       pm = -1;
     }
     if (pm < 0) pm = 0;
-    basis_d = d;
-    basis_eta = prm.eta;
-    basis_q = prm.q;
   }
+  basis_d = d;
+  basis_eta = prm.eta;
+  basis_q = prm.q;
   const int p = (int)nus.size();
   const int n = grid.n;
   if (!prm.allow_underdetermined && 2 * p > n) {
