@@ -1806,6 +1806,7 @@ cudaError_t launch(const ModelHost& m, const GridHost& g, const ProblemDev& P, i
   // the points of this launch: all n, or the block [shard_i0, shard_i0 + shard_n)
   const int npts = P.shard_n > 0 ? P.shard_n : P.n;
   if (npts <= 0) return cudaSuccess;
+  if ((long long)npts * P.chunks > 2147483647ll) return cudaErrorInvalidValue;
   const unsigned grid = (unsigned)npts * (unsigned)P.chunks;
   if (dense) {
     // the host selects: degree <= 3 loops (any d), degree-4 loops (d <= 5),

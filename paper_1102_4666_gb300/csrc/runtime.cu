@@ -214,6 +214,10 @@ void Problem::ensure_events(int count) {
   }
 }
 
+// CTAs of a path kernel launch
+static constexpr long long MAX_CTAS = 2147483647;
+static constexpr size_t PARTIAL_MOST = (size_t)64 << 20;
+
 // launch shape of the path kernel: threads per CTA, limited by the shared memory
 // of the per-thread Chebyshev tables, and paths per thread.  The dense
 // evaluations (tree: degree of the prefix tree, else 0):
@@ -284,7 +288,7 @@ size_t Problem::estimate_bytes(int d, int n, int p, int M, int N, bool mx, int t
   (void)N;
   const int n_pad = (n + 31) / 32 * 32;
   const int p_pad = (p + 127) / 128 * 128;
-  const int chunks = (M + tpb * ppt - 1) / (tpb * ppt);
+  const long long chunks = ((long long)M + tpb * ppt - 1) / (tpb * ppt);
   size_t b = 0;
   auto add = [&](size_t x) { b += (x + 255) / 256 * 256; };
   add((size_t)n * 8);
@@ -416,14 +420,41 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
     err = "solve: eval_mode 2 (dense) needs a constant correlation";
     return BSDE_ERR_INVALID_ARG;
   }
-  s.dense = pm > 0 && (const_corr || tree_deg == 0) && prm.eval_mode != 1;
-  s.dense4 = s.dense && tree_deg == 0 && mono_deg == 4;
-  s.tree = s.dense ? tree_deg : 0;
   if (prm.ls_mode != 0 && prm.ls_mode != 1) {
     err = "solve: ls_mode must be 0 (normal equations) or 1 (pivoted QR)";
     return BSDE_ERR_INVALID_ARG;
   }
   s.qr = prm.ls_mode == 1;
+  if (prm.gram_splits < 0 || prm.gram_splits > 4096) {
+    err = "solve: gram_splits must be in 0..4096";
+    return BSDE_ERR_INVALID_ARG;
+  }
+  s.splits = mixed ? gram_tc_splits(s.p_pad, s.n_pad, prm.gram_splits) : 0;
+  const int nf = fact_group(p, prm.K_it, grid.resample != 0, s.qr);
+  const long long points = (n + sh_n - 1) / sh_n;  // of this rank
+  long long chunks = 0;
+  auto bytes = [&](int nfact_in) {
+    return estimate_bytes(d, n, p, s.M, s.N, mixed, s.tpb, s.ppt, s.pm, s.dense ? (int)conv_l.size() : 0, s.qr,
+                          nfact_in, s.splits);
+  };
+  // More rounds of paths per CTA, and so fewer partial sums, up to the four rounds or
+  // 512 paths (FP64: 256) that the memory a solve needs is reckoned with: shapes with
+  // fewer rounds are faster, and taken while the budget has room for their partial sums
+  // and these take PARTIAL_MOST bytes at most (10^9 paths an iteration with 128 a CTA).
+  auto widen = [&]() {
+    if (prm.paths_ppt || (s.ppt >= 4 && s.tpb * s.ppt >= (mixed ? 512 : 256))) return false;
+    s.ppt *= 2;
+    return true;
+  };
+  auto fits = [&]() {
+    chunks = ((long long)s.M + s.tpb * s.ppt - 1) / (s.tpb * s.ppt);
+    return !(budget && bytes(nf) > budget) && chunks * points <= MAX_CTAS;
+  };
+  bool dense = pm > 0 && (const_corr || tree_deg == 0) && prm.eval_mode != 1;
+again:
+  s.dense = dense;
+  s.dense4 = s.dense && tree_deg == 0 && mono_deg == 4;
+  s.tree = s.dense ? tree_deg : 0;
   s.pm = s.dense ? pm : 0;
   if (choose_launch(d, n, s.dense ? pm : p, s.eta, s.N, s.M, mixed, s.dense, s.tree, s.tpb, s.ppt) !=
       BSDE_OK) {
@@ -445,30 +476,29 @@ int Problem::prepare(const bsde_solve_params& prm, Allocator& al, size_t budget,
     }
     s.ppt = prm.paths_ppt;
   }
-  s.chunks = (s.M + s.tpb * s.ppt - 1) / (s.tpb * s.ppt);
-  if (prm.gram_splits < 0 || prm.gram_splits > 4096) {
-    err = "solve: gram_splits must be in 0..4096";
-    return BSDE_ERR_INVALID_ARG;
-  }
-  s.splits = mixed ? gram_tc_splits(s.p_pad, s.n_pad, prm.gram_splits) : 0;
-  const int nf = fact_group(p, prm.K_it, grid.resample != 0, s.qr);
-  {
-    const size_t total = estimate_bytes(d, n, p, s.M, s.N, mixed, s.tpb, s.ppt, s.pm,
-                                        s.dense ? (int)conv_l.size() : 0, s.qr, nf, s.splits);
-    if (budget && total > budget) {
-      std::ostringstream os;
-      os << "solve: needs " << total << " bytes of device memory, budget " << budget;
-      err = os.str();
-      return BSDE_ERR_NOMEM;
+  while (!fits() || few_partials || (size_t)(chunks * n) * 8 > PARTIAL_MOST)
+    if (!widen()) break;
+  if (!fits()) {
+    if (chunks * points > MAX_CTAS) {
+      err = "solve: n * ceil(M / paths per CTA) exceeds 2^31 - 1";
+      return BSDE_ERR_INVALID_ARG;
     }
+    if (dense && !const_corr) {  // the tables of this form do not fit, the per-thread ones may
+      dense = false;
+      goto again;
+    }
+    std::ostringstream os;
+    os << "solve: needs " << bytes(nf) << " bytes of device memory, budget " << budget;
+    err = os.str();
+    return BSDE_ERR_NOMEM;
   }
+  s.chunks = (int)chunks;
   if (!block || !(s == alloc_shape)) {
-    const size_t need = estimate_bytes(d, n, p, s.M, s.N, mixed, s.tpb, s.ppt, s.pm,
-                                       s.dense ? (int)conv_l.size() : 0, s.qr, 0, s.splits);
     destroy_graph();
     if (block) al.put(block, st);
     block = nullptr;
     block_bytes = 0;
+    const size_t need = bytes(0);
     void* b = al.get(need, st);
     if (!b) {
       release(al, st);  // a failed call leaves the context holding no device memory

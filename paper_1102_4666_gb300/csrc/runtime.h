@@ -37,6 +37,7 @@ class Problem {
   bool has_model = false, has_grid = false, coeffs_valid = false;
   bool mixed = true;
   Shape shape;
+  bool few_partials = false;  // always as few partial sums as estimate_bytes at four rounds reckons with
   ProblemDev dev;
   std::vector<uint32_t> pairs;
   std::vector<uint32_t> prog;  // the basis as a tree (build_eval_program)

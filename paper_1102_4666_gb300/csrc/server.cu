@@ -39,6 +39,7 @@ struct Req {
   double t_submit = 0.0, t_done = 0.0;
   size_t bytes = 0;
   double work = 0.0;  // K_it n M N, the shortest-first key
+  bool few_partials = false;  // the budget has no room for one round of paths per CTA
   int prio = 0;       // 1: admitted on a high-priority stream
   std::unique_ptr<Problem> prob;
   cudaStream_t stream = nullptr;
@@ -147,6 +148,7 @@ bool bsde_server::admit_one(std::unique_lock<std::mutex>& lk) {
   P.model = req->model;
   P.grid = req->grid;
   P.has_model = P.has_grid = true;
+  P.few_partials = req->few_partials;
   cudaEventCreate(&req->e0);
   cudaEventCreate(&req->e1);
   req->rc = P.start(req->prm, al, 0, st, req->e0, req->e1);
@@ -260,11 +262,17 @@ int bsde_server_submit(bsde_server* s, const bsde_request* rq, uint64_t* id) {
     int p = 0;
     rc = bsde_basis_size(r->model.d, r->prm.eta, r->prm.q, &p);
     if (rc != BSDE_OK) return rc;
-    const int tpb = s->opts.precision == BSDE_PREC_MIXED ? 128 : 64;
-    const bool qr = r->prm.ls_mode == 1;
-    r->bytes = Problem::estimate_bytes(r->model.d, rq->n, p, r->prm.M, r->prm.N_steps,
-                                       s->opts.precision == BSDE_PREC_MIXED, tpb, 4, 0, 0, qr,
-                                       Problem::fact_group(p, r->prm.K_it, true, qr));
+    const bool mx = s->opts.precision == BSDE_PREC_MIXED, qr = r->prm.ls_mode == 1;
+    auto bytes = [&](int ppt) {
+      return Problem::estimate_bytes(r->model.d, rq->n, p, r->prm.M, r->prm.N_steps, mx, mx ? 128 : 64, ppt, 0, 0,
+                                     qr, Problem::fact_group(p, r->prm.K_it, true, qr));
+    };
+    // FP64 paths take one round per CTA, unless the partial sums of that exceed the budget
+    r->bytes = bytes(mx ? 4 : 1);
+    if (s->opts.mem_budget && r->bytes > s->opts.mem_budget && !mx) {
+      r->bytes = bytes(4);
+      r->few_partials = true;
+    }
     r->work = (double)r->prm.K_it * rq->n * (double)r->prm.M * r->prm.N_steps;
     r->t_submit = now_s();
     std::lock_guard<std::mutex> g(s->mu);
