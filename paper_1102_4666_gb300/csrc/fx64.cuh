@@ -322,10 +322,11 @@ FX_FN double exp(double x) {
   return pack(E, -63 - (int)(nt >> 54), 0);
 }
 
-// ln x with an absolute error below 2^-52 (the rounding of the result beyond
-// |ln x| = 2): x = y 2^e, y c = 1 - rho as in neg_log, rho exact from the low 64
-// bits of the product; the library's function for x <= 0, subnormal numbers,
-// NaN and infinities.  Not for relative accuracy next to x = 1.
+// ln x within 0.63 ulp for 1/4 <= |ln x|: x = y 2^e, y c = 1 - rho as in neg_log, rho
+// exact from the low 64 bits of the product.  The sum e ln 2 + ln y is kept at 2^59, its
+// error a few 2^-59, or where it does not fit (x beyond e^+-14.5) at 2^53; next to
+// x = 1 it cancels, and the library's function takes over, as it does for x <= 0,
+// subnormal numbers, NaN and infinities.
 FX_FN double log_abs(double x) {
   const uint64_t b = bits(x);
   const int ex = (int)(b >> 52);
@@ -345,10 +346,16 @@ FX_FN double log_abs(double x) {
   const uint64_t ny = lnc + (rho >> 9) + (mulhi(s2, P) >> 17);  // -ln y at 2^59, below 2^59
   const int e = ex - 1022;
   const uint32_t ae = (uint32_t)(e < 0 ? -e : e);
-  const uint64_t l2 = (wide(ae, hi32(FX_LN2_64)) << 21) + (wide(ae, lo32(FX_LN2_64)) >> 11);  // |e| ln 2 at 2^53
-  const int64_t r = (e < 0 ? -(int64_t)l2 : (int64_t)l2) - (int64_t)((ny + 32) >> 6);
-  if (r == 0) return 0.0;
-  return pack((uint64_t)(r < 0 ? -r : r), -53, r < 0 ? 1u : 0u);
+  if (ae > 21) {
+    const uint64_t l2 = (wide(ae, hi32(FX_LN2_64)) << 21) + (wide(ae, lo32(FX_LN2_64)) >> 11);  // |e| ln 2 at 2^53
+    const int64_t r = (e < 0 ? -(int64_t)l2 : (int64_t)l2) - (int64_t)((ny + 32) >> 6);
+    return pack((uint64_t)(r < 0 ? -r : r), -53, r < 0 ? 1u : 0u);
+  }
+  const uint64_t l2 = (wide(ae, hi32(FX_LN2_64)) << 27) + (wide(ae, lo32(FX_LN2_64)) >> 5);  // |e| ln 2 at 2^59
+  const int64_t r = (e < 0 ? -(int64_t)l2 : (int64_t)l2) - (int64_t)ny;
+  const uint64_t a = (uint64_t)(r < 0 ? -r : r);
+  if (a < (1ull << 57)) return log_lib(x);
+  return pack(a, -59, r < 0 ? 1u : 0u);
 }
 
 }  // namespace fx64

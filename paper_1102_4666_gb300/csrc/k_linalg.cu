@@ -756,6 +756,9 @@ __global__ void __launch_bounds__(256) k_eval_few(const __grid_constant__ EvalAr
 // functions that differ in their last variate only, neighbours in the basis
 // order, share the product P of the others and one sum S of the last factors:
 // three FP64 instructions per function and a few per group instead of twelve.
+// The functions are taken from the last, of the highest degree, to the first: the
+// constant and the linear terms, mostly the largest, come last, so that few
+// additions round at their size.
 // 20000 points, d = 10, p = 364: one CTA per point 840 us, function by function
 // 352 us, this 112 us.
 __global__ void __launch_bounds__(256) k_eval_many(const __grid_constant__ EvalArgs ea, int nq,
@@ -800,7 +803,7 @@ __global__ void __launch_bounds__(256) k_eval_many(const __grid_constant__ EvalA
       acc[va * 32] += gd;
     }
   };
-  for (int l = slice * per; l < l1; ++l) {
+  for (int l = l1 - 1; l >= slice * per; --l) {
     const double al = alpha[l];
     const int nz = nnz[l];
     if (nz == 0) {
@@ -829,11 +832,13 @@ __global__ void __launch_bounds__(256) k_eval_many(const __grid_constant__ EvalA
   close();
   acc[0] = u;
   __syncthreads();
-  // sums over the slices in order, row j = 0: u, else the derivative in x_j
+  // sums over the slices, in pairs, the last first; row j = 0: u, else the derivative in x_j
   const double* a0 = ev + (size_t)2 * rows * 32 + lane;
   for (int j = slice; j <= d; j += slices) {
     double s = 0.0;
-    for (int w = 0; w < slices; ++w) s += a0[((size_t)w * (d + 1) + j) * 32];
+    for (int w = slices - 2; w >= 0; w -= 2)
+      s += a0[((size_t)(w + 1) * (d + 1) + j) * 32] + a0[((size_t)w * (d + 1) + j) * 32];
+    if (slices == 1) s = a0[j * 32];
     if (q >= nq) continue;
     if (j == 0)
       price[q] = s;

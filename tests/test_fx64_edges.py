@@ -8,6 +8,7 @@ import ctypes
 import math
 import os
 import subprocess
+from decimal import Decimal, getcontext
 
 import numpy as np
 import pytest
@@ -43,6 +44,9 @@ extern "C" int roots(long n, const uint64_t* a, uint8_t* ok) {
 extern "C" void radicands(long n, const uint32_t* w, uint64_t* a) {
   int sc;
   for (long i = 0; i < n; i++) a[i] = neg_log(w[i], sc);
+}
+extern "C" void logs(long n, const double* x, double* o) {
+  for (long i = 0; i < n; i++) o[i] = log_abs(x[i]);
 }
 extern "C" void normals(long n, const uint32_t* w0, const uint32_t* w1, double* z0, double* z1) {
   Scale s;
@@ -120,6 +124,29 @@ def _check_pairs(w0, w1, z0, z1):
     th = np.pi * ((w1 + 0.5) * 2.0 ** -31)
     assert np.max(np.abs(z0 - rad * np.cos(th))) < 1e-14
     assert np.max(np.abs(z1 - rad * np.sin(th))) < 1e-14
+
+
+def test_logarithm_of_prices(tmp_path):
+    """Within 0.63 ulp (an eighth from the fixed point, half from the rounding) of the true value,
+    next to 1, where the sum cancels, next to the changes of form, and far out."""
+    (tmp_path / "t.cpp").write_text(HOST)
+    subprocess.check_call(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-I" + CSRC, "-o", str(tmp_path / "t.so"),
+                           str(tmp_path / "t.cpp")])
+    lib = ctypes.CDLL(str(tmp_path / "t.so"))
+    rng = np.random.default_rng(9)
+    near = [1.0 + s * 2.0 ** -k for k in range(1, 53) for s in (-1.0, 1.0)]
+    forms = [f * b for b in (math.exp(0.25), math.exp(-0.25), 2.0 ** 21, 2.0 ** 22, 2.0 ** -21, 2.0 ** -22, 2.0 ** -23)
+             for f in (1.0, 1.0 - 1e-15, 1.0 + 1e-15, 0.999, 1.001)]
+    x = np.concatenate([near, forms, np.exp(rng.uniform(-1, 1, 1500)), 100.0 * np.exp(rng.uniform(-1.5, 1.5, 1500)),
+                        np.exp(rng.uniform(-700, 700, 1500))])
+    x = x[x != 1.0]
+    o = np.zeros(len(x))
+    lib.logs(ctypes.c_long(len(x)), _p(x), _p(o))
+    getcontext().prec = 50
+    for v, got in zip(x, o):
+        want = Decimal(float(v)).ln()
+        ulp = Decimal(float(np.spacing(abs(float(want)))))
+        assert abs(Decimal(float(got)) - want) <= ulp * Decimal("0.63"), v
 
 
 @pytest.mark.gpu
