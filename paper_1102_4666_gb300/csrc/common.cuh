@@ -58,7 +58,8 @@ struct Philox {
 // ---------------------------------------------------------------------------
 // Precision traits (Box-Muller returns scale * (z0, z1)): the FP32 path uses the fast hardware approximations
 // (MUFU) where their error is far below the Monte Carlo noise; the FP64 path
-// uses CUDA's double-precision math library.
+// forms normals, exponentials and the logistic function in 64-bit fixed point
+// (fx64.cuh) and takes the rest from CUDA's double-precision library.
 // ---------------------------------------------------------------------------
 template <typename R>
 struct Math;

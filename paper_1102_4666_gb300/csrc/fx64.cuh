@@ -180,7 +180,8 @@ FX_FN uint64_t sqrt58(uint64_t A, int& e) {
 
 // |sin| and |cos| (at 2^63) of the phase (2 w + 1) 2^-33 revolutions within
 // its quadrant: the cell point's from the table, the rest delta = f pi/128,
-// |f| <= 1/2, by Taylor polynomials; absolute error below 2^-60
+// |f| <= 1/2, by Taylor polynomials; absolute error below 1.3 2^-60 (1.25 2^-60 at w = 855513624, the
+// largest of all words)
 FX_FN void trig_quadrant(uint32_t w, uint64_t& sn, uint64_t& cs) {
   const uint32_t r = (w << 2) | 2u;  // fraction of the quadrant at 2^32, exact
   uint64_t Sj, Cj;
@@ -278,7 +279,8 @@ FX_FN uint64_t pow2_neg(uint64_t f57) {
 }
 
 // 1 + r in [1, 2] with r = 1 / (1 + E) (inverse false: 1 - that), E = 2^-t,
-// t at 2^57, t < 128: absolute error below 2^-52.9 (the result's rounding)
+// t at 2^57, t < 128: absolute error below 2^-52.8, the result's rounding and the
+// truncation of t (largest of 10^9 arguments: 2^-52.95 from a double, 2^-52.85 in fixed point)
 FX_FN double logistic_of(uint64_t t, bool complement) {
   const uint64_t E = shr(pow2_neg(t & ((1ull << 57) - 1)), (int)(t >> 57));
   // q = 1 / (1 + E) in [1/2, 1]: R (1 + e + e^2), e = 1 - (1 + E) R exact to 2^-61
@@ -309,8 +311,8 @@ FX_FN double logistic_p1_fixed(int64_t y, bool absolute) {
   return logistic_of(t < (1ull << 62) ? t << 2 : ~0ull, y >= 0 || absolute);
 }
 
-// e^x: relative error below 2^-52.5; the library's function for |x| >= 256,
-// NaN and infinities
+// e^x: relative error below 2^-52.3 (largest of 5 10^8 arguments 2^-52.39, for |x| < 8
+// 2^-52.57); the library's function for |x| >= 256, NaN and infinities
 FX_FN double exp(double x) {
   const uint64_t b = bits(x);
   const int ex = (int)(b >> 52) & 0x7ff;

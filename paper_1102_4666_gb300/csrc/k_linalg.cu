@@ -151,8 +151,8 @@ __global__ void k_save_diag(const double* A, int p, double* diag0) {
 // (rows unscaled), E_r -= l_rc / l_cc E_c: eight columns per warp either way.
 // Every warp computes the pivot's reciprocal root for itself, so that a column
 // costs one barrier.  Bound by the chain pivot - root - column - next pivot and
-// the eight FMAs between (64 cycles of the pipe each): about 1500 cycles a
-// column.  Per block: one warp on shared memory 65 us, this 26 us.
+// the eight FMAs between (64 cycles of the pipe each): about 1800 cycles a
+// column.  Per block: one warp on shared memory 65 us, this 28 us.
 // A pivot below 1e-13 of its original diagonal entry (or not finite) marks the
 // matrix as numerically singular: ST_NOT_PD, and the pivot becomes NaN.
 __global__ void __launch_bounds__(128) k_chol_diag(double* A, int p, int j0,
@@ -1022,7 +1022,10 @@ void launch_update(const ModelHost& m, const GridHost& g, const ProblemDev& P, i
 // memory and is not more than its 16 SMs are worth.  An iteration with hardly any
 // paths as eleven launches and so: n = 200, p = 15 32.7 and 21.1 us, n = 2000, p = 35
 // 49.4 and 39.5, n = 2600, p = 56 (the line) 60.5 and 55.0, n = 20000, p = 6 92.7 and
-// 89.1, n = 37000, p = 3 141 and 145 (the means of that many points).
+// 89.1, n = 37000, p = 3 141 and 145 (the means of that many points).  Beside other
+// work the cluster waits a little for its SMs: small requests one at a time next to a
+// d = 10 solve in the server, median and 90th percentile: 7.4 and 10.4 ms so, 7.2 and
+// 9.5 as a chain, 6.9 and 11.5 with eight CTAs; alone on the device 1.7, 2.0 and 1.7 ms.
 constexpr long long REFIT_NP = 150000;
 constexpr int REFIT_SMEM = 203 * 1024;  // of p^2 + (p + 1) nl + ... at eight CTAs
 bool refit_small(int n, int p) { return p <= REFIT_P && n <= 16384 && (long long)n * (p + 1) <= REFIT_NP; }

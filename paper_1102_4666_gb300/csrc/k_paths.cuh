@@ -1038,8 +1038,8 @@ __device__ __forceinline__ void euler_step(const Args<R, D>& a, const R* tabs, c
 // d = 10 degree 4 4.84 -> 4.77 ms; against the vote and second pass d = 5
 // degree 4 3.42 -> 3.31 ms, degree 5 3.38 -> 3.26 ms, degree 6 4.63 -> 4.54
 // ms, but d = 4 degree 4 2.08 -> 2.14 ms (G = 1: the second pass is one
-// step) and d = 3 degree 3 0.104 -> 0.106 ms; FP64 paths keep the registers
-// (and the vote).
+// step) and d = 3 degree 3 0.104 -> 0.106 ms.  FP64 paths keep states and copies in
+// local memory (euler_path_f64), where an asset's copy is a store; none of the three.
 __host__ __device__ constexpr bool copy_vote(int ev, int d) {
   return d >= 3 && ev != EV_DENSE3 && !(ev >= EV_TREE4 && d >= 6);
 }
@@ -1316,12 +1316,12 @@ __device__ __forceinline__ void paths_cta(const Args<R, D>& a) {
     // the states before and after step s* (copy_vote, copy_smem); the vote
     // is over the lanes that reach a copy together, and a lane whose copy is
     // due always votes for itself, so it is never skipped
-    constexpr bool VOTE = copy_vote(EV, D) && !XCOPY;
+    constexpr bool VOTE = sizeof(R) == 4 && copy_vote(EV, D) && !XCOPY;
     // one predicated store a step into the slot that s asks for, instead of one
     // before and one after it, where a step is a whole group (d = 4 degree 4 2.27 ->
     // 2.21 ms a launch, d = 8 degree 3 4.34 -> 4.32; d = 6 loses 2 %)
     constexpr bool MERGED = G == 1;
-    constexpr bool REBUILD = sizeof(R) == 4 && VOTE;
+    constexpr bool REBUILD = VOTE;
     const int g_hit = sstar - sstar % G;  // first step of the group that contains s*
     constexpr bool ZSUM = sizeof(R) == 8 && VK == VK_CONST;  // states are sums of normals
     R X[D], Xg[D], Xs[D], Xn[D];

@@ -95,7 +95,7 @@ __device__ __forceinline__ long long qr_key(double a) {
 // lanes per SM and clock: 1 us per column of 2000 rows) and by the latencies of
 // a step (barrier, pivot column from L2, two block sums).  Measured at n = 2000,
 // p = 210 (two columns per CTA), the whole refit in a graph: 3.69 ms with two
-// launches per column, 2.11 ms now (n = 700: 2.39 -> 1.45 ms).
+// launches per column, 2.12 ms now.
 // sync[0]: arrivals (zero before the launch), sync[1]: set when a wait gave up.
 // STAGE: the pivot column is copied to shared memory (n doubles); KEEP: the
 // CTA's own columns are kept there too (and written through to W, where the
