@@ -152,8 +152,9 @@ def test_logarithm_of_prices(tmp_path):
 @pytest.mark.gpu
 def test_every_word_on_the_gpu(tmp_path):
     import torch
+    from paper_1102_4666_gb300 import _build
     (tmp_path / "t.cu").write_text(DEVICE)
-    subprocess.check_call(["nvcc", "-gencode", "arch=compute_103a,code=sm_103a", "-O2", "-std=c++17", "-shared",
+    subprocess.check_call([_build.nvcc(), "-gencode", "arch=compute_103a,code=sm_103a", "-O2", "-std=c++17", "-shared",
                            "-Xcompiler", "-fPIC", "-I" + CSRC, "-o", str(tmp_path / "t.so"), str(tmp_path / "t.cu")])
     lib = ctypes.CDLL(str(tmp_path / "t.so"))
     out = torch.zeros(2, dtype=torch.int64, device="cuda")
